@@ -3,6 +3,8 @@
 // fixed-point systematic resampling with a decoupled look-back scan, Halton
 // jitter and step counts with a counting sort by step count, and the
 // reweighting / evidence / ChEES-adaptation epilogue.
+#include <algorithm>
+#include <cmath>
 #include <math_constants.h>
 #include "smc_kernels.cuh"
 
@@ -186,74 +188,131 @@ __global__ void __launch_bounds__(SLICE) k_weights_steps(StepBufs b) {
 // do not resample write the identity source index.
 constexpr long long LOOKBACK_SPIN_LIMIT = 1ll << 22;
 
+// floor(X / T) with rT = 1 / (float)T: the FP32 quotient is off by at most
+// about 2^-22 of itself, so two of them (the second on the remainder) leave
+// the exact quotient within one unit, which the two loops settle.  About 25
+// instructions instead of the roughly 100 of the 64-bit division; T up to
+// 2^62 (every normalised weight vector) keeps the remainders in an int64,
+// larger totals divide.
+__host__ __device__ __forceinline__ unsigned long long quotient_u64(unsigned long long X, unsigned long long T, float rT) {
+    if (T >> 62) return X / T;
+    unsigned long long c = (unsigned long long)((float)X * rT);
+    long long rem = (long long)(X - c * T);
+    const long long d = (long long)((float)rem * rT);
+    c += (unsigned long long)d;
+    rem -= d * (long long)T;
+    while (rem < 0) {
+        --c;
+        rem += (long long)T;
+    }
+    while (rem >= (long long)T) {
+        ++c;
+        rem -= (long long)T;
+    }
+    return c;
+}
+
 __device__ __forceinline__ unsigned long long systematic_count(unsigned long long C, unsigned long long N,
-                                                               unsigned long long T, unsigned long long U) {
+                                                               unsigned long long T, unsigned long long U, float rT) {
     const unsigned long long NC = N * C;
     if (NC <= U) return 0ull;
-    const unsigned long long c = (NC - U + T - 1ull) / T;
+    const unsigned long long c = quotient_u64(NC - U + T - 1ull, T, rT);
     return c < N ? c : N;
 }
 
-// Decoupled look-back of tile g (thread 0 only): publishes the tile's
-// aggregate, walks back over the predecessors of its run (tiles first .. g-1)
-// summing aggregates until an inclusive prefix, and publishes its own
-// inclusive prefix.  Every wait on a predecessor is bounded: after `limit`
-// polls without progress it gives up, sets *failed (the caller has already
-// stored the run's error status, which is ordered before the publication) and
-// returns the partial sum; the tile still publishes, so no successor waits
-// forever.  Returns the exclusive prefix of the tile.
+// Decoupled look-back of tile g, by the 32 lanes of one warp: publishes the
+// tile's aggregate, walks back over the predecessors of its run (tiles first ..
+// g-1), 32 descriptors at a time, summing aggregates until an inclusive prefix,
+// and publishes its own inclusive prefix.  (One thread walking tile by tile
+// pays an L2 round trip per predecessor.)  Every wait on
+// a predecessor is bounded: after `limit` polls without progress it gives up,
+// sets *failed (*status is set to -5 before the publication) and returns the
+// partial sum; the tile still publishes, so no successor waits forever.
+// Returns the exclusive prefix of the tile to every lane.
 __device__ unsigned long long lookback_prefix(TileDesc* tiles, int64_t g, int64_t first, unsigned int epoch,
                                               unsigned long long tile_agg, long long limit, int* status,
                                               bool& failed) {
     TileDesc* me = tiles + g;
+    const int lane = threadIdx.x & 31;
     unsigned long long excl = 0ull;
     failed = false;
     if (g == first) {
-        me->incl = tile_agg;
-        __threadfence();
-        atomicExch(&me->flag, (epoch << 2) | 2u);
+        if (lane == 0) {
+            me->incl = tile_agg;
+            __threadfence();
+            atomicExch(&me->flag, (epoch << 2) | 2u);
+        }
         return 0ull;
     }
-    me->agg = tile_agg;
-    __threadfence();
-    atomicExch(&me->flag, (epoch << 2) | 1u);
+    if (lane == 0) {
+        me->agg = tile_agg;
+        __threadfence();
+        atomicExch(&me->flag, (epoch << 2) | 1u);
+    }
     int64_t pred = g - 1;
     long long spins = 0;
     while (true) {
-        const volatile TileDesc* pd = tiles + pred;
-        const unsigned int f = pd->flag;
-        if ((f >> 2) == epoch && (f & 3u) != 0u) {
+        // lane l reads predecessor pred - l; lanes before the run's first tile
+        // count as ready and empty (the first tile publishes its prefix, so
+        // the walk ends there)
+        const int64_t t = pred - lane;
+        const bool in = t >= first;
+        const volatile TileDesc* pd = tiles + (in ? t : first);
+        const unsigned int f = in ? pd->flag : 0u;
+        const bool ready = !in || ((f >> 2) == epoch && (f & 3u) != 0u);
+        const unsigned rmask = __ballot_sync(0xffffffffu, ready);
+        const unsigned imask = __ballot_sync(0xffffffffu, in && ready && (f & 3u) == 2u);
+        const int n_ready = rmask == 0xffffffffu ? 32 : __ffs(~rmask) - 1;   // ready lanes without a gap
+        const int n_incl = imask ? __ffs(imask) - 1 : 32;                     // nearest inclusive prefix
+        if (n_ready > 0) {
             __threadfence();
-            if ((f & 3u) == 2u) {
-                excl += pd->incl;
-                break;
-            }
-            excl += pd->agg;
-            --pred;
+            const bool done = n_incl < n_ready;
+            const int n = done ? n_incl + 1 : n_ready;
+            unsigned long long v = 0ull;
+            if (in && lane < n) v = lane == n_incl ? pd->incl : pd->agg;
+            excl += warp_sum(v);
+            if (done) break;
+            pred -= n;
             spins = 0;
             continue;
         }
         if (++spins > limit) {   // bounded wait: report, never hang
-            *(volatile int*)status = -5;
-            __threadfence();
+            if (lane == 0) {
+                *(volatile int*)status = -5;
+                __threadfence();
+            }
             failed = true;
             break;
         }
         __nanosleep(64);
     }
-    me->incl = excl + tile_agg;
-    __threadfence();
-    atomicExch(&me->flag, (epoch << 2) | 2u);
+    if (lane == 0) {
+        me->incl = excl + tile_agg;
+        __threadfence();
+        atomicExch(&me->flag, (epoch << 2) | 2u);
+    }
     return excl;
 }
+
+// Output ranges longer than EMIT_SHORT slots are written by a warp (by the
+// whole CTA from EMIT_BLOCK on) instead of their particle's thread: where a few
+// particles hold the mass (the first weighting of a run), one thread writing
+// its range slot by slot is the whole launch.
+constexpr unsigned int EMIT_SHORT = 8, EMIT_BLOCK = 2048;
 
 __global__ void __launch_bounds__(SCAN_THREADS) k_resample_scan(StepBufs b) {
     __shared__ unsigned int tile_s;
     __shared__ unsigned long long wsum[SCAN_THREADS / 32];
     __shared__ unsigned long long excl_s;
     __shared__ int failed_s;
+    __shared__ unsigned int long_lo[SCAN_TILE], long_hi[SCAN_TILE];   // the tile's long output ranges
+    __shared__ int long_i[SCAN_TILE];
+    __shared__ int n_long;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (tid == 0) tile_s = atomicAdd(b.counter, 1u);
+    if (tid == 0) {
+        tile_s = atomicAdd(b.counter, 1u);
+        n_long = 0;
+    }
     __syncthreads();
     const int64_t g = tile_s;
     if (g >= b.n_tiles) return;
@@ -311,13 +370,17 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_resample_scan(StepBufs b) {
     const unsigned long long tile_agg = wsum[SCAN_THREADS / 32 - 1];
 
     // look-back over predecessor tiles of the same run
-    if (tid == 0) {
+    if (wid == 0) {
         bool failed;
-        excl_s = lookback_prefix(b.tiles, g, rp.tile0, epoch, tile_agg, LOOKBACK_SPIN_LIMIT, &st.status, failed);
+        const unsigned long long excl =
+            lookback_prefix(b.tiles, g, rp.tile0, epoch, tile_agg, LOOKBACK_SPIN_LIMIT, &st.status, failed);
         // a run whose look-back gave up anywhere (here or in a predecessor,
         // whose status store precedes its publication) gets no resampling from
         // this tile on: identity source indices for the tile's own slots
-        failed_s = failed || *(volatile int*)&st.status != 0;
+        if (lane == 0) {
+            excl_s = excl;
+            failed_s = failed || *(volatile int*)&st.status != 0;
+        }
     }
     __syncthreads();
     if (failed_s) {
@@ -331,23 +394,50 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_resample_scan(StepBufs b) {
         return;
     }
     const unsigned long long off = excl_s + thread_excl;
-    // systematic: particle i of the run owns output slots [cnt(C_{i-1}),
-    // cnt(C_i)); multinomial: the prefix is kept for k_multinomial_search
-    const bool multi = rp.resample_scheme == 1;
+    // multinomial: the prefix is kept for k_multinomial_search; systematic:
+    // particle i of the run owns output slots [cnt(C_{i-1}), cnt(C_i))
+    if (rp.resample_scheme == 1) {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) {
+            const int64_t i = base + (int64_t)tid * SCAN_ITEMS + k;
+            if (i < rp.n) b.cprefix[rp.off + i] = off + v[k];
+        }
+        return;
+    }
+    const float rT = 1.0f / (float)T;
+    int32_t* const anc = b.anc + rp.off;
+    int32_t* const src = b.src ? b.src + rp.off : nullptr;
+    // a particle's range ends where the next one's begins: one count per particle
+    unsigned int lo = (unsigned int)systematic_count(off, N, T, U, rT);
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k) {
         const int64_t i = base + (int64_t)tid * SCAN_ITEMS + k;
         if (i >= rp.n) break;
-        const unsigned long long Ci = off + v[k];
-        if (multi) {
-            b.cprefix[rp.off + i] = Ci;
-            continue;
+        const unsigned int hi = (unsigned int)systematic_count(off + v[k], N, T, U, rT);
+        if (hi - lo > EMIT_SHORT && hi > lo) {
+            const int e = atomicAdd(&n_long, 1);   // the list's order does not matter: disjoint ranges
+            long_lo[e] = lo;
+            long_hi[e] = hi;
+            long_i[e] = (int)i;
+        } else {
+            for (unsigned int o = lo; o < hi; ++o) {
+                anc[o] = (int32_t)i;
+                if (src) src[o] = (int32_t)(rp.off + i);
+            }
         }
-        const unsigned long long Cp = Ci - b.q[rp.off + i];
-        const unsigned long long lo = systematic_count(Cp, N, T, U), hi = systematic_count(Ci, N, T, U);
-        for (unsigned long long o = lo; o < hi; ++o) {
-            b.anc[rp.off + (int64_t)o] = (int32_t)i;
-            if (b.src) b.src[rp.off + (int64_t)o] = (int32_t)(rp.off + i);
+        lo = hi;
+    }
+    __syncthreads();
+    const int nl = n_long;
+    for (int e = 0; e < nl; ++e) {
+        const unsigned int l = long_lo[e], h = long_hi[e];
+        const int32_t i = long_i[e];
+        const bool by_block = h - l >= EMIT_BLOCK;
+        if (!by_block && (e % (SCAN_THREADS / 32)) != wid) continue;
+        const unsigned int step = by_block ? SCAN_THREADS : 32u;
+        for (unsigned int o = l + (by_block ? (unsigned)tid : (unsigned)lane); o < h; o += step) {
+            anc[o] = i;
+            if (src) src[o] = (int32_t)rp.off + i;
         }
     }
 }
@@ -894,10 +984,82 @@ __global__ void __launch_bounds__(RUN_THREADS) k_normalise_flat(const double* lo
         *ess_out = 1.0 / s2;
     }
 }
+// The same over the whole GPU, for more than one CTA's worth of weights.  FP64
+// exponentials bound it (an SM retires about two FP64 operations per clock),
+// so they are spread over every SM: one CTA took 962 us at 100003 weights, the
+// three kernels take 32.  The partials (max, sum exp, sum exp^2 of each CTA's
+// contiguous share) wait in the first 3 gridDim.x entries of W, which the last
+// kernel overwrites, so nothing is allocated.
+constexpr int NORM_THREADS = 256, NORM_MAX_PARTS = 2 * 152;
+__global__ void __launch_bounds__(NORM_THREADS) k_norm_part(const double* logw, int64_t N, double* part) {
+    __shared__ double buf[2 * 32];
+    const int64_t lo = N * blockIdx.x / gridDim.x, hi = N * (blockIdx.x + 1) / gridDim.x;
+    double m = -CUDART_INF;
+    bool nan = false;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += NORM_THREADS) {
+        const double x = logw[i];
+        nan |= isnan(x);
+        m = fmax(m, x);
+    }
+    m = block_reduce(m, buf, OpMax());
+    double s[2] = {0.0, 0.0};
+    if (m > -CUDART_INF) {
+        for (int64_t i = lo + threadIdx.x; i < hi; i += NORM_THREADS) {
+            const double e = exp(logw[i] - m);
+            s[0] += e;
+            s[1] += e * e;
+        }
+    } else if (nan) {
+        s[0] = s[1] = CUDART_NAN;   // a share of NaN and -inf only still makes the sums NaN
+    }
+    block_reduce_n(s, buf, OpSum());
+    if (threadIdx.x == 0) {
+        part[3 * blockIdx.x] = m;
+        part[3 * blockIdx.x + 1] = s[0];
+        part[3 * blockIdx.x + 2] = s[1];
+    }
+}
+__global__ void __launch_bounds__(NORM_MAX_PARTS + 16) k_norm_combine(const double* part, int n_parts, double* lse_out,
+                                                                      double* ess_out) {
+    __shared__ double buf[2 * 32];
+    const int t = threadIdx.x;
+    const double mt = t < n_parts ? part[3 * t] : -CUDART_INF;
+    const double m = block_reduce(mt, buf, OpMax());
+    double s[2] = {0.0, 0.0};
+    if (t < n_parts) {
+        const double f = mt > -CUDART_INF ? exp(mt - m) : 1.0;   // without mass the sums are 0, or NaN
+        s[0] = part[3 * t + 1] * f;
+        s[1] = part[3 * t + 2] * f * f;
+    }
+    block_reduce_n(s, buf, OpSum());
+    if (t == 0) {
+        const bool any = m > -CUDART_INF;
+        *lse_out = any ? m + log(s[0]) : -CUDART_INF;
+        *ess_out = any ? s[0] * s[0] / s[1] : 0.0;
+    }
+}
+__global__ void __launch_bounds__(NORM_THREADS) k_norm_write(const double* logw, int64_t N, const double* lse,
+                                                             double* W) {
+    const int64_t i = (int64_t)blockIdx.x * NORM_THREADS + threadIdx.x;
+    if (i >= N) return;
+    const double l = *lse;
+    W[i] = l == -CUDART_INF ? 0.0 : exp(logw[i] - l);
+}
+
 cudaError_t launch_normalise_flat(const double* logw, int64_t N, double* W, double* lse, double* ess,
                                   cudaStream_t s) {
     if (N <= 0) return cudaErrorInvalidValue;
-    k_normalise_flat<<<1, RUN_THREADS, 0, s>>>(logw, N, W, lse, ess);
+    const int64_t nb = std::min<int64_t>((N + NORM_THREADS - 1) / NORM_THREADS, NORM_MAX_PARTS);
+    // one CTA: a single share, or weights written over the log-weights (W holds
+    // the partials while the log-weights are still read)
+    const bool overlap = W < logw + N && logw < W + N;
+    if (nb == 1 || overlap) {
+        k_normalise_flat<<<1, RUN_THREADS, 0, s>>>(logw, N, W, lse, ess);
+        return cudaGetLastError();
+    }
+    k_norm_part<<<(unsigned)nb, NORM_THREADS, 0, s>>>(logw, N, W);
+    k_norm_combine<<<1, NORM_MAX_PARTS + 16, 0, s>>>(W, (int)nb, lse, ess);
+    k_norm_write<<<(unsigned)((N + NORM_THREADS - 1) / NORM_THREADS), NORM_THREADS, 0, s>>>(logw, N, lse, W);
     return cudaGetLastError();
 }
 
@@ -912,15 +1074,19 @@ int64_t resample_scratch_bytes(int64_t N) {
     return (int64_t)(((sizeof(FlatScratch) + 255) / 256) * 256 + sizeof(TileDesc) * (size_t)flat_tiles(N));
 }
 
-__global__ void __launch_bounds__(RUN_THREADS) k_quantise_flat(const double* W, int64_t N, uint64_t r64,
-                                                               unsigned long long* q, FlatScratch* fs,
-                                                               int64_t n_tiles) {
+// q_j = floor(W_j 2^S) and T = sum q (an exact integer sum, so the atomics'
+// order does not matter) over the whole GPU; the header and the descriptors
+// were zeroed before.  Bound by memory: 16 bytes per weight (one CTA over all
+// of them took most of the 942 us of a 1M-particle resampling, now 46 in all).
+constexpr int QUANT_THREADS = 256;
+__global__ void __launch_bounds__(QUANT_THREADS) k_quantise_flat(const double* W, int64_t N, uint64_t r64,
+                                                                 unsigned long long* q, FlatScratch* fs,
+                                                                 int64_t n_tiles, double scale) {
     __shared__ unsigned long long ubuf[32];
-    int c = 0;
-    while (((int64_t)1 << c) < N) ++c;
-    const double scale = ldexp(1.0, 62 - c);
     unsigned long long T = 0ull;
-    for (int64_t i = threadIdx.x; i < N; i += blockDim.x) {
+    const int64_t stride = (int64_t)gridDim.x * QUANT_THREADS;
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * QUANT_THREADS + threadIdx.x; i < N; i += stride) {
         const double v = W[i] * scale;
         const unsigned long long qi = v > 0.0 ? __double2ull_rz(v) : 0ull;
         q[i] = qi;
@@ -928,21 +1094,15 @@ __global__ void __launch_bounds__(RUN_THREADS) k_quantise_flat(const double* W, 
     }
     T = block_reduce(T, ubuf, OpSum());
     if (threadIdx.x == 0) {
-        RunParams rp = {};
-        rp.off = 0;
-        rp.n = N;
-        rp.n_tiles = (int32_t)n_tiles;
-        rp.tile0 = 0;
-        fs->rp = rp;
-        RunState st = {};
-        st.k = 1;
-        st.T = T;
-        st.r64 = (unsigned long long)r64;
-        st.resample = T != 0ull;
-        st.status = T != 0ull ? 0 : -4;
-        fs->st = st;
-        fs->counter[0] = 0u;
-        fs->counter[1] = 1u;        // tiles are zeroed before every call
+        if (T) atomicAdd(&fs->st.T, T);
+        if (blockIdx.x == 0) {      // the other fields stay zero
+            fs->rp.n = N;
+            fs->rp.n_tiles = (int32_t)n_tiles;
+            fs->st.k = 1;
+            fs->st.r64 = (unsigned long long)r64;
+            fs->st.resample = 1;    // T == 0 is found (status -4) by the scan
+            fs->counter[1] = 1u;    // the descriptors' epoch: they were zeroed
+        }
     }
 }
 
@@ -953,14 +1113,16 @@ __global__ void k_copy_status(const FlatScratch* fs, int32_t* status) { *status 
 // of the current epoch, with the caller's poll limit; the wait must give up
 // and report -5 in *status (device), never hang.
 __global__ void k_lookback_wait_check(TileDesc* tiles, long long limit, int* status) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    tiles[0].flag = 0u;   // epoch 0, not ready: nothing will ever publish it
-    tiles[0].agg = tiles[0].incl = 0ull;
-    *status = 0;
-    __threadfence();
+    if (threadIdx.x == 0) {
+        tiles[0].flag = 0u;   // epoch 0, not ready: nothing will ever publish it
+        tiles[0].agg = tiles[0].incl = 0ull;
+        *status = 0;
+        __threadfence();
+    }
+    __syncwarp();
     bool failed;
     (void)lookback_prefix(tiles, 1, 0, 1u, 1ull, limit, status, failed);
-    if (!failed) *status = 1;   // cannot happen: the predecessor never publishes
+    if (!failed && threadIdx.x == 0) *status = 1;   // cannot happen: the predecessor never publishes
 }
 cudaError_t launch_lookback_wait_check(long long limit, TileDesc* tiles, int* status, cudaStream_t s) {
     k_lookback_wait_check<<<1, 32, 0, s>>>(tiles, limit, status);
@@ -974,9 +1136,13 @@ cudaError_t launch_resample_flat(const double* W, int64_t N, uint64_t r64, unsig
     FlatScratch* fs = reinterpret_cast<FlatScratch*>(scratch);
     TileDesc* tiles = reinterpret_cast<TileDesc*>(reinterpret_cast<char*>(scratch) +
                                                   ((sizeof(FlatScratch) + 255) / 256) * 256);
-    cudaError_t e = cudaMemsetAsync(tiles, 0, sizeof(TileDesc) * (size_t)nt, s);
+    cudaError_t e = cudaMemsetAsync(scratch, 0, (size_t)resample_scratch_bytes(N), s);   // header and descriptors
     if (e != cudaSuccess) return e;
-    k_quantise_flat<<<1, RUN_THREADS, 0, s>>>(W, N, r64, q, fs, nt);
+    int c = 0;
+    while (((int64_t)1 << c) < N) ++c;
+    // four weights per thread until the GPU is full (8 CTAs of 256 per SM)
+    const int64_t qb = std::min<int64_t>((N + 4 * QUANT_THREADS - 1) / (4 * QUANT_THREADS), 152 * 8);
+    k_quantise_flat<<<(unsigned)qb, QUANT_THREADS, 0, s>>>(W, N, r64, q, fs, nt, std::ldexp(1.0, 62 - c));
     StepBufs b = {};
     b.runs = &fs->rp;
     b.rstate = &fs->st;
