@@ -132,8 +132,13 @@ cudaError_t build_glm_mma_image(const uint16_t* xh, const uint16_t* xl, int64_t 
 // runs the same arithmetic in the same order, so the choice never changes a
 // result, only its speed.
 int32_t traj_tile_count(const DevModel& m, int32_t precision);
+// several threads per particle (traj_split.cu): the banana by pairs, the
+// dense Gaussian D <= 32 by rows where N particles alone do not fill the GPU
+cudaError_t launch_traj_banana(const DevModel& m, const TrajArgs& a, cudaStream_t s);
+bool gauss_rows_supported(const DevModel& m, int64_t N);
+cudaError_t launch_traj_gauss_rows(const DevModel& m, const TrajArgs& a, cudaStream_t s);
 // thread-per-particle kernels (traj_thread.cu): dense Gaussian D <= 32,
-// banana, hierarchical normal; FP32
+// hierarchical normal; FP32
 cudaError_t launch_traj_thread(const DevModel& m, const TrajArgs& a, cudaStream_t s);
 int32_t traj_thread_tiles(const DevModel& m);
 cudaError_t launch_traj(const DevModel& m, const TrajArgs& a, int32_t precision, cudaStream_t s);

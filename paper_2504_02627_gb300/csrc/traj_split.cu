@@ -1,0 +1,294 @@
+// traj_split.cu -- leapfrog trajectories (Algorithm 1) with one particle spread
+// over several threads, for the cheap targets whose gradient splits without
+// changing a single rounding:
+//  * the banana: its pairs (theta_2i, theta_2i+1) never meet, so each pair is
+//    a trajectory of its own, in one thread's registers;
+//  * the dense Gaussian with D <= 32: a lane per row of the precision, the
+//    deviations exchanged through shared memory each step.
+// A particle per thread (traj_thread.cu) leaves the GPU idle at the particle
+// counts of one run: a step is then one thread's chain over all dimensions,
+// with a warp or less per scheduler to hide it.
+#include <algorithm>
+#include <math_constants.h>
+#include "traj.cuh"
+
+namespace smc {
+namespace {
+
+// What a thread needs of its particle.
+struct Slot {
+    int64_t j, src;
+    int S;
+    double eps;
+    uint64_t seed;
+    uint32_t kk, jl;
+};
+__device__ __forceinline__ Slot slot_of(const TrajArgs& a, int64_t t) {
+    Slot x;
+    x.j = a.perm ? a.perm[t] : t;
+    x.src = a.src ? a.src[x.j] : x.j;
+    int r;
+    particle_run(a, x.j, r, x.eps, x.seed, x.kk, x.jl);
+    x.S = a.eval_only ? 0 : a.steps[x.j];
+    return x;
+}
+
+// Energies of the particle in slot order: H_0 from p_0, log pi at the end.
+__device__ __forceinline__ void finish(const TrajArgs& a, int64_t j, double lp1, double H0, double kin1) {
+    a.logpi_out[j] = lp1;
+    if (a.eval_only) return;
+    double dH = (0.5 * kin1 - lp1) - H0;
+    if (!isfinite(dH)) dH = CUDART_INF;
+    if (a.dH) a.dH[j] = dH;
+    if (a.alpha) a.alpha[j] = dH <= 0.0 ? 1.0 : exp(-dH);
+}
+
+// ============================================================ banana
+// Banana pairs (Sec. 4, Rosenbrock): x_o ~ N(0, a), x_e ~ N(b (x_o^2 - a), 1).
+__device__ __forceinline__ void banana_grad(float a, float b, float inva, float xo, float xe, float& g0, float& g1) {
+    float u = xe - b * (xo * xo - a);
+    g0 = -xo * inva + 2.0f * b * u * xo;
+    g1 = -u;
+}
+
+// A warp holds 32 consecutive slots; the PW warps of a slot group share the
+// particles' pairs, warp w taking pairs w, w + PW, ..., NPT of them side by
+// side (independent chains that fill each other's latency).  Loads and stores
+// are those of 32 consecutive particles of one dimension.  The FP64 sums (p'p
+// before and after, log pi) run in the order of the dimensions, by the group's
+// first warp from shared memory, so they have the bits of a thread that holds
+// the whole particle.  Bound by the FMA pipe (12 operations a pair and step)
+// and, in unsorted launches, by the longest of a warp's 32 trajectories: 50-d,
+// 8192 particles, up to 100 steps 59.6 -> 44.6 us with the caller's copies (29
+// of them this kernel; a thread per particle filled 64 CTAs).
+template <int NPT>
+__global__ void __launch_bounds__(256) traj_banana_kernel(DevModel m, TrajArgs a, int pw) {
+    extern __shared__ __align__(16) float sm[];
+    const int D = m.D, np = D / 2;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int w = wid % pw, grp = wid / pw, ngrp = (blockDim.x >> 5) / pw;
+    const int64_t t = ((int64_t)blockIdx.x * ngrp + grp) * 32 + lane;
+    const bool on = t < a.N;
+    float* sp0 = sm + (size_t)grp * 32 * (2 * D + np);     // [D][32] momenta before
+    float* sp1 = sp0 + 32 * D;                              // [D][32] momenta after
+    float* slp = sp1 + 32 * D;                              // [np][32] log pi terms
+    const float fa = (float)m.h0, fb = (float)m.h1, inva = (float)(1.0 / m.h0), half_inva = (float)(0.5 / m.h0);
+    Slot x{};
+    double lp0 = 0.0;
+    if (on) {
+        x = slot_of(a, t);
+        if (w == 0 && !a.eval_only) lp0 = a.logpi_in[x.src];
+        float xo[NPT], xe[NPT], po[NPT], pe[NPT], g0[NPT], g1[NPT];
+        const float ef = (float)x.eps, he = (float)(0.5 * x.eps);
+#pragma unroll
+        for (int k = 0; k < NPT; ++k) {
+            const int i = w + k * pw;
+            xo[k] = xe[k] = po[k] = pe[k] = g0[k] = g1[k] = 0.0f;
+            if (i >= np) continue;
+            const int64_t o = (int64_t)(2 * i) * a.ld;
+            xo[k] = a.theta_in[o + x.src];
+            xe[k] = a.theta_in[o + a.ld + x.src];
+            if (a.eval_only) {
+                banana_grad(fa, fb, inva, xo[k], xe[k], g0[k], g1[k]);
+                continue;
+            }
+            g0[k] = a.grad_in[o + x.src];
+            g1[k] = a.grad_in[o + a.ld + x.src];
+            if (a.p_in) {
+                po[k] = a.p_in[o + x.j];
+                pe[k] = a.p_in[o + a.ld + x.j];
+            } else {
+                normal_pair_f32(x.seed, (uint32_t)i, x.jl, x.kk, TAG_MOM, po[k], pe[k]);
+            }
+            sp0[2 * i * 32 + lane] = po[k];
+            sp0[(2 * i + 1) * 32 + lane] = pe[k];
+        }
+        for (int s = 0; s < x.S; ++s) {
+#pragma unroll
+            for (int k = 0; k < NPT; ++k) {
+                po[k] = fmaf(he, g0[k], po[k]);
+                pe[k] = fmaf(he, g1[k], pe[k]);
+                xo[k] = fmaf(ef, po[k], xo[k]);
+                xe[k] = fmaf(ef, pe[k], xe[k]);
+                banana_grad(fa, fb, inva, xo[k], xe[k], g0[k], g1[k]);
+                po[k] = fmaf(he, g0[k], po[k]);
+                pe[k] = fmaf(he, g1[k], pe[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < NPT; ++k) {
+            const int i = w + k * pw;
+            if (i >= np) continue;
+            const int64_t o = (int64_t)(2 * i) * a.ld + x.j;
+            const float u = xe[k] - fb * (xo[k] * xo[k] - fa);
+            slp[i * 32 + lane] = -half_inva * xo[k] * xo[k] - 0.5f * u * u;
+            a.grad_out[o] = g0[k];
+            a.grad_out[o + a.ld] = g1[k];
+            if (a.eval_only) continue;
+            sp1[2 * i * 32 + lane] = po[k];
+            sp1[(2 * i + 1) * 32 + lane] = pe[k];
+            a.theta_out[o] = xo[k];
+            a.theta_out[o + a.ld] = xe[k];
+            if (a.p_out) {
+                a.p_out[o] = po[k];
+                a.p_out[o + a.ld] = pe[k];
+            }
+        }
+    }
+    __syncthreads();
+    if (!on || w != 0) return;
+    double s = 0.0;
+    for (int i = 0; i < np; ++i) s += (double)slp[i * 32 + lane];
+    double kin0 = 0.0, kin1 = 0.0;
+    if (!a.eval_only)
+        for (int d = 0; d < D; ++d) {
+            const float v0 = sp0[d * 32 + lane], v1 = sp1[d * 32 + lane];
+            kin0 += (double)v0 * (double)v0;
+            kin1 += (double)v1 * (double)v1;
+        }
+    finish(a, x.j, s + m.lconst, 0.5 * kin0 - lp0, kin1);
+}
+
+template <int NPT>
+cudaError_t launch_banana_n(const DevModel& m, const TrajArgs& a, int pw, int ngrp, cudaStream_t s) {
+    const size_t sm = (size_t)ngrp * 32 * (2 * m.D + m.D / 2) * sizeof(float);
+    auto kern = traj_banana_kernel<NPT>;
+    if (sm > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+    }
+    const int64_t grid = (a.N + 32 * ngrp - 1) / (32 * ngrp);
+    kern<<<(unsigned)grid, 32 * pw * ngrp, sm, s>>>(m, a, pw);
+    return cudaGetLastError();
+}
+
+// ============================================================ dense Gaussian, row per lane
+// G lanes per particle (G the power of two from D on): lane r keeps row r of P
+// and dimension r of theta and p in registers.  A step: the deviations go to
+// shared memory, each lane reads them back as 16-byte broadcasts and runs its
+// row's sum in the order of the columns (the sum, and so every bit, of a
+// thread that holds the whole particle).  Bound by the step's chain (exchange
+// and one row's sum): the 10-d Gaussian's move of 256 particles, up to about 100
+// steps, takes 11.6 instead of 30.5 us, its 20-iteration run 1.51 -> 1.16 ms.
+template <int G>
+__global__ void __launch_bounds__(128) traj_gauss_rows_kernel(DevModel m, TrajArgs a) {
+    constexpr int PPC = 128 / G;                       // particles per CTA
+    __shared__ __align__(16) float dl_s[PPC][G];
+    __shared__ float p0_s[PPC][G], p1_s[PPC][G], q_s[PPC][G];
+    const int D = m.D, r = threadIdx.x % G, pi = threadIdx.x / G;
+    const int64_t t = (int64_t)blockIdx.x * PPC + pi;
+    // the lanes of one particle; all of them take every branch together
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << (G % 32)) - 1u) << ((threadIdx.x & 31) / G * G);
+    if (t >= a.N) return;
+    const bool in = r < D;
+    float P[G];
+#pragma unroll
+    for (int b = 0; b < G; ++b) P[b] = (in && b < D) ? m.P[r * D + b] : 0.0f;
+    const float mu = in ? m.mu[r] : 0.0f;
+    const Slot x = slot_of(a, t);
+    const int64_t o = (int64_t)r * a.ld;
+    float th = in ? a.theta_in[o + x.src] : 0.0f, p = 0.0f, g = 0.0f;
+    // grad log pi = -P (theta - mu), this lane's row
+    auto grad = [&]() {
+        dl_s[pi][r] = th - mu;
+        __syncwarp(gmask);
+        float acc = 0.0f;
+#pragma unroll
+        for (int b = 0; b < G; b += 4) {
+            if (b < D) {
+                const float4 v = *reinterpret_cast<const float4*>(&dl_s[pi][b]);
+                acc = fmaf(P[b], v.x, acc);
+                acc = fmaf(P[b + 1], v.y, acc);
+                acc = fmaf(P[b + 2], v.z, acc);
+                acc = fmaf(P[b + 3], v.w, acc);
+            }
+        }
+        __syncwarp(gmask);
+        return -acc;
+    };
+    if (a.eval_only) {
+        g = grad();
+    } else {
+        if (in) {
+            g = a.grad_in[o + x.src];
+            if (a.p_in) {
+                p = a.p_in[o + x.j];
+            } else {   // both lanes of a pair draw it
+                float z0, z1;
+                normal_pair_f32(x.seed, (uint32_t)(r >> 1), x.jl, x.kk, TAG_MOM, z0, z1);
+                p = (r & 1) ? z1 : z0;
+            }
+        }
+        p0_s[pi][r] = p;
+        const float ef = (float)x.eps, he = (float)(0.5 * x.eps);
+        for (int s = 0; s < x.S; ++s) {
+            p = fmaf(he, g, p);
+            th = fmaf(ef, p, th);
+            g = grad();
+            p = fmaf(he, g, p);
+        }
+        p1_s[pi][r] = p;
+    }
+    q_s[pi][r] = (th - mu) * g;
+    if (in) {
+        a.grad_out[o + x.j] = g;
+        if (!a.eval_only) {
+            a.theta_out[o + x.j] = th;
+            if (a.p_out) a.p_out[o + x.j] = p;
+        }
+    }
+    __syncwarp(gmask);
+    if (r != 0) return;
+    // log pi = c + 1/2 (theta - mu)' g: FP32 products, FP64 accumulation in
+    // the order of the dimensions, as are the kinetic energies
+    double q = 0.0, kin0 = 0.0, kin1 = 0.0;
+    for (int d = 0; d < D; ++d) {
+        q += (double)q_s[pi][d];
+        if (!a.eval_only) {
+            kin0 += (double)p0_s[pi][d] * (double)p0_s[pi][d];
+            kin1 += (double)p1_s[pi][d] * (double)p1_s[pi][d];
+        }
+    }
+    const double lp0 = a.eval_only ? 0.0 : a.logpi_in[x.src];
+    finish(a, x.j, m.lconst + 0.5 * q, 0.5 * kin0 - lp0, kin1);
+}
+
+template <int G>
+cudaError_t launch_rows(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
+    traj_gauss_rows_kernel<G><<<(unsigned)((a.N + 128 / G - 1) / (128 / G)), 128, 0, s>>>(m, a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// The launch variants of the banana (the autotuner's; 0 for the stage-level
+// calls) differ in the slot groups per CTA only.
+cudaError_t launch_traj_banana(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
+    if (m.D > 64) return cudaErrorInvalidValue;
+    const int np = m.D / 2;
+    int pw = 1;
+    while (pw < 8 && pw < np) pw <<= 1;
+    const int ngrp = std::max(1, std::min(8 / pw, a.tile % 4 == 1 ? 2 : a.tile % 4 == 2 ? 4 : 8 / pw));
+    switch ((np + pw - 1) / pw) {
+        case 1: return launch_banana_n<1>(m, a, pw, ngrp, s);
+        case 2: return launch_banana_n<2>(m, a, pw, ngrp, s);
+        case 3: return launch_banana_n<3>(m, a, pw, ngrp, s);
+        default: return launch_banana_n<4>(m, a, pw, ngrp, s);
+    }
+}
+
+bool gauss_rows_supported(const DevModel& m, int64_t N) {
+    // up to a few warps per scheduler in all (1245184 rows); beyond that the GPU
+    // is full with a particle per thread, which needs fewer instructions for
+    // each (no exchange, no idle lanes).  Below five dimensions there is
+    // nothing to split.
+    return m.kind == GAUSS_DENSE && m.D > 4 && m.D <= 32 && N * m.D <= (int64_t)152 * 2048 * 4;
+}
+
+cudaError_t launch_traj_gauss_rows(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
+    if (m.D <= 8) return launch_rows<8>(m, a, s);
+    if (m.D <= 16) return launch_rows<16>(m, a, s);
+    return launch_rows<32>(m, a, s);
+}
+
+}  // namespace smc

@@ -1,9 +1,16 @@
 // traj_thread.cu -- thread-per-particle leapfrog trajectories (Algorithm 1)
 // for targets whose gradient is cheap per particle: the dense Gaussian with
-// D <= 32, the banana and the non-centred hierarchical normal.  One thread
-// carries theta, p and grad of its particle in registers for the whole
-// trajectory, draws its momentum from the (seed, i, j, k, MOM) Philox stream
-// and returns the end-point energy error Delta H and min(1, exp(-Delta H)).
+// D <= 32 and the non-centred hierarchical normal.  One thread carries theta
+// and p of its particle in registers for the whole trajectory, draws its
+// momentum from the (seed, i, j, k, MOM) Philox stream and returns the
+// end-point energy error Delta H and min(1, exp(-Delta H)).
+//
+// What bounds them is the FMA pipe and, before that, the registers: a
+// gradient component is used up as it is formed (it closes its dimension's
+// kick, opens the next one and drifts the position at once), so no gradient
+// array lives next to theta and p.  The 52-d hierarchical normal then fits
+// 128 registers, four CTAs an SM (223, or 168 with 2 KB of spills, before):
+// 64 runs, 278k particles, three iterations 8.73 -> 6.53 ms.
 #include <algorithm>
 #include <cstdio>
 #include <math_constants.h>
@@ -12,81 +19,54 @@
 namespace smc {
 
 // ============================================================ thread models
+// A model's grad_each forms the gradient component by component and hands
+// each to f(d, g_d), which may already move theta_d and p_d: every value that
+// other components still need is read before the first call.
 template <int DM>
 struct GaussDenseM {
-    static size_t smem_bytes(const DevModel& m) { return (size_t)(m.D * m.D + m.D) * sizeof(float); }
+    static constexpr bool ENERGY_FROM_GRAD = true;
+    static constexpr int CTAS = DM > 16 ? 3 : 4;   // resident CTAs of 128 that the registers are capped for
+    static constexpr int LD = (DM + 3) / 4 * 4;    // row stride of P in shared memory
+    static size_t smem_bytes(const DevModel&) { return (size_t)(DM * LD + LD) * sizeof(float); }
     __device__ static void load(const DevModel& m, float* sm) {
-        for (int i = threadIdx.x; i < m.D * m.D; i += blockDim.x) sm[i] = m.P[i];
-        for (int i = threadIdx.x; i < m.D; i += blockDim.x) sm[m.D * m.D + i] = m.mu[i];
+        for (int i = threadIdx.x; i < DM * LD; i += blockDim.x) {
+            const int r = i / LD, c = i % LD;
+            sm[i] = (r < m.D && c < m.D) ? m.P[r * m.D + c] : 0.0f;
+        }
+        for (int i = threadIdx.x; i < LD; i += blockDim.x) sm[DM * LD + i] = i < m.D ? m.mu[i] : 0.0f;
     }
-    // grad log pi = -P (theta - mu)
-    __device__ static void grad(const DevModel& m, const float* sm, const float (&th)[DM], float (&g)[DM]) {
-        const int D = m.D;
-        const float* P = sm;
-        const float* mu = sm + D * D;
-        float dl[DM];
+    // grad log pi = -P (theta - mu); a row's sum runs over the padded width
+    // (zero times zero adds nothing), four elements of P per shared load
+    template <class F>
+    __device__ static void grad_each(const DevModel& m, const float* sm, const float (&th)[DM], F&& f) {
+        const float* mu = sm + DM * LD;
+        float dl[LD];
 #pragma unroll
-        for (int d = 0; d < DM; ++d) dl[d] = d < D ? th[d] - mu[d] : 0.0f;
+        for (int d = 0; d < LD; ++d) dl[d] = d < DM ? th[d < DM ? d : 0] - mu[d] : 0.0f;
 #pragma unroll
         for (int a = 0; a < DM; ++a) {
+            if (a >= m.D) break;
             float acc = 0.0f;
-            if (a < D) {
 #pragma unroll
-                for (int b = 0; b < DM; ++b)
-                    if (b < D) acc = fmaf(P[a * D + b], dl[b], acc);
+            for (int b = 0; b < LD; b += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(sm + a * LD + b);
+                acc = fmaf(v.x, dl[b], acc);
+                acc = fmaf(v.y, dl[b + 1], acc);
+                acc = fmaf(v.z, dl[b + 2], acc);
+                acc = fmaf(v.w, dl[b + 3], acc);
             }
-            g[a] = -acc;
+            f(a, -acc);
         }
     }
     // log pi = c - 1/2 (theta - mu)' P (theta - mu) = c + 1/2 (theta - mu)' g
     // with g = -P (theta - mu) the FP32 gradient at theta: FP32 products,
     // FP64 accumulation (the FP64 quadratic form costs D^2 operations at the
     // FP64 rate, a small fraction of the FP32 rate here)
-    __device__ static double logpi(const DevModel& m, const float* sm, const float (&th)[DM],
-                                   const float (&g)[DM]) {
-        const float* mu = sm + m.D * m.D;
-        double q = 0.0;
-#pragma unroll
-        for (int d = 0; d < DM; ++d)
-            if (d < m.D) q += (double)((th[d] - mu[d]) * g[d]);
+    __device__ static double energy_term(const float* sm, const float (&th)[DM], int d, float g) {
+        return (double)((th[d] - sm[DM * LD + d]) * g);
+    }
+    __device__ static double logpi(const DevModel& m, const float*, const float (&)[DM], double q) {
         return m.lconst + 0.5 * q;
-    }
-};
-
-// Banana pairs (Sec. 4, Rosenbrock): x_o ~ N(0, a), x_e ~ N(b (x_o^2 - a), 1).
-template <int DM>
-struct BananaM {
-    static size_t smem_bytes(const DevModel&) { return 0; }
-    __device__ static void load(const DevModel&, float*) {}
-    __device__ static void grad(const DevModel& m, const float*, const float (&th)[DM], float (&g)[DM]) {
-        const float a = (float)m.h0, b = (float)m.h1, inva = (float)(1.0 / m.h0);
-#pragma unroll
-        for (int i = 0; i + 1 < DM; i += 2) {
-            if (i + 1 < m.D) {
-                float xo = th[i], xe = th[i + 1];
-                float u = xe - b * (xo * xo - a);
-                g[i] = -xo * inva + 2.0f * b * u * xo;
-                g[i + 1] = -u;
-            } else {
-                g[i] = 0.0f;
-                g[i + 1] = 0.0f;
-            }
-        }
-        if (DM & 1) g[DM - 1] = 0.0f;
-    }
-    // FP32 terms per pair, FP64 accumulation
-    __device__ static double logpi(const DevModel& m, const float*, const float (&th)[DM], const float (&)[DM]) {
-        const float a = (float)m.h0, b = (float)m.h1, half_inva = (float)(0.5 / m.h0);
-        double s = 0.0;
-#pragma unroll
-        for (int i = 0; i + 1 < DM; i += 2) {
-            if (i + 1 < m.D) {
-                const float xo = th[i], xe = th[i + 1];
-                const float u = xe - b * (xo * xo - a);
-                s += (double)(-half_inva * xo * xo - 0.5f * u * u);
-            }
-        }
-        return s + m.lconst;
     }
 };
 
@@ -94,6 +74,8 @@ struct BananaM {
 // theta = (mu, log tau, eta_1..eta_G), b_g = mu + tau eta_g.
 template <int DM>
 struct HierM {
+    static constexpr bool ENERGY_FROM_GRAD = false;
+    static constexpr int CTAS = DM > 52 ? 3 : 4;   // resident CTAs of 128 that the registers are capped for
     // shared memory: (ybar_g, n_g / sigma^2) pairs for the gradient (one 8-byte
     // load per group), then n_g and the within-group sums of squares
     static size_t smem_bytes(const DevModel& m) { return (size_t)4 * m.n * sizeof(float); }
@@ -106,29 +88,40 @@ struct HierM {
             sm[3 * m.n + i] = m.gss[i];
         }
     }
-    __device__ static void grad(const DevModel& m, const float* sm, const float (&th)[DM], float (&g)[DM]) {
+    template <class F>
+    __device__ static void grad_each(const DevModel& m, const float* sm, const float (&th)[DM], F&& f) {
         const float2* st = reinterpret_cast<const float2*>(sm);
         const float mu = th[0], logtau = th[1], tau = expf(logtau);
         float dmu = 0.0f, dlt = 0.0f;
+        auto group = [&](int d) {
+            const float2 yn = st[d - 2];               // ybar_g, n_g / sigma^2
+            const float eta = th[d];
+            const float r = yn.y * (yn.x - fmaf(tau, eta, mu));
+            dmu += r;
+            dlt = fmaf(r * tau, eta, dlt);
+            f(d, fmaf(r, tau, -eta));
+        };
+        // groups in fours, one bounds check each, so that the scheduler has
+        // four independent groups between branches
 #pragma unroll
-        for (int d = 2; d < DM; ++d) {
-            float gd = 0.0f;
-            if (d < m.D) {
-                const float2 yn = st[d - 2];               // ybar_g, n_g / sigma^2
-                const float eta = th[d];
-                const float r = yn.y * (yn.x - fmaf(tau, eta, mu));
-                dmu += r;
-                dlt = fmaf(r * tau, eta, dlt);
-                gd = fmaf(r, tau, -eta);
+        for (int d0 = 2; d0 < DM; d0 += 4) {
+            if (d0 + 4 <= DM && d0 + 4 <= m.D) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (d0 + u < DM) group(d0 + u);
+            } else if (d0 < m.D) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (d0 + u < DM && d0 + u < m.D) group(d0 + u);
             }
-            g[d] = gd;
         }
-        g[0] = dmu - mu;
-        g[1] = dlt - logtau;
+        f(0, dmu - mu);
+        f(1, dlt - logtau);
     }
+    __device__ static double energy_term(const float*, const float (&)[DM], int, float) { return 0.0; }
     // FP32 terms per group, FP64 accumulation (as the GEMM-shaped models'
     // end points): FP64 runs at a small fraction of the FP32 rate here
-    __device__ static double logpi(const DevModel& m, const float* sm, const float (&th)[DM], const float (&)[DM]) {
+    __device__ static double logpi(const DevModel& m, const float* sm, const float (&th)[DM], double) {
         const float inv_2s2 = (float)(0.5 / (m.h0 * m.h0));
         const float mu = th[0], logtau = th[1], tau = expf(logtau);
         double s = -0.5 * (double)mu * (double)mu - 0.5 * (double)logtau * (double)logtau;
@@ -160,22 +153,20 @@ __device__ __forceinline__ void particle_move(const DevModel& m, const TrajArgs&
     uint32_t kk, jl;
     particle_run(a, j, r, eps, seed, kk, jl);
 
-    float th[DM], g[DM], p[DM];
+    float th[DM], p[DM];
 #pragma unroll
     for (int d = 0; d < DM; ++d) th[d] = d < D ? a.theta_in[(int64_t)d * a.ld + src] : 0.0f;
 
     if (a.eval_only) {
-        M::grad(m, sm, th, g);
-        double lp = M::logpi(m, sm, th, g);
-#pragma unroll
-        for (int d = 0; d < DM; ++d)
-            if (d < D) a.grad_out[(int64_t)d * a.ld + j] = g[d];
-        a.logpi_out[j] = lp;
+        double q = 0.0;
+        M::grad_each(m, sm, th, [&](int d, float g) {
+            if (M::ENERGY_FROM_GRAD) q += M::energy_term(sm, th, d, g);
+            a.grad_out[(int64_t)d * a.ld + j] = g;
+        });
+        a.logpi_out[j] = M::logpi(m, sm, th, q);
         return;   // from the particle's move
     }
 
-#pragma unroll
-    for (int d = 0; d < DM; ++d) g[d] = d < D ? a.grad_in[(int64_t)d * a.ld + src] : 0.0f;
     const double lp0 = a.logpi_in[src];
     if (a.p_in) {
 #pragma unroll
@@ -196,16 +187,37 @@ __device__ __forceinline__ void particle_move(const DevModel& m, const TrajArgs&
 
     const int S = a.steps[j];
     const float ef = (float)eps, he = (float)(0.5 * eps);
-    for (int s = 0; s < S; ++s) {
+    double q = 0.0;
+    if (S > 0) {
+        // the first half kick and drift from the cached gradient
 #pragma unroll
-        for (int d = 0; d < DM; ++d) p[d] = fmaf(he, g[d], p[d]);
+        for (int d = 0; d < DM; ++d)
+            if (d < D) {
+                p[d] = fmaf(he, a.grad_in[(int64_t)d * a.ld + src], p[d]);
+                th[d] = fmaf(ef, p[d], th[d]);
+            }
+        // a step's gradient closes its kick, opens the next and drifts
+        for (int s = 1; s < S; ++s)
+            M::grad_each(m, sm, th, [&](int d, float g) {
+                const float pv = fmaf(he, g, fmaf(he, g, p[d]));
+                p[d] = pv;
+                th[d] = fmaf(ef, pv, th[d]);
+            });
+        M::grad_each(m, sm, th, [&](int d, float g) {
+            if (M::ENERGY_FROM_GRAD) q += M::energy_term(sm, th, d, g);
+            p[d] = fmaf(he, g, p[d]);
+            a.grad_out[(int64_t)d * a.ld + j] = g;
+        });
+    } else {
 #pragma unroll
-        for (int d = 0; d < DM; ++d) th[d] = fmaf(ef, p[d], th[d]);
-        M::grad(m, sm, th, g);
-#pragma unroll
-        for (int d = 0; d < DM; ++d) p[d] = fmaf(he, g[d], p[d]);
+        for (int d = 0; d < DM; ++d)
+            if (d < D) {
+                const float g = a.grad_in[(int64_t)d * a.ld + src];
+                if (M::ENERGY_FROM_GRAD) q += M::energy_term(sm, th, d, g);
+                a.grad_out[(int64_t)d * a.ld + j] = g;
+            }
     }
-    const double lp1 = M::logpi(m, sm, th, g);
+    const double lp1 = M::logpi(m, sm, th, q);
     double kin1 = 0.0;
 #pragma unroll
     for (int d = 0; d < DM; ++d) kin1 += (double)p[d] * (double)p[d];
@@ -215,7 +227,6 @@ __device__ __forceinline__ void particle_move(const DevModel& m, const TrajArgs&
     for (int d = 0; d < DM; ++d) {
         if (d < D) {
             a.theta_out[(int64_t)d * a.ld + j] = th[d];
-            a.grad_out[(int64_t)d * a.ld + j] = g[d];
             if (a.p_out) a.p_out[(int64_t)d * a.ld + j] = p[d];
         }
     }
@@ -300,8 +311,8 @@ cudaError_t launch_thread_persist(const DevModel& m, const TrajArgs& a, cudaStre
 }
 
 // Variants of the thread-per-particle kernel for the autotuner: CTA size
-// (the granularity with which length-sorted slots are dealt to the SMs), a
-// register cap that trades spills for a third resident CTA, and for each of
+// (the granularity with which length-sorted slots are dealt to the SMs),
+// registers capped for three or four resident CTAs of 128, and for each of
 // these the persistent form (4-7: tiles from a device counter; they need
 // TrajArgs::work, else the launch falls back to the one-shot form).  Same
 // code, same arithmetic.  Small particles (DM < 16) have only the default.
@@ -309,19 +320,21 @@ constexpr int32_t THREAD_TILES = 8;
 template <template <int> class MT, int DM>
 cudaError_t launch_thread(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     if constexpr (DM >= 16) {
+        constexpr int C = MT<DM>::CTAS, O = 7 - C;   // the default cap, and the other one
         const int v = (a.tile >= 4 && !a.work) ? a.tile - 4 : a.tile;
         switch (v) {
-            case 1: return launch_thread_v<MT, DM, 64, 1>(m, a, s);
-            case 2: return launch_thread_v<MT, DM, 256, 1>(m, a, s);
-            case 3: return launch_thread_v<MT, DM, 128, 3>(m, a, s);
-            case 4: return launch_thread_persist<MT, DM, 128, 1>(m, a, s);
-            case 5: return launch_thread_persist<MT, DM, 64, 1>(m, a, s);
-            case 6: return launch_thread_persist<MT, DM, 256, 1>(m, a, s);
-            case 7: return launch_thread_persist<MT, DM, 128, 3>(m, a, s);
-            default: break;
+            case 1: return launch_thread_v<MT, DM, 64, 2 * C>(m, a, s);
+            case 2: return launch_thread_v<MT, DM, 256, 2>(m, a, s);
+            case 3: return launch_thread_v<MT, DM, 128, O>(m, a, s);
+            case 4: return launch_thread_persist<MT, DM, 128, C>(m, a, s);
+            case 5: return launch_thread_persist<MT, DM, 64, 2 * C>(m, a, s);
+            case 6: return launch_thread_persist<MT, DM, 256, 2>(m, a, s);
+            case 7: return launch_thread_persist<MT, DM, 128, O>(m, a, s);
+            default: return launch_thread_v<MT, DM, 128, C>(m, a, s);
         }
+    } else {
+        return launch_thread_v<MT, DM, 128, 1>(m, a, s);
     }
-    return launch_thread_v<MT, DM, 128, 1>(m, a, s);
 }
 
 template <template <int> class MT>
@@ -351,8 +364,11 @@ int32_t traj_thread_tiles(const DevModel& m) { return m.D > 12 ? THREAD_TILES : 
 
 cudaError_t launch_traj_thread(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     switch (m.kind) {
-        case GAUSS_DENSE: return m.D <= 32 ? dispatch_thread<GaussDenseM>(m, a, s) : cudaErrorInvalidValue;
-        case BANANA: return dispatch_thread_wide<BananaM>(m, a, s);
+        case GAUSS_DENSE:
+            if (m.D > 32) return cudaErrorInvalidValue;
+            return a.tile == 0 && gauss_rows_supported(m, a.N) ? launch_traj_gauss_rows(m, a, s)
+                                                               : dispatch_thread<GaussDenseM>(m, a, s);
+        case BANANA: return launch_traj_banana(m, a, s);
         case HIER_NORMAL: return dispatch_thread_wide<HierM>(m, a, s);
         default: return cudaErrorInvalidValue;
     }
