@@ -137,6 +137,8 @@ int32_t traj_tile_count(const DevModel& m, int32_t precision);
 cudaError_t launch_traj_banana(const DevModel& m, const TrajArgs& a, cudaStream_t s);
 bool gauss_rows_supported(const DevModel& m, int64_t N);
 cudaError_t launch_traj_gauss_rows(const DevModel& m, const TrajArgs& a, cudaStream_t s);
+// dense Gaussian 32 < D <= 128, FP32 (traj_dense.cu)
+cudaError_t launch_traj_dense(const DevModel& m, const TrajArgs& a, cudaStream_t s);
 // thread-per-particle kernels (traj_thread.cu): dense Gaussian D <= 32,
 // hierarchical normal; FP32
 cudaError_t launch_traj_thread(const DevModel& m, const TrajArgs& a, cudaStream_t s);
