@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 #include <cuda_runtime.h>
@@ -88,10 +89,24 @@ struct CentredScratch {
     std::vector<int32_t> h_padoff;
 };
 
+// Room for the launch order of the stage-level moves on a model (smc_model_create
+// only; 1 MB).  Calls may come from several threads and streams: a call takes
+// the room when the last one that used it ran on the same stream or has
+// finished, and otherwise goes without (the order changes speed only).
+struct OrderRoom {
+    static constexpr int64_t CAP = 262144;   // particles
+    int32_t* perm = nullptr;
+    cudaEvent_t used = nullptr;              // after the last launch that reads perm
+    unsigned long long stream_id = 0;
+    bool any = false;
+    std::mutex mu;
+};
+
 struct smc_dev_model {
     DevModel m{};
     DevAlloc mem;
     CentredScratch cs1;   // one run: the stage-level calls on caller buffers
+    OrderRoom order;
 };
 
 namespace {
@@ -1311,6 +1326,11 @@ smc_status smc_model_create(smc_dev_model** out, const smc_model* model, void* s
         delete m;
         return SMC_E_INVAL;
     }
+    if (cudaEventCreateWithFlags(&m->order.used, cudaEventDisableTiming) == cudaSuccess) {
+        m->order.perm = m->mem.get<int32_t>((size_t)OrderRoom::CAP);
+        cudaStreamSynchronize(m->mem.s);   // calls on other streams may use it from now on
+    }
+    if (!m->order.perm) (void)cudaGetLastError();   // moves then run in the particles' order
     *out = m;
     return SMC_OK;
 }
@@ -1320,6 +1340,7 @@ void smc_model_destroy(smc_dev_model* m) {
     cudaStream_t s = m->mem.s;
     m->mem.release();
     cudaStreamSynchronize(s);
+    if (m->order.used) cudaEventDestroy(m->order.used);
     delete m;
 }
 
@@ -1407,7 +1428,33 @@ smc_status smc_k_leapfrog(const smc_dev_model* m, float* theta, float* p, float*
     a.N = N;
     a.ld = ld;
     set_centred(a, m->cs1);
-    return kstatus(launch_traj(m->m, a, precision, static_cast<cudaStream_t>(stream)));
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // Ragged step counts: tiles of particles of similar length, in the room the
+    // model keeps for their order.  Not while a graph is captured (a replay
+    // could overlap later calls on the room).
+    OrderRoom& room = const_cast<smc_dev_model*>(m)->order;
+    if (!room.perm || N < 2 || N > OrderRoom::CAP || !order_pays(m->m, precision, N))
+        return kstatus(launch_traj(m->m, a, precision, s));
+    std::lock_guard<std::mutex> lock(room.mu);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    bool mine = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+                cudaStreamGetId(s, &id) == cudaSuccess;
+    if (mine && room.any && id != room.stream_id) mine = cudaEventQuery(room.used) == cudaSuccess;
+    if (!mine) {
+        (void)cudaGetLastError();   // cudaErrorNotReady is no error of this call
+        return kstatus(launch_traj(m->m, a, precision, s));
+    }
+    cudaError_t e = launch_order_steps(steps, N, room.perm, s);
+    if (e == cudaSuccess) {
+        a.perm = room.perm;
+        a.order_wait = 1;
+        e = launch_traj(m->m, a, precision, s);
+    }
+    room.any = true;
+    room.stream_id = id;
+    if (cudaEventRecord(room.used, s) != cudaSuccess && e == cudaSuccess) e = cudaGetLastError();
+    return kstatus(e);
 }
 
 smc_status smc_k_normalise(const double* logw, int64_t N, double* W, double* lse, double* ess, void* stream) {

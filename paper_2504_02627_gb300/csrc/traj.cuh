@@ -73,6 +73,7 @@ struct TrajArgs {
     int32_t eval_only;      // 1: compute log pi and grad at theta_in, no move
     int32_t tile;           // launch-configuration variant of the model's kernel (0: default)
     int* dev_err;           // set to 1 when a bounded device wait gives up (may be nullptr)
+    int32_t order_wait;     // 1: perm comes from a kernel that may still run (see wait_order)
     unsigned int* work;     // tile counter of the persistent launch variants (may be nullptr)
     // centred tensor-core path only: per-move reference quantities of each
     // run (written by the launcher before the trajectory kernel)
@@ -118,6 +119,36 @@ __device__ __forceinline__ void particle_run(const TrajArgs& a, int64_t j, int& 
     }
     kk = a.rstate ? (uint32_t)a.rstate[r].k : 0u;
 }
+
+// Before the first read of perm: with order_wait the launch overlaps the kernel
+// that writes perm (a programmatic dependent launch), which has to end first.
+// Everything older in the stream had ended before that kernel started.
+__device__ __forceinline__ void wait_order(const TrajArgs& a) {
+    if (a.order_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launches a trajectory kernel, overlapping the kernel that writes its order
+// when the arguments say so.
+template <typename K>
+cudaError_t launch_ordered(K kern, int64_t grid, int block, size_t smem, cudaStream_t s, const DevModel& m,
+                           const TrajArgs& a) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = a.order_wait ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kern, m, a);
+}
+
+// order.cu: perm = the particles by descending steps (any order within a
+// five-hundredth of the counts' range), and where that is worth a launch
+cudaError_t launch_order_steps(const int32_t* steps, int64_t N, int32_t* perm, cudaStream_t s);
+bool order_pays(const DevModel& m, int32_t precision, int64_t N);
 
 // Launchers (kernels in traj_simt.cu / traj_tc.cu).  Return cudaError_t of
 // the launch; `supported` reports whether the model/shape has a kernel.

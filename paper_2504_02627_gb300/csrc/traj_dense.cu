@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(DENSE_MAX_THREADS) traj_dense_kernel(DevModel 
         const int r = e / D, k = e - r * D;               // reads of a row of P
         Pt[k * RP + r] = r < D ? m.P[r * D + k] : 0.0f;
     }
+    wait_order(a);
     for (int q = tid; q < G; q += NT) {
         const int64_t t = (int64_t)blockIdx.x * G + q;
         int64_t j = -1, src = -1;
@@ -326,8 +327,7 @@ cudaError_t launch_dense(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const int64_t grid = (a.N + G - 1) / G;
     if (grid == 0) return cudaSuccess;
-    kern<<<(unsigned)grid, (L.nrg * (G / PT) + 31) / 32 * 32, sm, s>>>(m, a);
-    return cudaGetLastError();
+    return launch_ordered(kern, grid, (L.nrg * (G / PT) + 31) / 32 * 32, sm, s, m, a);
 }
 
 }  // namespace

@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(32 * KS, 2) traj_gauss_mma_kernel(DevModel m, 
             }
 
     // ---- particle scalars of this CTA
+    wait_order(a);
     const int64_t slot0 = (int64_t)blockIdx.x * GG_P;
     if (tid < GG_P) {
         const int64_t t = slot0 + tid;
@@ -274,7 +275,8 @@ __global__ void __launch_bounds__(32 * KS, 2) traj_gauss_mma_kernel(DevModel m, 
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) gr[u][e] = -(acc[u][e] + cor[u][e]);
+            for (int e = 0; e < 4; ++e)   // a trajectory without steps keeps its gradient
+                if (a.eval_only || s <= S[e >> 1]) gr[u][e] = -(acc[u][e] + cor[u][e]);
         // ---- closing half kick of step s; opening kick + drift of step s + 1
         //      and its A operand into the other buffer (its readers, step
         //      s - 1, finished at the previous barrier)
@@ -398,8 +400,7 @@ cudaError_t launch_gg(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const int64_t grid = (a.N + GG_P - 1) / GG_P;
     if (grid == 0) return cudaSuccess;
-    kern<<<(unsigned)grid, 32 * KS, L.bytes, s>>>(m, a);
-    return cudaGetLastError();
+    return launch_ordered(kern, grid, 32 * KS, L.bytes, s, m, a);
 }
 
 template <bool X3>

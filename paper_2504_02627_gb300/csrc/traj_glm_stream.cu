@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(GS_T, 2) traj_glm_stream_kernel(DevModel m, Tr
     int64_t j = -1, src = -1;
     int S = 0;
     float ef = 0.0f;
+    wait_order(a);
     const int64_t t = (int64_t)blockIdx.x * GS_P + pq;
     uint64_t seed = 0;
     uint32_t kk = 0, jl = 0;
@@ -281,8 +282,7 @@ cudaError_t launch_gs(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     auto kern = traj_glm_stream_kernel<LOGIT, HQ>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, GS_T, sm, s>>>(m, a);
-    return cudaGetLastError();
+    return launch_ordered(kern, grid, GS_T, sm, s, m, a);
 }
 
 template <bool LOGIT>

@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(NT, 1) traj_glm_kernel(DevModel m, TrajArgs a)
     const float inv_s = LOGIT ? 0.0f : (float)(1.0 / m.h0);
 
     // ---- particle state of this CTA
+    wait_order(a);
     const int64_t slot0 = (int64_t)blockIdx.x * G;
     __shared__ int64_t j_s[G], src_s[G];
     __shared__ float eps_s[G];
@@ -347,8 +348,7 @@ cudaError_t launch_glm(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const int64_t grid = (a.N + G - 1) / G;
     if (grid == 0) return cudaSuccess;
-    kern<<<(unsigned)grid, NT, sm, s>>>(m, a);
-    return cudaGetLastError();
+    return launch_ordered(kern, grid, NT, sm, s, m, a);
 }
 
 template <bool LOGIT>

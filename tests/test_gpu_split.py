@@ -64,3 +64,42 @@ def test_banana_pairs_are_independent_of_their_neighbours(D):
         for a, b in zip(one, whole):
             assert torch.equal(a[..., 0], b[..., i])
     dm.close()
+
+
+@pytest.mark.parametrize("kind,D,n,N", [("gauss", 100, 0, 3100), ("gauss", 40, 0, 20011), ("logistic", 25, 1000, 515),
+                                        ("logistic", 40, 3000, 130)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_ordered_moves_give_the_bits_of_unordered_ones(kind, D, n, N, precision):
+    """Launches above the ordering threshold against the same particles in
+    launches of 97 (below it): ragged, equal and zero step counts, on two
+    streams in turn."""
+    need_gpu()
+    if kind == "logistic" and precision:
+        pytest.skip("the regressions are ordered in FP32 only")
+    rng = np.random.default_rng(N)
+    if kind == "gauss":
+        A = rng.standard_normal((D, D))
+        md = B.ModelData(B.GAUSS_DENSE, D, mu=rng.standard_normal(D), prec=A @ A.T / D + np.eye(D))
+    else:
+        md = B.ModelData(B.LOGISTIC, D, n, X=rng.standard_normal((n, D)), y=(rng.uniform(size=n) < 0.5), hyper=(1.0,))
+    dm = B.DevModel(md, stream())
+    th, p, gr = (torch.randn(D, N, device="cuda") for _ in range(3))
+    lp = torch.randn(N, dtype=torch.float64, device="cuda")
+    other = torch.cuda.Stream()
+    for turn, S in enumerate((rng.integers(0, 9, size=N), np.full(N, 3), rng.integers(0, 2000, size=N) // 400)):
+        S_d = dev(S.astype(np.int32))
+        torch.cuda.synchronize()
+        whole = [x.clone() for x in (th, p, gr, lp)]
+        torch.cuda.synchronize()
+        s = other.cuda_stream if turn == 1 else stream()
+        B.check(B.lib().smc_k_leapfrog(dm.h, *map(ptr, whole), ptr(S_d), 0.01, N, N, precision, s), "leapfrog")
+        torch.cuda.synchronize()
+        for lo in range(0, N, 97):
+            hi = min(N, lo + 97)
+            part = [x[..., lo:hi].clone(memory_format=torch.contiguous_format) for x in (th, p, gr, lp)]
+            Sp = S_d[lo:hi].clone()
+            B.check(B.lib().smc_k_leapfrog(dm.h, *map(ptr, part), ptr(Sp), 0.01, hi - lo, hi - lo, precision, stream()),
+                    "leapfrog")
+            for a, b in zip(part, whole):
+                assert torch.equal(a, b[..., lo:hi])
+    dm.close()
