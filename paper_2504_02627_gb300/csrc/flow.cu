@@ -9,15 +9,12 @@
 // activations [rows x 32] stay in shared memory and the weights stream from
 // L2 as 16-byte rows of padded work copies (a transposed copy serves the
 // backward products), each thread accumulating a 4 x 4 tile.  FP32 with the
-// trajectory end-point energy accumulated in FP64.  The BF16 forms run the
-// same products on m16n8k16 warp MMAs (BF16 operands, FP32 accumulation):
-// the trajectories' conditioner and transposed products from pre-arranged
-// weight fragments, and in training also the weight gradients, which are
-// products over the CTA's 32 particles.
+// trajectory end-point energy accumulated in FP64.  The BF16 forms of both
+// (m16n8k16 warp MMAs) are in flow_mma.cu; their weight fragments are built
+// here.
 #include <cuda_bf16.h>
 #include <math_constants.h>
 #include "flow.cuh"
-#include "tc_ptx.cuh"
 
 namespace smc {
 namespace {
@@ -31,7 +28,8 @@ constexpr int FT = 256;          // threads per CTA
 size_t flow_smem_bytes(int D, int H, int L, int O4) {
     return sizeof(float) * (size_t)FG * (6 * D + L * D + 3 * H + O4) + sizeof(double) * 9 * FG;
 }
-// ... plus the BF16 operand buffer of the MMA form: [32][K + 8] for K <= 128
+// ... plus a BF16 operand buffer, [32][K + 8] for K <= 128: the BF16 forms serve
+// the shapes for which this fits (what they need themselves is less)
 static size_t flow_pm_bytes() { return sizeof(uint16_t) * (size_t)FG * (128 + 8); }
 
 namespace {
@@ -178,102 +176,9 @@ __device__ __forceinline__ void cta_mm(const float* __restrict__ At, int K, int 
     }
 }
 
-// FP32 rows X [R x 32] -> BF16 particle-major B [32][ldb] (k contiguous),
-// zero for R <= k < Kpad: the B operand of the next MMA.  A thread converts
-// eight consecutive k of one particle (lanes = particles: the row reads are
-// conflict-free, and the 16-byte stores at a row stride of ldb = K + 8 fall
-// in distinct bank groups).
-__device__ __noinline__ void to_pm(const float* X, int R, int Kpad, __nv_bfloat16* B, int ldb) {
-    for (int e = threadIdx.x; e < FG * (Kpad / 8); e += FT) {
-        const int q = e & (FG - 1), k0 = 8 * (e / FG);
-        uint32_t w[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int k = k0 + 2 * h;
-            const float v0 = k < R ? X[k * FG + q] : 0.0f, v1 = k + 1 < R ? X[(k + 1) * FG + q] : 0.0f;
-            const __nv_bfloat162 b2 = __floats2bfloat162_rn(v0, v1);
-            w[h] = *reinterpret_cast<const uint32_t*>(&b2);
-        }
-        *reinterpret_cast<uint4*>(B + q * ldb + k0) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-}
-
-// Y[r][p] = act(sum_k A[r][k] B[k][p] + bias[r]) for rows r < Mvalid and the
-// CTA's 32 particles, on m16n8k16 BF16 MMAs with FP32 accumulation.  A: MT x KS
-// tiles of fragments (L2), B: BF16 particle-major [32][ldb] in shared memory
-// (ldb = K + 8: the eight 16-byte rows of a matrix load fall in distinct bank
-// groups).  A warp takes one m-tile and all four n-tiles when there are eight
-// or more m-tiles, else one m-tile and two n-tiles.
-template <bool TANH, bool BIAS>
-__device__ __noinline__ void cta_mma(const uint4* __restrict__ Af, int MT, int KS, const __nv_bfloat16* B, int ldb,
-                                        float* Y, const float* __restrict__ bias, int Mvalid) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int mi = lane >> 3, mr = lane & 7;
-    const bool full = MT >= FT / 32;
-    const int items = full ? MT : 2 * MT;
-    const uint32_t bbase = tc::smem_u32(B);
-    for (int it = wid; it < items; it += FT / 32) {
-        const int mt = full ? it : it >> 1;
-        const int nt0 = full ? 0 : 2 * (it & 1);
-        const int nh = full ? 2 : 1;          // n-tile pairs of this item
-        float acc[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = 0.0f;
-        // every A fragment of this m-tile in flight at once (KS <= 8): the
-        // loads come from L2 and the products behind them are short
-        uint4 afr[8];
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks)
-            if (ks < KS) afr[ks] = __ldg(Af + ((int64_t)mt * KS + ks) * 32 + lane);
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            if (ks >= KS) break;
-            const uint32_t av[4] = {afr[ks].x, afr[ks].y, afr[ks].z, afr[ks].w};
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (h < nh) {
-                    // matrices (n-tile nt0 + 2h + (mi >> 1), k half mi & 1)
-                    const int prow = 8 * (nt0 + 2 * h + (mi >> 1)) + mr;
-                    const int kcol = 16 * ks + 8 * (mi & 1);
-                    uint32_t b[4];
-                    tc::ldsm4(b, bbase + (uint32_t)(prow * ldb + kcol) * 2u);
-                    tc::mma_bf16_16816(acc[2 * h], av, b[0], b[1]);
-                    tc::mma_bf16_16816(acc[2 * h + 1], av, b[2], b[3]);
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (u < 2 * nh) {
-                const int pc = 8 * (nt0 + u) + 2 * t;
-                const int r0 = 16 * mt + g, r1 = r0 + 8;
-                float v0 = acc[u][0], v1 = acc[u][1], v2 = acc[u][2], v3 = acc[u][3];
-                if (BIAS) {
-                    const float b0 = r0 < Mvalid ? __ldg(bias + r0) : 0.0f, b1 = r1 < Mvalid ? __ldg(bias + r1) : 0.0f;
-                    v0 += b0;
-                    v1 += b0;
-                    v2 += b1;
-                    v3 += b1;
-                }
-                if (TANH) {
-                    v0 = tanhf(v0);
-                    v1 = tanhf(v1);
-                    v2 = tanhf(v2);
-                    v3 = tanhf(v3);
-                }
-                if (r0 < Mvalid) *reinterpret_cast<float2*>(Y + r0 * FG + pc) = make_float2(v0, v1);
-                if (r1 < Mvalid) *reinterpret_cast<float2*>(Y + r1 * FG + pc) = make_float2(v2, v3);
-            }
-        }
-    }
-}
-
 struct FlowSmem {
     float *z, *p, *gz, *x, *c, *gx, *zl, *h1, *h2, *o, *ch;
     double *ldp, *ld;    // [8][32] partials, [32]
-    __nv_bfloat16* pm;   // BF16 form: the B operand of the next product, [32][<= 136]
 };
 
 __device__ __forceinline__ FlowSmem flow_smem(unsigned char* base, int D, int H, int L, int O4) {
@@ -296,31 +201,10 @@ __device__ __forceinline__ FlowSmem flow_smem(unsigned char* base, int D, int H,
 }
 
 // Conditioner of layer l at rows [aoff, aoff + Dh) of `in`: h1, h2, o.
-// MMA: the three products on BF16 warp MMAs (operands rounded to BF16, FP32
-// accumulation, bias and tanh in FP32).
-template <bool MMA = false>
 __device__ __forceinline__ void conditioner(const DevFlow& f, int l, const float* in, FlowSmem& s) {
     const FlowLayerOff o = flow_layer_off(f.H, f.Dh, f.Dh4, f.O4);
     const float* w = f.work + (int64_t)l * f.layer_work;
     const int aoff = (l & 1) ? f.Dh : 0;
-    if (MMA) {
-        const uint4* fr = f.frag + (int64_t)l * f.layer_frag;
-        const FlowFragOff fo = flow_frag_off(f.H, f.kp1, f.o4p);
-        const int H = f.H;
-        to_pm(in + aoff * FG, f.Dh, f.kp1, s.pm, f.kp1 + 8);
-        __syncthreads();
-        cta_mma<true, true>(fr + fo.W1, H / 16, f.kp1 / 16, s.pm, f.kp1 + 8, s.h1, w + o.b1, H);
-        __syncthreads();
-        to_pm(s.h1, H, H, s.pm, H + 8);
-        __syncthreads();
-        cta_mma<true, true>(fr + fo.W2, H / 16, H / 16, s.pm, H + 8, s.h2, w + o.b2, H);
-        __syncthreads();
-        to_pm(s.h2, H, H, s.pm, H + 8);
-        __syncthreads();
-        cta_mma<false, true>(fr + fo.W3, f.o4p / 16, H / 16, s.pm, H + 8, s.o, w + o.b3, f.O4);
-        __syncthreads();
-        return;
-    }
     cta_mm<true, true>(w + o.W1t, f.Dh, f.H, in + aoff * FG, s.h1, w + o.b1);
     __syncthreads();
     cta_mm<true, true>(w + o.W2t, f.H, f.H, s.h1, s.h2, w + o.b2);
@@ -344,14 +228,13 @@ __device__ __forceinline__ void ld_accumulate(FlowSmem& s, double v, bool add_to
 }
 
 // x <- T(x), recording the input of every layer in zl; s.ld = log|det dT/dz|.
-template <bool MMA = false>
 __device__ void flow_forward(const DevFlow& f, FlowSmem& s, float* x) {
     const int t = threadIdx.x, D = f.D;
     if (t < FG) s.ld[t] = 0.0;
     for (int l = 0; l < f.L; ++l) {
         for (int e = t; e < D * FG; e += FT) s.zl[l * D * FG + e] = x[e];
         __syncthreads();
-        conditioner<MMA>(f, l, x, s);
+        conditioner(f, l, x, s);
         const int boff = (l & 1) ? 0 : f.Dh;
         double part = 0.0;
         for (int k = t >> 5; k < f.Dh; k += 8) {
@@ -367,13 +250,12 @@ __device__ void flow_forward(const DevFlow& f, FlowSmem& s, float* x) {
 
 // x <- T^-1(x), recording the output of every inverse layer (= the input of
 // forward layer l) in zl; s.ld = log|det dT^-1/dx| = -sum s.
-template <bool MMA = false>
 __device__ void flow_inverse(const DevFlow& f, FlowSmem& s, float* x) {
     const int t = threadIdx.x, D = f.D;
     if (t < FG) s.ld[t] = 0.0;
     __syncthreads();
     for (int l = f.L - 1; l >= 0; --l) {
-        conditioner<MMA>(f, l, x, s);
+        conditioner(f, l, x, s);
         const int boff = (l & 1) ? 0 : f.Dh;
         double part = 0.0;
         for (int k = t >> 5; k < f.Dh; k += 8) {
@@ -390,14 +272,13 @@ __device__ void flow_inverse(const DevFlow& f, FlowSmem& s, float* x) {
 }
 
 // c <- J_T(z)^T c + grad_z log|det dT/dz| using the recorded layer inputs.
-template <bool MMA = false>
 __device__ void flow_backward(const DevFlow& f, FlowSmem& s, float* c) {
     const int t = threadIdx.x, D = f.D;
     const FlowLayerOff off = flow_layer_off(f.H, f.Dh, f.Dh4, f.O4);
     for (int l = f.L - 1; l >= 0; --l) {
         const float* in = s.zl + l * D * FG;
         const float* w = f.work + (int64_t)l * f.layer_work;
-        conditioner<MMA>(f, l, in, s);
+        conditioner(f, l, in, s);
         const int boff = (l & 1) ? 0 : f.Dh, aoff = (l & 1) ? f.Dh : 0;
         for (int e = t; e < f.Dh4 * FG; e += FT) {
             const int k = e / FG, q = e % FG;
@@ -415,39 +296,16 @@ __device__ void flow_backward(const DevFlow& f, FlowSmem& s, float* c) {
             s.o[(f.Dh4 + k) * FG + q] = ct;
         }
         __syncthreads();
-        if (MMA) {
-            // the transposed products: W3^T og, W2^T d2, W1^T d1 (BF16 operands)
-            const uint4* fr = f.frag + (int64_t)l * f.layer_frag;
-            const FlowFragOff fo = flow_frag_off(f.H, f.kp1, f.o4p);
-            const int H = f.H;
-            to_pm(s.o, f.O4, f.o4p, s.pm, f.o4p + 8);
-            __syncthreads();
-            cta_mma<false, false>(fr + fo.W3t, H / 16, f.o4p / 16, s.pm, f.o4p + 8, s.ch, nullptr, H);
-            __syncthreads();
-            for (int e = t; e < H * FG; e += FT) s.h2[e] = s.ch[e] * (1.0f - s.h2[e] * s.h2[e]);
-            __syncthreads();
-            to_pm(s.h2, H, H, s.pm, H + 8);
-            __syncthreads();
-            cta_mma<false, false>(fr + fo.W2t, H / 16, H / 16, s.pm, H + 8, s.ch, nullptr, H);
-            __syncthreads();
-            for (int e = t; e < H * FG; e += FT) s.h1[e] = s.ch[e] * (1.0f - s.h1[e] * s.h1[e]);
-            __syncthreads();
-            to_pm(s.h1, H, H, s.pm, H + 8);
-            __syncthreads();
-            cta_mma<false, false>(fr + fo.W1t, f.kp1 / 16, H / 16, s.pm, H + 8, s.ch, nullptr, f.Dh4);
-            __syncthreads();
-        } else {
-            cta_mm<false, false>(w + off.W3, f.O4, f.H, s.o, s.ch, nullptr);
-            __syncthreads();
-            for (int e = t; e < f.H * FG; e += FT) s.h2[e] = s.ch[e] * (1.0f - s.h2[e] * s.h2[e]);
-            __syncthreads();
-            cta_mm<false, false>(w + off.W2, f.H, f.H, s.h2, s.ch, nullptr);
-            __syncthreads();
-            for (int e = t; e < f.H * FG; e += FT) s.h1[e] = s.ch[e] * (1.0f - s.h1[e] * s.h1[e]);
-            __syncthreads();
-            cta_mm<false, false>(w + off.W1, f.H, f.Dh4, s.h1, s.ch, nullptr);
-            __syncthreads();
-        }
+        cta_mm<false, false>(w + off.W3, f.O4, f.H, s.o, s.ch, nullptr);
+        __syncthreads();
+        for (int e = t; e < f.H * FG; e += FT) s.h2[e] = s.ch[e] * (1.0f - s.h2[e] * s.h2[e]);
+        __syncthreads();
+        cta_mm<false, false>(w + off.W2, f.H, f.H, s.h2, s.ch, nullptr);
+        __syncthreads();
+        for (int e = t; e < f.H * FG; e += FT) s.h1[e] = s.ch[e] * (1.0f - s.h1[e] * s.h1[e]);
+        __syncthreads();
+        cta_mm<false, false>(w + off.W1, f.H, f.Dh4, s.h1, s.ch, nullptr);
+        __syncthreads();
         for (int e = t; e < f.Dh * FG; e += FT) c[aoff * FG + e] += s.ch[e];
         __syncthreads();
     }
@@ -530,12 +388,11 @@ __device__ double target_logpi(const DevModel& m, const float* x, const float* g
 }
 
 // -------------------------------------------------------------- trajectories
-template <int TARGET, bool MMA>
+template <int TARGET>
 __global__ void __launch_bounds__(FT, 1) traj_flow_kernel(DevModel m, DevFlow f, TrajArgs a, float* z0out,
                                                           float* z1out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FlowSmem s = flow_smem(smem_raw, f.D, f.H, f.L, f.O4);
-    s.pm = reinterpret_cast<__nv_bfloat16*>(s.ld + FG);   // past the FP64 block: flow_smem_bytes from the base
     // h1, h2, o and ch are contiguous: (3 H + O4) x 32 floats of scratch for P and mu
     const bool pfits = m.kind == GAUSS_DENSE && m.D * m.D + m.D <= (3 * f.H + f.O4) * FG;
     __shared__ int64_t j_s[FG], src_s[FG];
@@ -598,11 +455,11 @@ __global__ void __launch_bounds__(FT, 1) traj_flow_kernel(DevModel m, DevFlow f,
     }
     const int smax = smax_s;
     // latent start z0 = T^-1(theta), its log pi_z and gradient
-    flow_inverse<MMA>(f, s, s.x);                // s.x = z0, s.ld = log|det dT^-1|
+    flow_inverse(f, s, s.x);                // s.x = z0, s.ld = log|det dT^-1|
     for (int e = t; e < D * FG; e += FT) s.z[e] = s.x[e];
     if (t < FG) lp_s[t] = (src_s[t] >= 0 ? a.logpi_in[src_s[t]] : 0.0) - s.ld[t];   // log pi_z(z0)
     __syncthreads();
-    flow_backward<MMA>(f, s, s.c);               // s.c = grad_z log pi_z(z0)
+    flow_backward(f, s, s.c);               // s.c = grad_z log pi_z(z0)
     for (int e = t; e < D * FG; e += FT) s.gz[e] = s.c[e];
     if (!a.p_in) {
         const int npairs = (D + 1) / 2;
@@ -641,12 +498,12 @@ __global__ void __launch_bounds__(FT, 1) traj_flow_kernel(DevModel m, DevFlow f,
     for (int st = 1; st <= smax; ++st) {
         for (int e = t; e < D * FG; e += FT) s.x[e] = s.z[e];
         __syncthreads();
-        flow_forward<MMA>(f, s, s.x);            // s.x = T(z), s.ld = log|det dT/dz|
+        flow_forward(f, s, s.x);            // s.x = T(z), s.ld = log|det dT/dz|
         target_grad<TARGET>(m, s.x, s.gx, s.h1, pfits);       // grad_x log pi
         __syncthreads();
         for (int e = t; e < D * FG; e += FT) s.c[e] = s.gx[e];
         __syncthreads();
-        flow_backward<MMA>(f, s, s.c);           // grad_z log pi_z
+        flow_backward(f, s, s.c);           // grad_z log pi_z
         for (int e = t; e < D * FG; e += FT) {
             const int q = e % FG;
             if (st <= S_s[q]) {
@@ -833,222 +690,6 @@ __global__ void __launch_bounds__(FT, 1) k_flow_train(DevFlow f, const float* th
     }
 }
 
-// -------------------------------------------------------------- BF16 training
-// The training step with every conditioner product on BF16 warp MMAs (FP32
-// accumulation; master weights, bias sums, Adam and the coupling arithmetic
-// stay FP32): the conditioner of the inverse pass and of the backward pass
-// (as in the BF16 trajectories), the transposed products W3^T c_o, W2^T c_h2,
-// W1^T c_h1 from the transposed fragments, and the weight gradients, which
-// are products over the CTA's 32 particles, c [rows x 32] . act^T [32 x cols].
-constexpr int WLD = FG + 8;      // row stride (BF16) of the weight-gradient operands
-
-// FP32 rows X [R x 32] -> BF16 rows Y [Rpad][WLD] (particles contiguous),
-// zero for R <= r < Rpad.  A thread converts eight particles of one row.
-__device__ __noinline__ void to_rows(const float* X, int R, int Rpad, __nv_bfloat16* Y) {
-    for (int e = threadIdx.x; e < Rpad * 4; e += FT) {
-        const int r = e >> 2, p0 = 8 * (e & 3);
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
-        if (r < R) {
-            const float4 a = *reinterpret_cast<const float4*>(X + r * FG + p0);
-            const float4 b = *reinterpret_cast<const float4*>(X + r * FG + p0 + 4);
-            const __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y), h1 = __floats2bfloat162_rn(a.z, a.w);
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(b.x, b.y), h3 = __floats2bfloat162_rn(b.z, b.w);
-            w[0] = *reinterpret_cast<const uint32_t*>(&h0);
-            w[1] = *reinterpret_cast<const uint32_t*>(&h1);
-            w[2] = *reinterpret_cast<const uint32_t*>(&h2);
-            w[3] = *reinterpret_cast<const uint32_t*>(&h3);
-        }
-        *reinterpret_cast<uint4*>(Y + r * WLD + p0) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-}
-
-// out[row(m) * ldo + n] = sum over the CTA's 32 particles p of A[m][p] B[n][p]
-// for m < 16 MT, n < min(16 NP, Nvalid); A, B BF16 rows [.][WLD] in shared
-// memory (K = the particles: two k-steps of m16n8k16).  A warp takes one
-// m-tile and four n-tiles.  CMAP: A's rows are the conditioner's padded
-// output rows (s rows from 0, t rows from Dh4), stored at the canonical rows
-// of W3 (s then t, Dh each); otherwise rows m < Mvalid are stored as they are.
-template <bool CMAP>
-__device__ __noinline__ void cta_wgrad(const __nv_bfloat16* A, int MT, const __nv_bfloat16* B, int NP, float* out,
-                                       int ldo, int Mvalid, int Nvalid, int Dh, int Dh4) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int mi = lane >> 3, mr = lane & 7;
-    const int NQ = (NP + 1) >> 1;
-    const uint32_t abase = tc::smem_u32(A), bbase = tc::smem_u32(B);
-    auto row_of = [&](int m) -> int {
-        if (!CMAP) return m < Mvalid ? m : -1;
-        return m < Dh ? m : (m >= Dh4 && m < Dh4 + Dh ? Dh + (m - Dh4) : -1);
-    };
-    for (int it = wid; it < MT * NQ; it += FT / 32) {
-        const int mt = it / NQ, q = it % NQ;
-        float acc[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = 0.0f;
-#pragma unroll
-        for (int ks = 0; ks < 2; ++ks) {
-            // A fragment: lanes 0-15 address rows 0-15 at k 0-7, lanes 16-31 the same rows at k 8-15
-            uint32_t a[4];
-            tc::ldsm4(a, abase + (uint32_t)(((16 * mt + (lane & 15)) * WLD + 16 * ks + 8 * (lane >> 4)) * 2));
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int np = 2 * q + h;     // n-tiles 2 np and 2 np + 1
-                if (np < NP) {
-                    const int nrow = 16 * np + 8 * (mi >> 1) + mr;
-                    const int kcol = 16 * ks + 8 * (mi & 1);
-                    uint32_t b[4];
-                    tc::ldsm4(b, bbase + (uint32_t)((nrow * WLD + kcol) * 2));
-                    tc::mma_bf16_16816(acc[2 * h], a, b[0], b[1]);
-                    tc::mma_bf16_16816(acc[2 * h + 1], a, b[2], b[3]);
-                }
-            }
-        }
-        const int r0 = row_of(16 * mt + g), r1 = row_of(16 * mt + g + 8);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (2 * q + (u >> 1) < NP) {
-                const int c0 = 8 * (4 * q + u) + 2 * t;
-                if (r0 >= 0) {
-                    if (c0 < Nvalid) out[(int64_t)r0 * ldo + c0] = acc[u][0];
-                    if (c0 + 1 < Nvalid) out[(int64_t)r0 * ldo + c0 + 1] = acc[u][1];
-                }
-                if (r1 >= 0) {
-                    if (c0 < Nvalid) out[(int64_t)r1 * ldo + c0] = acc[u][2];
-                    if (c0 + 1 < Nvalid) out[(int64_t)r1 * ldo + c0 + 1] = acc[u][3];
-                }
-            }
-        }
-    }
-}
-
-// Shared memory of the BF16 training kernel: FP32 x, c [D x 32], the layer
-// inputs zl [L x D x 32], h1, h2 [H x 32], o [O4 x 32], ch [H x 32]; then the
-// particle-major BF16 operand [32][<= 136] and the two row-major BF16
-// operands of the weight-gradient products [128][WLD].
-__device__ __forceinline__ FlowSmem flow_train_smem(unsigned char* base, int D, int H, int L, int O4,
-                                                    __nv_bfloat16*& A16, __nv_bfloat16*& B16) {
-    FlowSmem s{};
-    float* f = reinterpret_cast<float*>(base);
-    s.x = f;
-    s.c = s.x + D * FG;
-    s.zl = s.c + D * FG;
-    s.h1 = s.zl + L * D * FG;
-    s.h2 = s.h1 + H * FG;
-    s.o = s.h2 + H * FG;
-    s.ch = s.o + O4 * FG;
-    s.pm = reinterpret_cast<__nv_bfloat16*>(s.ch + H * FG);
-    A16 = s.pm + FG * (128 + 8);
-    B16 = A16 + 128 * WLD;
-    return s;
-}
-
-// The weighted-NLL gradient of k_flow_train with BF16 products; the same
-// partials layout (canonical parameter order, one row per CTA).
-__global__ void __launch_bounds__(FT, 1) k_flow_train_mma(DevFlow f, const float* theta, int64_t ld,
-                                                          const int32_t* src, const double* W, FlowGate gate,
-                                                          int64_t N, float* partials) {
-    if (!gate.open()) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __nv_bfloat16 *A16, *B16;
-    FlowSmem s = flow_train_smem(smem_raw, f.D, f.H, f.L, f.O4, A16, B16);
-    __shared__ float w_s[FG];
-    const int t = threadIdx.x, D = f.D, H = f.H, Dh = f.Dh, Dh4 = f.Dh4;
-    const int64_t slot0 = (int64_t)blockIdx.x * FG;
-    if (t < FG) {
-        const int64_t j = slot0 + t;
-        float wv = 0.0f;
-        if (j < N) {
-            wv = (gate.rs && gate.rs->resample) ? (float)(1.0 / (double)gate.rp->n) : (float)W[j];
-        }
-        w_s[t] = wv;
-    }
-    __syncthreads();
-    for (int e = t; e < D * FG; e += FT) {
-        const int d = e / FG, q = e % FG;
-        const int64_t j = slot0 + q;
-        s.x[e] = (j < N && w_s[q] != 0.0f) ? theta[(int64_t)d * ld + (src ? src[j] : j)] : 0.0f;
-    }
-    __syncthreads();
-    for (int l = f.L - 1; l >= 0; --l) {
-        for (int e = t; e < D * FG; e += FT) s.zl[l * D * FG + e] = s.x[e];
-        __syncthreads();
-        conditioner<true>(f, l, s.x, s);
-        const int boff = (l & 1) ? 0 : Dh;
-        for (int e = t; e < Dh * FG; e += FT) {
-            const int k = e / FG, q = e % FG;
-            const float sv = 2.0f * tanhf(s.o[k * FG + q]);
-            const float tv = s.o[(Dh4 + k) * FG + q];
-            s.x[(boff + k) * FG + q] = (s.x[(boff + k) * FG + q] - tv) * expf(-sv);
-        }
-        __syncthreads();
-    }
-    for (int e = t; e < D * FG; e += FT) s.c[e] = w_s[e % FG] * s.x[e];
-    __syncthreads();
-    const int64_t lsz = (int64_t)H * Dh + H + (int64_t)H * H + H + (int64_t)D * H + D;
-    const FlowFragOff fo = flow_frag_off(H, f.kp1, f.o4p);
-    float* part = partials + (int64_t)blockIdx.x * f.n_params;
-    for (int l = 0; l < f.L; ++l) {
-        const float* in = s.zl + l * D * FG;
-        const uint4* fr = f.frag + (int64_t)l * f.layer_frag;
-        float* gl = part + l * lsz;
-        float *gW1 = gl, *gb1 = gW1 + (int64_t)H * Dh, *gW2 = gb1 + H, *gb2 = gW2 + (int64_t)H * H, *gW3 = gb2 + H,
-              *gb3 = gW3 + (int64_t)D * H;
-        conditioner<true>(f, l, in, s);
-        const int boff = (l & 1) ? 0 : Dh, aoff = (l & 1) ? Dh : 0;
-        for (int e = t; e < Dh4 * FG; e += FT) {
-            const int k = e / FG, q = e % FG;
-            float cs_raw = 0.0f, ct = 0.0f;
-            if (k < Dh) {
-                const float th = tanhf(s.o[k * FG + q]);
-                const float ems = expf(-2.0f * th);
-                const float b = (in[(boff + k) * FG + q] - s.o[(Dh4 + k) * FG + q]) * ems;
-                const float cb = s.c[(boff + k) * FG + q];
-                const float cs = fmaf(-cb, b, w_s[q]);
-                cs_raw = cs * 2.0f * (1.0f - th * th);
-                ct = -cb * ems;
-                s.c[(boff + k) * FG + q] = cb * ems;
-            }
-            s.o[k * FG + q] = cs_raw;
-            s.o[(Dh4 + k) * FG + q] = ct;
-        }
-        __syncthreads();
-        // c_o: dW3 = c_o h2^T, db3 = row sums, c_h2 = (W3^T c_o) (1 - h2^2)
-        to_rows(s.o, f.O4, f.o4p, A16);
-        to_rows(s.h2, H, H, B16);
-        to_pm(s.o, f.O4, f.o4p, s.pm, f.o4p + 8);
-        __syncthreads();
-        cta_wgrad<true>(A16, f.o4p / 16, B16, H / 16, gW3, H, 0, H, Dh, Dh4);
-        row_sums<true>(s.o, D, gb3, Dh, Dh4);
-        cta_mma<false, false>(fr + fo.W3t, H / 16, f.o4p / 16, s.pm, f.o4p + 8, s.ch, nullptr, H);
-        __syncthreads();
-        for (int e = t; e < H * FG; e += FT) s.ch[e] *= 1.0f - s.h2[e] * s.h2[e];
-        __syncthreads();
-        // c_h2: dW2 = c_h2 h1^T, db2, c_h1 = (W2^T c_h2) (1 - h1^2)
-        to_rows(s.ch, H, H, A16);
-        to_rows(s.h1, H, H, B16);
-        to_pm(s.ch, H, H, s.pm, H + 8);
-        __syncthreads();
-        cta_wgrad<false>(A16, H / 16, B16, H / 16, gW2, H, H, H, Dh, Dh4);
-        row_sums<false>(s.ch, H, gb2, Dh, Dh4);
-        cta_mma<false, false>(fr + fo.W2t, H / 16, H / 16, s.pm, H + 8, s.h2, nullptr, H);   // h2 no longer needed
-        __syncthreads();
-        for (int e = t; e < H * FG; e += FT) s.h2[e] *= 1.0f - s.h1[e] * s.h1[e];
-        __syncthreads();
-        // c_h1: dW1 = c_h1 a^T, db1, c_a += W1^T c_h1
-        to_rows(s.h2, H, H, A16);
-        to_rows(in + aoff * FG, Dh, f.kp1, B16);
-        to_pm(s.h2, H, H, s.pm, H + 8);
-        __syncthreads();
-        cta_wgrad<false>(A16, H / 16, B16, f.kp1 / 16, gW1, Dh, H, Dh, Dh, Dh4);
-        row_sums<false>(s.h2, H, gb1, Dh, Dh4);
-        cta_mma<false, false>(fr + fo.W1t, f.kp1 / 16, H / 16, s.pm, H + 8, s.ch, nullptr, Dh4);
-        __syncthreads();
-        for (int e = t; e < Dh * FG; e += FT) s.c[aoff * FG + e] += s.ch[e];
-        __syncthreads();
-    }
-}
-
 // grad[i] = sum over CTAs of partials[c][i], in CTA order.
 __global__ void k_flow_reduce(const float* partials, int64_t n_blocks, int64_t n_params, float* grad,
                               FlowGate gate) {
@@ -1094,9 +735,10 @@ bool flow_bf16_supported(int64_t D, int H, int L) {
     return flow_smem_bytes((int)D, H, L, 2 * Dh4) + flow_pm_bytes() <= 226 * 1024;
 }
 
+// Room of the training gradient's BF16 form, an upper bound of what it takes
 static size_t flow_train_mma_smem_bytes(int D, int H, int L, int O4) {
     return sizeof(float) * (size_t)FG * (2 * D + L * D + 3 * H + O4) + flow_pm_bytes() +
-           sizeof(uint16_t) * 2 * 128 * WLD;
+           sizeof(uint16_t) * 2 * 128 * (FG + 8);
 }
 
 bool flow_train_bf16_supported(int64_t D, int H, int L) {
@@ -1133,11 +775,11 @@ cudaError_t flow_refresh(const DevFlow& f, cudaStream_t s, bool bump, FlowGate g
     return e;
 }
 
-template <int TARGET, bool MMA>
+template <int TARGET>
 static cudaError_t launch_flow_t(const DevModel& m, const DevFlow& f, const TrajArgs& a, float* z0, float* z1,
                                  int64_t grid, cudaStream_t s) {
-    const size_t sm = flow_smem_bytes(f.D, f.H, f.L, f.O4) + (MMA ? flow_pm_bytes() : 0);
-    auto kern = traj_flow_kernel<TARGET, MMA>;
+    const size_t sm = flow_smem_bytes(f.D, f.H, f.L, f.O4);
+    auto kern = traj_flow_kernel<TARGET>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)grid, FT, sm, s>>>(m, f, a, z0, z1);
@@ -1148,11 +790,12 @@ cudaError_t launch_traj_flow(const DevModel& m, const DevFlow& f, const TrajArgs
                              cudaStream_t s) {
     const int64_t grid = (a.N + FG - 1) / FG;
     if (grid == 0) return cudaSuccess;
-    const bool mma = f.bf16 != 0;
-    if (mma && (!f.frag || f.layer_frag <= 0)) return cudaErrorInvalidValue;
-    if (m.kind == GAUSS_DENSE)
-        return mma ? launch_flow_t<0, true>(m, f, a, z0, z1, grid, s) : launch_flow_t<0, false>(m, f, a, z0, z1, grid, s);
-    return mma ? launch_flow_t<1, true>(m, f, a, z0, z1, grid, s) : launch_flow_t<1, false>(m, f, a, z0, z1, grid, s);
+    if (f.bf16 != 0) {
+        if (!f.frag || f.layer_frag <= 0) return cudaErrorInvalidValue;
+        // an evaluation of the target involves no map
+        if (!a.eval_only) return launch_traj_flow_mma(m, f, a, z0, z1, s);
+    }
+    return m.kind == GAUSS_DENSE ? launch_flow_t<0>(m, f, a, z0, z1, grid, s) : launch_flow_t<1>(m, f, a, z0, z1, grid, s);
 }
 
 int64_t flow_partials_floats(const DevFlow& f, int64_t N) { return ((N + FG - 1) / FG) * f.n_params; }
@@ -1164,10 +807,8 @@ cudaError_t flow_loss_grad(const DevFlow& f, const float* theta, int64_t ld, con
     cudaError_t e;
     if (f.train_bf16) {
         if (!f.frag || f.layer_frag <= 0) return cudaErrorInvalidValue;
-        const size_t sm = flow_train_mma_smem_bytes(f.D, f.H, f.L, f.O4);
-        e = cudaFuncSetAttribute(k_flow_train_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = launch_flow_train_mma(f, theta, ld, src, W, gate, N, partials, s);
         if (e != cudaSuccess) return e;
-        k_flow_train_mma<<<(unsigned)grid, FT, sm, s>>>(f, theta, ld, src, W, gate, N, partials);
     } else {
         const size_t sm = flow_smem_bytes(f.D, f.H, f.L, f.O4);
         e = cudaFuncSetAttribute(k_flow_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);

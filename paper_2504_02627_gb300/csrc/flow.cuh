@@ -111,6 +111,11 @@ cudaError_t flow_refresh(const DevFlow& f, cudaStream_t s, bool bump = false, Fl
 // (may be nullptr) receive the latent start and end points [D x ld].
 cudaError_t launch_traj_flow(const DevModel& m, const DevFlow& f, const TrajArgs& a, float* z0, float* z1,
                              cudaStream_t s);
+// ... its BF16 form, and the BF16 form of the training gradient's partials (flow_mma.cu)
+cudaError_t launch_traj_flow_mma(const DevModel& m, const DevFlow& f, const TrajArgs& a, float* z0, float* z1,
+                                 cudaStream_t s);
+cudaError_t launch_flow_train_mma(const DevFlow& f, const float* theta, int64_t ld, const int32_t* src, const double* W,
+                                  FlowGate gate, int64_t N, float* partials, cudaStream_t s);
 // Gradient of the weighted NLL of the particles (theta gathered through src,
 // weights 1/n after resampling, else W) into f.grad, using `partials`
 // (n_blocks x n_params floats) for a fixed-order reduction; with f.train_bf16
