@@ -38,6 +38,7 @@ struct RunParams {
     const double* init_mean;    // [D] device copy, or null (0)
     const double* init_chol;    // [D x D] device copy, row-major lower-triangular, or null (init_scale I)
     double init_logdet;     // sum_d log L_dd (D log init_scale without a factor)
+    double log_n;           // log n (an FP64 logarithm costs a warp 2 us here)
 };
 
 constexpr int SLICE = 128;  // particles per CTA in the weight / statistics kernels (four warps:
@@ -253,6 +254,28 @@ __device__ __forceinline__ int32_t step_count(double h, double L, double eps, in
     return (int32_t)s;
 }
 
+// ---------------------------------------------------------------- FP64, sparingly
+// An SM retires about two FP64 operations per clock, a warp one instruction
+// per 64 clocks, and the FP32 -> FP64 conversion counts as one.  The
+// conversion is exact, so it can be had from integer operations at eight times
+// the rate (16 against 2 lanes per clock and SM).
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x);
+    if (((u >> 23) & 0xffu) - 1u < 254u)
+        return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+    return (double)x;   // subnormal, infinite, NaN
+}
+// Larger of two FP64 values, neither of them NaN, by their bits: the two's
+// complement order of the bits with the magnitude of negative values flipped.
+__device__ __forceinline__ long long order_key(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double from_order_key(long long k) {
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+
 // ---------------------------------------------------------------- FP32 pairs
 // An unevaluated pair hi + lo of FP32 values carries about 48 significant
 // bits.  Sums use Knuth's TwoSum and products the FMA form of Dekker's
@@ -372,6 +395,43 @@ __device__ __forceinline__ void block_reduce_n(T (&v)[N], T* buf, Op op) {
         for (int w = 1; w < nw; ++w) r = op(r, buf[i * 32 + w]);
         v[i] = r;
     }
+}
+
+// N <= 8 FP64 block sums at once, of which thread i < N gets sum i: the bits of
+// block_reduce's tree and warp order.  Within a warp the values are
+// reduce-scattered (a lane keeps half of them at each of the first levels: 9
+// additions instead of 5 N), and the warps' results are added by one thread
+// per sum.  `buf` needs N * 32 entries.
+template <int N>
+__device__ __forceinline__ double block_sums(const double (&in)[N], double* buf) {
+    constexpr int P = N <= 2 ? 2 : N <= 4 ? 4 : 8;
+    static_assert(N >= 1 && N <= 8, "at most eight sums");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double v[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) v[i] = i < N ? in[i < N ? i : 0] : 0.0;
+    int idx = 0, o = 16;
+#pragma unroll
+    for (int h = P / 2; h >= 1; h >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        idx += up ? h : 0;
+        o >>= 1;
+    }
+    for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    __syncthreads();
+    if ((lane & (32 / P - 1)) == 0 && idx < N) buf[idx * 32 + wid] = v[0];
+    __syncthreads();
+    double r = 0.0;
+    if (threadIdx.x < N) {
+        r = buf[threadIdx.x * 32];
+        for (int w = 1; w < nw; ++w) r += buf[threadIdx.x * 32 + w];
+    }
+    return r;
 }
 
 struct OpSum { template <typename T> __device__ T operator()(T a, T b) const { return a + b; } };

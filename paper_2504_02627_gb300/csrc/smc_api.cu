@@ -534,7 +534,9 @@ cudaError_t initial_draw(smc_handle* h) {
     cudaStream_t s = h->stream;
     h->cur = 0;
     StepBufs b = make_bufs(h);
-    cudaError_t ce = launch_init_draw(b, h->theta[0], s);
+    // empty before the first iteration; every iteration's statistics empty it again
+    cudaError_t ce = cudaMemsetAsync(h->hist, 0, sizeof(int32_t) * (size_t)(h->max_steps_all + 1), s);
+    if (ce == cudaSuccess) ce = launch_init_draw(b, h->theta[0], s);
     if (ce == cudaSuccess) {
         TrajArgs a{};
         a.theta_in = h->theta[0];
@@ -710,6 +712,7 @@ smc_status create(smc_handle** out, int64_t n_runs, const smc_config* cfg, const
         rp = RunParams{};
         rp.off = N;
         rp.n = cfg[r].n_particles;
+        rp.log_n = std::log((double)rp.n);
         rp.seed = cfg[r].seed;
         rp.eps = cfg[r].step_size;
         rp.ess_frac = cfg[r].ess_frac;

@@ -71,17 +71,17 @@ __device__ __forceinline__ unsigned long long resample_r64(uint64_t seed, int64_
 
 // Decision for the next iteration from the current log-weights: LSE, ESS
 // (Eqs. for W and J_eff) and the resampling test J_eff < frac J (Sec. 3).
-__device__ __forceinline__ void set_decision(RunState& st, const RunParams& rp, double m, double e1, double e2) {
+__device__ __forceinline__ void set_decision(RunState& st, const RunParams& rp, double m, double lse, double ess,
+                                             double L) {
     if (!(m > -CUDART_INF)) {
         st.status = -4;
         st.resample = 0;
         return;
     }
-    const double ess = e1 * e1 / e2;
-    st.lse = m + log(e1);
+    st.lse = lse;
     st.ess_pre = ess;
     st.resample = ess < rp.ess_frac * (double)rp.n;
-    st.L_used = exp(st.log_L);
+    st.L_used = L;
     st.T = 0ull;
     st.r64 = resample_r64(rp.seed, st.k);
 }
@@ -89,19 +89,20 @@ __device__ __forceinline__ void set_decision(RunState& st, const RunParams& rp, 
 // w_1 = pi(theta_0) / q_init(theta_0) (Eq. for w_1); log Z_0 = LSE(log w) - log J;
 // and the weight decision of iteration 1.
 __global__ void __launch_bounds__(RUN_THREADS) k_init_finish(StepBufs b, const double* logpi) {
-    __shared__ double buf[32];
+    __shared__ double buf[2 * 32], tot_s[2];
+    __shared__ long long lbuf[32];
     const int r = blockIdx.x;
     const RunParams rp = b.runs[r];
-    double m = -CUDART_INF;
+    long long mk = order_key(-CUDART_INF);
     for (int64_t i = threadIdx.x; i < rp.n; i += blockDim.x) {
         const int64_t j = rp.off + i;
         const double lp = logpi[j];
         // independent chains (Algorithm 2) carry no importance weight
         const double lw = rp.mcmc ? 0.0 : (isfinite(lp) ? lp - b.logw[j] : -CUDART_INF);
         b.logw[j] = lw;
-        m = fmax(m, lw);
+        mk = max(mk, order_key(lw));
     }
-    m = block_reduce(m, buf, OpMax());
+    const double m = from_order_key(block_reduce(mk, lbuf, OpMax()));
     double s = 0.0, s2 = 0.0;
     if (m > -CUDART_INF)
         for (int64_t i = threadIdx.x; i < rp.n; i += blockDim.x) {
@@ -109,13 +110,18 @@ __global__ void __launch_bounds__(RUN_THREADS) k_init_finish(StepBufs b, const d
             s += e;
             s2 += e * e;
         }
-    s = block_reduce(s, buf, OpSum());
-    s2 = block_reduce(s2, buf, OpSum());
+    const double sums[2] = {s, s2};
+    const double tot = block_sums(sums, buf);
+    if (threadIdx.x < 2) tot_s[threadIdx.x] = tot;
+    __syncthreads();
     if (threadIdx.x == 0) {
+        s = tot_s[0];
+        s2 = tot_s[1];
         RunState& st = b.rstate[r];
-        st.log_z = (m > -CUDART_INF) ? m + log(s) - log((double)rp.n) : -CUDART_INF;
+        const double lse = (m > -CUDART_INF) ? m + log(s) : -CUDART_INF;
+        st.log_z = (m > -CUDART_INF) ? lse - rp.log_n : -CUDART_INF;
         st.status = 0;
-        set_decision(st, rp, m, s, s2);
+        set_decision(st, rp, m, lse, s * s / s2, exp(st.log_L));
         b.done[r] = 0u;
     }
 }
@@ -541,14 +547,16 @@ __device__ __forceinline__ void block_lse(double a, double* buf, double& M, doub
 
 __global__ void __launch_bounds__(SLICE) k_move_stats(StepBufs b) {
     __shared__ double buf[5 * 32];
-    __shared__ long long lbuf[32];
+    __shared__ long long lbuf[2 * 32];
     __shared__ int ibuf[2 * 32];
     const SliceIdx x = slice_idx(b);
     const RunParams& rp = b.runs[x.r];
     const RunState& st = b.rstate[x.r];
-    if (st.status != 0) return;
     const int c = blockIdx.x;
-    const double logn = log((double)rp.n);
+    // the step histogram of the next iteration starts empty (this one's order
+    // has been made)
+    for (int i = c * SLICE + threadIdx.x; i <= b.max_steps_all; i += gridDim.x * SLICE) b.hist[i] = 0;
+    if (st.status != 0) return;
     double za = -CUDART_INF, lw = -CUDART_INF, al = 0.0;
     long long S = 0;
     int smin = 0x7fffffff, smax = 0;
@@ -556,40 +564,47 @@ __global__ void __launch_bounds__(SLICE) k_move_stats(StepBufs b) {
         // with the Metropolis select the incremental weight is one
         const double dH = rp.accept_reject ? 0.0 : b.dH[x.j];
         const double old = b.logw[x.j];
-        za = (st.resample ? -logn : old - st.lse) - dH;
-        lw = (st.resample ? -logn : old) - dH;
+        za = (st.resample ? -rp.log_n : old - st.lse) - dH;
+        lw = (st.resample ? -rp.log_n : old) - dH;
         b.logw[x.j] = lw;
         al = b.alpha[x.j];
         S = b.steps[x.j];
         smin = smax = (int)S;
     }
     // the slice's reductions, each with block_reduce's tree, in three passes:
-    // the two maxima, then the five sums that need them; the integer parts
-    SlicePart part;
-    double mx[2] = {za, lw};
-    block_reduce_n(mx, buf, OpMax());
-    part.za_m = mx[0];
-    part.w_m = mx[1];
-    const double e = (x.valid && part.w_m > -CUDART_INF) ? exp(lw - part.w_m) : 0.0;
+    // the two maxima (by their bits), then the sums that need them; the
+    // integer parts.  After resampling the two log-weights are the same value.
+    SlicePart& part = b.parts[c];
+    double* const pd = reinterpret_cast<double*>(&part);   // za_m, za_s, w_m, w_e1, w_e2, alpha_sum, inv_alpha_sum
+    long long mx[2] = {order_key(za), order_key(lw)};
+    block_reduce_n(mx, lbuf, OpMax());
+    const double za_m = from_order_key(mx[0]), w_m = from_order_key(mx[1]);
+    const double e = (x.valid && w_m > -CUDART_INF) ? exp(lw - w_m) : 0.0;
+    const double ez = st.resample ? e : (za_m > -CUDART_INF ? exp(za - za_m) : 0.0);
     const bool step_rule = rp.step_rate > 0.0 && st.k < rp.n_warmup;
-    double sm[5] = {part.za_m > -CUDART_INF ? exp(za - part.za_m) : 0.0, e, e * e, al,
-                    step_rule ? (x.valid ? 1.0 / al : 0.0) : 0.0};
-    block_reduce_n(sm, buf, OpSum());
-    part.za_s = sm[0];
-    part.w_e1 = sm[1];
-    part.w_e2 = sm[2];
-    part.alpha_sum = sm[3];
-    part.inv_alpha_sum = step_rule ? sm[4] : 0.0;
+    if (step_rule) {
+        const double sm[5] = {ez, e, e * e, al, x.valid ? 1.0 / al : 0.0};
+        const double r = block_sums(sm, buf);
+        if (threadIdx.x < 5) pd[threadIdx.x == 0 ? 1 : threadIdx.x + 2] = r;
+    } else {
+        const double sm[4] = {ez, e, e * e, al};
+        const double r = block_sums(sm, buf);
+        if (threadIdx.x < 4) pd[threadIdx.x == 0 ? 1 : threadIdx.x + 2] = r;
+        if (threadIdx.x == 4) part.inv_alpha_sum = 0.0;
+    }
     long long ls[1] = {S};
     block_reduce_n(ls, lbuf, OpSum());
-    part.steps_sum = ls[0];
     int mm[2] = {-smin, smax};   // min S as -max(-S)
     block_reduce_n(mm, ibuf, OpMax());
-    part.smin = -mm[0];
-    part.smax = mm[1];
-    part.g_num = 0.0;
-    part.g_den = 0.0;
-    if (threadIdx.x == 0) b.parts[c] = part;
+    if (threadIdx.x == 0) {
+        part.za_m = za_m;
+        part.w_m = w_m;
+        part.steps_sum = ls[0];
+        part.smin = -mm[0];
+        part.smax = mm[1];
+        part.g_num = 0.0;
+        part.g_den = 0.0;
+    }
     if (rp.adapt && st.k < rp.n_warmup) {
         // ChEES column sums of the pre-move states (after resampling) and the
         // proposals: warp w takes dimensions w, w + SLICE / 32, ...; a lane
@@ -643,14 +658,20 @@ __global__ void __launch_bounds__(SLICE) k_move_stats(StepBufs b) {
     }
 }
 
+// Bound by FP64 (an exponential is some 25 instructions) and by the pair sums
+// over the dimensions: 64 hierarchical runs, 278k particles, 129 -> 83 us; one
+// run of 256 particles 13 -> 8 us.
+//
 // Second pass: ChEES gradient estimates g_j = l_j (|t1_j - mean t1|^2 -
 // |t0_j - mean t0|^2) (t1_j - mean t1)' p_j weighted by alpha_j (Algorithm 2),
 // then the last slice of each run combines every slice in a fixed order:
 // evidence, log-weights' ESS, Adam ascent on log L, Lbar, the freeze at
-// M_warmup, statistics, and the weight decision of the next iteration.
+// M_warmup, statistics, and the weight decision of the next iteration.  One run of
+// 256 particles: 34 -> 13 us, nearly all of it the FP64 latency of the last
+// slice's chain.
 __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
-    __shared__ double buf[7 * 32];
-    __shared__ long long lbuf[32];
+    __shared__ double buf[7 * 32], tot_s[7], res_s[4];
+    __shared__ long long lbuf[2 * 32];
     __shared__ int ibuf[2 * 32];
     __shared__ float mean_s[4 * MAX_CHEES_DIM];   // negated means as FP32 pairs: hi [2D], lo [2D]
     __shared__ bool last_s;
@@ -718,12 +739,9 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
             num = a * ((h * st.L_used) * (f2_to_double(sq1) - f2_to_double(sq0)) * f2_to_double(proj));
             den = a;
         }
-        double nd[2] = {num, den};
-        block_reduce_n(nd, buf, OpSum());
-        if (threadIdx.x == 0) {
-            b.parts[c].g_num = nd[0];
-            b.parts[c].g_den = nd[1];
-        }
+        const double nd[2] = {num, den};
+        const double r = block_sums(nd, buf);
+        if (threadIdx.x < 2) (threadIdx.x == 0 ? b.parts[c].g_num : b.parts[c].g_den) = r;
     }
     // Metropolis variant (Eqs. for alpha and the select rule): keep the
     // proposal when u < alpha, otherwise restore the start state; the ChEES
@@ -740,6 +758,8 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
         }
     }
     // ticket: the last slice of the run to get here finishes the iteration
+    if (threadIdx.x < 2) __threadfence();   // the threads that wrote this slice's sums
+    __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         const unsigned int t = atomicAdd(&b.done[x.r], 1u);
@@ -752,16 +772,14 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
     // t, t + SLICE, ... and the block reduces in a fixed tree
     // (the other slices' parts are read from L2 with cache-global loads, after
     // the fence that followed the ticket, so no stale L1 copy is seen)
-    double za_m = -CUDART_INF, w_m = -CUDART_INF;
+    long long mx[2] = {order_key(-CUDART_INF), order_key(-CUDART_INF)};
     for (int q = threadIdx.x; q < rp.n_slices; q += blockDim.x) {
         const SlicePart* p = b.parts + rp.slice0 + q;
-        za_m = fmax(za_m, __ldcg(&p->za_m));
-        w_m = fmax(w_m, __ldcg(&p->w_m));
+        mx[0] = max(mx[0], order_key(__ldcg(&p->za_m)));
+        mx[1] = max(mx[1], order_key(__ldcg(&p->w_m)));
     }
-    double mx[2] = {za_m, w_m};
-    block_reduce_n(mx, buf, OpMax());
-    za_m = mx[0];
-    w_m = mx[1];
+    block_reduce_n(mx, lbuf, OpMax());
+    const double za_m = from_order_key(mx[0]), w_m = from_order_key(mx[1]);
     double za_s = 0.0, w_e1 = 0.0, w_e2 = 0.0, asum = 0.0, gnum = 0.0, gden = 0.0, iasum = 0.0;
     long long ssum = 0;
     int smin = 0x7fffffff, smax = 0;
@@ -795,15 +813,11 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
         smax = max(smax, p.smax);
     }
     // the run's sums, each with block_reduce's tree, in one pass per type
-    double sm[7] = {za_s, w_e1, w_e2, asum, iasum, gnum, gden};
-    block_reduce_n(sm, buf, OpSum());
-    za_s = sm[0];
-    w_e1 = sm[1];
-    w_e2 = sm[2];
-    asum = sm[3];
-    iasum = sm[4];
-    gnum = sm[5];
-    gden = sm[6];
+    {
+        const double sm[7] = {za_s, w_e1, w_e2, asum, iasum, gnum, gden};
+        const double r = block_sums(sm, buf);
+        if (threadIdx.x < 7) tot_s[threadIdx.x] = r;
+    }
     long long ls[1] = {ssum};
     block_reduce_n(ls, lbuf, OpSum());
     ssum = ls[0];
@@ -811,37 +825,66 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
     block_reduce_n(mm, ibuf, OpMax());
     smin = -mm[0];
     smax = mm[1];
-    if (threadIdx.x != 0) return;
-    const int64_t k = st.k;
-    if (adapting) {
-        if (gden > 0.0 && isfinite(gnum / gden)) {
-            const double gh = gnum / gden;
-            st.adam_t += 1.0;
-            st.adam_m = rp.adam_b1 * st.adam_m + (1.0 - rp.adam_b1) * gh;
-            st.adam_v = rp.adam_b2 * st.adam_v + (1.0 - rp.adam_b2) * gh * gh;
-            st.adam_b1t *= rp.adam_b1;     // b1^t, b2^t by running products (no FP64 pow)
-            st.adam_b2t *= rp.adam_b2;
-            const double mh = st.adam_m / (1.0 - st.adam_b1t);
-            const double vh = st.adam_v / (1.0 - st.adam_b2t);
-            st.log_L += rp.adam_lr * mh / (sqrt(vh) + rp.adam_eps);
-            // clamp L to [eps, max_steps eps] of this iteration's step size
-            const double lo = rp.step_rate > 0.0 ? log(st.eps) : rp.log_L_lo;
-            const double hi = rp.step_rate > 0.0 ? log((double)rp.max_steps * st.eps) : rp.log_L_hi;
-            st.log_L = fmin(fmax(st.log_L, lo), hi);
+    // (the barriers above order tot_s)
+    // The run's update is a chain of FP64 logarithms, exponentials and
+    // divisions, a microsecond each in one thread: its independent parts run in
+    // one warp each.  Warp 1: the evidence factor; warp 2: the new LSE; warp 3:
+    // the ESS and the mean acceptance; warp 0: Adam on log L.
+    const int wid = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0 && wid > 0) {
+        if (wid == 1) res_s[0] = za_m > -CUDART_INF ? za_m + log(tot_s[0]) : -CUDART_INF;
+        if (wid == 2) res_s[1] = w_m > -CUDART_INF ? w_m + log(tot_s[1]) : -CUDART_INF;
+        if (wid == 3) {
+            res_s[2] = w_m > -CUDART_INF ? tot_s[1] * tot_s[1] / tot_s[2] : 0.0;
+            res_s[3] = tot_s[3] / (double)rp.n;
         }
-        st.Lbar = 0.9 * st.Lbar + 0.1 * exp(st.log_L);
     }
-    if (rp.adapt && k == rp.n_warmup && st.Lbar > 0.0) st.log_L = log(st.Lbar);
-    // optional warm-up step-size rule (not in the paper), after the ChEES
-    // update: log eps += rate (a_h - target), a_h = n / sum 1/alpha_j the
-    // harmonic mean (0 when some alpha_j = 0: the sum is +inf)
-    if (rp.step_rate > 0.0 && k < rp.n_warmup)
-        st.eps = exp(log(st.eps) + rp.step_rate * ((double)rp.n / iasum - rp.step_target));
-    const double inc = za_m > -CUDART_INF ? za_m + log(za_s) : -CUDART_INF;
+    const int64_t k = st.k;
+    double L_next = 0.0;      // exp(log L) of the next iteration
+    if (threadIdx.x == 0) {
+        bool have = false;
+        double log_L = st.log_L;
+        if (adapting) {
+            gnum = tot_s[5];
+            gden = tot_s[6];
+            if (gden > 0.0 && isfinite(gnum / gden)) {
+                const double gh = gnum / gden;
+                st.adam_t += 1.0;
+                st.adam_m = rp.adam_b1 * st.adam_m + (1.0 - rp.adam_b1) * gh;
+                st.adam_v = rp.adam_b2 * st.adam_v + (1.0 - rp.adam_b2) * gh * gh;
+                st.adam_b1t *= rp.adam_b1;     // b1^t, b2^t by running products (no FP64 pow)
+                st.adam_b2t *= rp.adam_b2;
+                const double mh = st.adam_m / (1.0 - st.adam_b1t);
+                const double vh = st.adam_v / (1.0 - st.adam_b2t);
+                log_L += rp.adam_lr * mh / (sqrt(vh) + rp.adam_eps);
+                // clamp L to [eps, max_steps eps] of this iteration's step size
+                const double lo = rp.step_rate > 0.0 ? log(st.eps) : rp.log_L_lo;
+                const double hi = rp.step_rate > 0.0 ? log((double)rp.max_steps * st.eps) : rp.log_L_hi;
+                log_L = fmin(fmax(log_L, lo), hi);
+            }
+            L_next = exp(log_L);
+            have = true;
+            st.Lbar = 0.9 * st.Lbar + 0.1 * L_next;
+        }
+        if (rp.adapt && k == rp.n_warmup && st.Lbar > 0.0) {
+            log_L = log(st.Lbar);
+            have = false;
+        }
+        st.log_L = log_L;
+        if (!have) L_next = exp(log_L);
+        // optional warm-up step-size rule (not in the paper), after the ChEES
+        // update: log eps += rate (a_h - target), a_h = n / sum 1/alpha_j the
+        // harmonic mean (0 when some alpha_j = 0: the sum is +inf)
+        if (rp.step_rate > 0.0 && k < rp.n_warmup)
+            st.eps = exp(log(st.eps) + rp.step_rate * ((double)rp.n / tot_s[4] - rp.step_target));
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    const double inc = res_s[0];
     st.log_z += inc;
     st.log_z_inc = inc;
-    st.mean_alpha = asum / (double)rp.n;
-    st.ess = w_m > -CUDART_INF ? w_e1 * w_e1 / w_e2 : 0.0;
+    st.mean_alpha = res_s[3];
+    st.ess = res_s[2];
     st.stat_ess_pre = st.ess_pre;
     st.stat_resampled = st.resample;
     st.L_last = st.L_used;
@@ -854,7 +897,7 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
     st.ess_sum += st.ess;
     if (k > rp.n_warmup) st.ess_sum_post += st.ess;
     st.k = k + 1;
-    set_decision(st, rp, w_m, w_e1, w_e2);
+    set_decision(st, rp, w_m, res_s[1], res_s[2], L_next);
     b.done[x.r] = 0u;
 }
 
@@ -869,8 +912,6 @@ cudaError_t launch_init_finish(const StepBufs& b, const double* logpi, cudaStrea
     return cudaGetLastError();
 }
 cudaError_t launch_weights_steps(const StepBufs& b, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(b.hist, 0, sizeof(int32_t) * (size_t)(b.max_steps_all + 1), s);
-    if (e != cudaSuccess) return e;
     k_weights_steps<<<(unsigned)b.n_slices, SLICE, 0, s>>>(b);
     return cudaGetLastError();
 }

@@ -55,11 +55,11 @@ __device__ __forceinline__ void banana_grad(float a, float b, float inva, float 
 // particles' pairs, warp w taking pairs w, w + PW, ..., NPT of them side by
 // side (independent chains that fill each other's latency).  Loads and stores
 // are those of 32 consecutive particles of one dimension.  The FP64 sums (p'p
-// before and after, log pi) run in the order of the dimensions, by the group's
-// first warp from shared memory, so they have the bits of a thread that holds
-// the whole particle.  Bound by the FMA pipe (12 operations a pair and step)
+// before and after, log pi) run in the order of the dimensions, a warp each,
+// from shared memory, so they have the bits of a thread that holds the whole
+// particle.  Bound by the FMA pipe (12 operations a pair and step)
 // and, in unsorted launches, by the longest of a warp's 32 trajectories: 50-d,
-// 8192 particles, up to 100 steps 59.6 -> 44.6 us with the caller's copies (29
+// 8192 particles, up to 100 steps 59.6 -> 38.9 us with the caller's copies (24
 // of them this kernel; a thread per particle filled 64 CTAs).
 template <int NPT>
 __global__ void __launch_bounds__(256) traj_banana_kernel(DevModel m, TrajArgs a, int pw) {
@@ -69,9 +69,10 @@ __global__ void __launch_bounds__(256) traj_banana_kernel(DevModel m, TrajArgs a
     const int w = wid % pw, grp = wid / pw, ngrp = (blockDim.x >> 5) / pw;
     const int64_t t = ((int64_t)blockIdx.x * ngrp + grp) * 32 + lane;
     const bool on = t < a.N;
-    float* sp0 = sm + (size_t)grp * 32 * (2 * D + np);     // [D][32] momenta before
+    float* sp0 = sm + (size_t)grp * 32 * (2 * D + np + 6); // [D][32] momenta before
     float* sp1 = sp0 + 32 * D;                              // [D][32] momenta after
     float* slp = sp1 + 32 * D;                              // [np][32] log pi terms
+    double* se = reinterpret_cast<double*>(slp + 32 * np);   // [3][32] log pi, p'p before and after
     const float fa = (float)m.h0, fb = (float)m.h1, inva = (float)(1.0 / m.h0), half_inva = (float)(0.5 / m.h0);
     Slot x{};
     double lp0 = 0.0;
@@ -136,22 +137,28 @@ __global__ void __launch_bounds__(256) traj_banana_kernel(DevModel m, TrajArgs a
         }
     }
     __syncthreads();
-    if (!on || w != 0) return;
-    double s = 0.0;
-    for (int i = 0; i < np; ++i) s += (double)slp[i * 32 + lane];
-    double kin0 = 0.0, kin1 = 0.0;
-    if (!a.eval_only)
-        for (int d = 0; d < D; ++d) {
-            const float v0 = sp0[d * 32 + lane], v1 = sp1[d * 32 + lane];
-            kin0 += (double)v0 * (double)v0;
-            kin1 += (double)v1 * (double)v1;
+    // three warps (of four schedulers) take a sum each: an FP64 instruction
+    // occupies a warp's scheduler for 64 clocks
+    if (on)
+        for (int e = w; e < (a.eval_only ? 1 : 3); e += pw) {
+            double s = 0.0;
+            if (e == 0)
+                for (int i = 0; i < np; ++i) s += widen(slp[i * 32 + lane]);
+            else
+                for (int d = 0; d < D; ++d) {
+                    const double v = widen((e == 1 ? sp0 : sp1)[d * 32 + lane]);
+                    s += v * v;
+                }
+            se[e * 32 + lane] = s;
         }
-    finish(a, x.j, s + m.lconst, 0.5 * kin0 - lp0, kin1);
+    __syncthreads();
+    if (on && w == 0)
+        finish(a, x.j, se[lane] + m.lconst, a.eval_only ? 0.0 : 0.5 * se[32 + lane] - lp0, a.eval_only ? 0.0 : se[64 + lane]);
 }
 
 template <int NPT>
 cudaError_t launch_banana_n(const DevModel& m, const TrajArgs& a, int pw, int ngrp, cudaStream_t s) {
-    const size_t sm = (size_t)ngrp * 32 * (2 * m.D + m.D / 2) * sizeof(float);
+    const size_t sm = (size_t)ngrp * 32 * (2 * m.D + m.D / 2 + 6) * sizeof(float);
     auto kern = traj_banana_kernel<NPT>;
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -169,7 +176,7 @@ cudaError_t launch_banana_n(const DevModel& m, const TrajArgs& a, int pw, int ng
 // row's sum in the order of the columns (the sum, and so every bit, of a
 // thread that holds the whole particle).  Bound by the step's chain (exchange
 // and one row's sum): the 10-d Gaussian's move of 256 particles, up to about 100
-// steps, takes 11.6 instead of 30.5 us, its 20-iteration run 1.51 -> 1.16 ms.
+// steps, takes 9 instead of 30.5 us.
 template <int G>
 __global__ void __launch_bounds__(128) traj_gauss_rows_kernel(DevModel m, TrajArgs a) {
     constexpr int PPC = 128 / G;                       // particles per CTA
@@ -238,19 +245,21 @@ __global__ void __launch_bounds__(128) traj_gauss_rows_kernel(DevModel m, TrajAr
         }
     }
     __syncwarp(gmask);
-    if (r != 0) return;
     // log pi = c + 1/2 (theta - mu)' g: FP32 products, FP64 accumulation in
-    // the order of the dimensions, as are the kinetic energies
-    double q = 0.0, kin0 = 0.0, kin1 = 0.0;
-    for (int d = 0; d < D; ++d) {
-        q += (double)q_s[pi][d];
-        if (!a.eval_only) {
-            kin0 += (double)p0_s[pi][d] * (double)p0_s[pi][d];
-            kin1 += (double)p1_s[pi][d] * (double)p1_s[pi][d];
+    // the order of the dimensions, as are the kinetic energies; lanes 0, 1 and
+    // 2 take one of the three sums each, in the same instructions
+    double sum = 0.0;
+    if (r < 3 && (r == 0 || !a.eval_only)) {
+        const float* v = r == 0 ? q_s[pi] : r == 1 ? p0_s[pi] : p1_s[pi];
+        for (int d = 0; d < D; ++d) {
+            const double e = widen(v[d]);
+            sum = fma(e, r == 0 ? 1.0 : e, sum);
         }
     }
+    const double kin0 = __shfl_sync(gmask, sum, 1, G), kin1 = __shfl_sync(gmask, sum, 2, G);
+    if (r != 0) return;
     const double lp0 = a.eval_only ? 0.0 : a.logpi_in[x.src];
-    finish(a, x.j, m.lconst + 0.5 * q, 0.5 * kin0 - lp0, kin1);
+    finish(a, x.j, m.lconst + 0.5 * sum, 0.5 * kin0 - lp0, kin1);
 }
 
 template <int G>

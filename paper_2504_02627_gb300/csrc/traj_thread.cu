@@ -63,7 +63,7 @@ struct GaussDenseM {
     // FP64 accumulation (the FP64 quadratic form costs D^2 operations at the
     // FP64 rate, a small fraction of the FP32 rate here)
     __device__ static double energy_term(const float* sm, const float (&th)[DM], int d, float g) {
-        return (double)((th[d] - sm[DM * LD + d]) * g);
+        return widen((th[d] - sm[DM * LD + d]) * g);
     }
     __device__ static double logpi(const DevModel& m, const float*, const float (&)[DM], double q) {
         return m.lconst + 0.5 * q;
@@ -132,7 +132,7 @@ struct HierM {
                 const float eta = th[d];
                 const float dev = sm[2 * k] - fmaf(tau, eta, mu);
                 const float term = -fmaf(sm[2 * m.n + k] * dev, dev, sm[3 * m.n + k]) * inv_2s2 - 0.5f * eta * eta;
-                s += (double)term;
+                s += widen(term);
             }
         }
         return s + m.lconst;
@@ -182,7 +182,11 @@ __device__ __forceinline__ void particle_move(const DevModel& m, const TrajArgs&
     }
     double kin0 = 0.0;
 #pragma unroll
-    for (int d = 0; d < DM; ++d) kin0 += (double)p[d] * (double)p[d];
+    for (int d = 0; d < DM; ++d)
+        if (d < D) {
+            const double v = widen(p[d]);
+            kin0 += v * v;
+        }
     const double H0 = 0.5 * kin0 - lp0;
 
     const int S = a.steps[j];
@@ -220,7 +224,11 @@ __device__ __forceinline__ void particle_move(const DevModel& m, const TrajArgs&
     const double lp1 = M::logpi(m, sm, th, q);
     double kin1 = 0.0;
 #pragma unroll
-    for (int d = 0; d < DM; ++d) kin1 += (double)p[d] * (double)p[d];
+    for (int d = 0; d < DM; ++d)
+        if (d < D) {
+            const double v = widen(p[d]);
+            kin1 += v * v;
+        }
     double dH = (0.5 * kin1 - lp1) - H0;
     if (!isfinite(dH)) dH = CUDART_INF;
 #pragma unroll
