@@ -109,7 +109,10 @@ enum : uint32_t { TAG_INIT = 1, TAG_MOM = 2, TAG_RESAMPLE = 3, TAG_MH = 4, TAG_J
 // value is (m + 0.5) 2^-52, exact in FP64.
 __device__ __forceinline__ double u01_52(uint32_t a, uint32_t b) {
     uint64_t m = ((uint64_t)(a >> 6) << 26) | (uint64_t)(b >> 6);
-    return ((double)m + 0.5) * 2.220446049250313080847263336181640625e-16;  // 2^-52
+    // (m + 1/2) 2^-52 as (1 + m 2^-52) - (1 - 2^-53): both terms and the result
+    // are exact, and one FP64 addition replaces a conversion, an addition and
+    // a product
+    return __hiloint2double((int)(0x3ff00000u | (uint32_t)(m >> 32)), (int)(uint32_t)m) - 0.99999999999999988897769753748434596;
 }
 
 // Two standard normals from one Philox block by Box-Muller in FP64.

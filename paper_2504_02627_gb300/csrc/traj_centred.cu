@@ -88,7 +88,7 @@ constexpr float C_X_MAX = 60.0f;           // clamp of the exponent: two factors
 
 struct CLayout {
     int atoms, tile_bytes, ref_bytes, stage_bytes, stages, xbufs;
-    int off_d, off_stage, off_gx, off_emisc, off_cref, off_bar, total;
+    int off_d, off_stage, off_gx, off_emisc, off_cref, off_bar, off_state, total;
 };
 
 // Byte layout of the dynamic shared memory (from a 1024-aligned base) with
@@ -116,6 +116,7 @@ __host__ __device__ inline CLayout c_layout_n(int dk, int Dp, int n_ref, int n_r
     const int endx = L.off_emisc + 9 * CP * 8;
     L.off_cref = ((pipe > endx ? pipe : endx) + 1023) & ~1023;
     L.off_bar = L.off_cref + 2 * n_run * dk * 4;          // reference points, reference gradients [runs][dk]
+    L.off_state = 0;
     L.total = L.off_bar + 256 + 1024;                     // + alignment slack of the base
     // more than half of the SM's shared memory, so that a second CTA, which
     // would wait for the 512 TMEM columns, is never co-scheduled
@@ -123,11 +124,20 @@ __host__ __device__ inline CLayout c_layout_n(int dk, int Dp, int n_ref, int n_r
     return L;
 }
 // The most X stages that fit (4, 3 or 2) with a double-buffered end point,
-// else two stages with a single end-point buffer.
-__host__ __device__ inline CLayout c_layout(int dk, int Dp, int n_ref, int n_run) {
+// else two stages with a single end-point buffer.  A CTA that is not part of a
+// cluster also keeps the move's theta and p there ([dk][128] each) when they
+// fit next to the stages: the update at a pass's end then waits for no L2
+// round trip (ten runs of 4096 particles, n = 1000, D = 25: a move of about
+// 375 steps 9.80 -> 9.48 ms).
+__host__ __device__ inline CLayout c_layout(int dk, int Dp, int n_ref, int n_run, bool alone) {
     CLayout L = c_layout_n(dk, Dp, n_ref, n_run, C_NS_MAX, 2);
     for (int st = C_NS_MAX - 1; st >= 2 && L.total > C_SMEM_MAX; --st) L = c_layout_n(dk, Dp, n_ref, n_run, st, 2);
     if (L.total > C_SMEM_MAX) L = c_layout_n(dk, Dp, n_ref, n_run, 2, 1);
+    const int state = L.off_bar + 256;
+    if (alone && state + 2 * dk * CP * 4 + 1024 <= C_SMEM_MAX) {
+        L.off_state = state;
+        if (L.total < state + 2 * dk * CP * 4 + 1024) L.total = state + 2 * dk * CP * 4 + 1024;
+    }
     return L;
 }
 
@@ -147,7 +157,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
     // 1024-aligned base by pointer arithmetic on the shared array, so that
     // accesses through it stay shared-space loads and stores
     unsigned char* sm = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
-    const CLayout L = c_layout(m.dk, m.Dp, LOGIT ? 1 : 0, a.c_runs);
+    const CLayout L = c_layout(m.dk, m.Dp, LOGIT ? 1 : 0, a.c_runs, a.c_split == 1);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int D = m.D, dk = m.dk, nch_all = m.n_tiles128;
     const int64_t ld = a.ld;
@@ -242,10 +252,12 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
     const float inv_s2 = LOGIT ? 0.0f : (float)(1.0 / (m.h0 * m.h0));
     const float inv_s = LOGIT ? 0.0f : (float)(1.0 / m.h0);
     const bool evalm = a.eval_only != 0;
-    const bool slotst = a.c_sth != nullptr && a.c_sp != nullptr && !evalm;
-    float* const thb = slotst ? a.c_sth : a.theta_out;
-    float* const pb = slotst ? a.c_sp : a.p_out;
-    const int64_t sld = slotst ? a.c_sld : ld;           // stride of thb / pb
+    // the state is kept by slot: in shared memory, else in c_sth / c_sp
+    const bool smst = L.off_state > 0 && !evalm;
+    const bool slotst = smst || (a.c_sth != nullptr && a.c_sp != nullptr && !evalm);
+    float* const thb = smst ? reinterpret_cast<float*>(sm + L.off_state) : slotst ? a.c_sth : a.theta_out;
+    float* const pb = smst ? thb + dk * CP : slotst ? a.c_sp : a.p_out;
+    const int64_t sld = smst ? CP : slotst ? a.c_sld : ld;   // stride of thb / pb
     int64_t j = -1, src = -1;
     int S = 0, run = 0;
     float ef = 0.0f;
@@ -290,8 +302,9 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
                             if (d + e < D) {
                                 kin += (double)pv[e] * (double)pv[e];
                                 if (own) {
-                                    pb[(int64_t)(d + e) * sld + (slotst ? t : j)] = pv[e];
-                                    thb[(int64_t)(d + e) * sld + (slotst ? t : j)] = tv[e];
+                                    const int64_t o = (int64_t)(d + e) * sld + (smst ? prow : slotst ? t : j);
+                                    pb[o] = pv[e];
+                                    thb[o] = tv[e];
                                 }
                             }
                     }
@@ -306,7 +319,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
         if (epi) kin0_s[q * CP + prow] = kin;
     }
     const float* cref = cref_s + run * dk;                // this particle's run reference point
-    const int64_t si = slotst ? slot0 + prow : j;         // index of this thread's state in thb / pb
+    const int64_t si = smst ? prow : slotst ? slot0 + prow : j;   // index of this thread's state in thb / pb
     // deviation operand: unit u (8 dimensions) of this thread's 32 dimensions
     // of its particle row, BF16, swizzled
     auto write_unit = [&](int u, const float* tv) {
@@ -887,45 +900,46 @@ __global__ void __launch_bounds__(256) k_centre_mean(TrajArgs a, int D, int dk) 
 // tile's (c, s) pairs c = -log2(e) eta_ref, s = sigmoid(eta_ref) for the
 // logistic model, and the tile's part of g_ref = X'(y - s) (logistic, with the
 // FP32 s the kernel subtracts from) or X'(y - eta_ref) / sigma^2 (linear).
+// One CTA per tile and run; FP64 bound, so the conversions are integer
+// operations (widen) and the reference point is converted once (ten runs, n =
+// 1000: 138 us with one CTA per tile over all runs, now 16).
 template <bool LOGIT>
 __global__ void __launch_bounds__(128) k_centre_obs(DevModel m, TrajArgs a) {
-    __shared__ double rr[CC];
-    const int c = blockIdx.x, t = threadIdx.x;
+    __shared__ double rr[CC], cr[128];
+    const int c = blockIdx.x, r = blockIdx.y, t = threadIdx.x;
     const int64_t i = (int64_t)c * CC + t;
     const int D = m.D, dk = m.dk, Dp = m.Dp, R = a.c_runs;
-    for (int r = 0; r < R; ++r) {
-        const float* cr = a.c_centre + (int64_t)r * dk;
-        double res = 0.0;
-        float2 cs = make_float2(0.0f, 0.5f);
-        if (i < m.n) {
-            double eta = 0.0;
-            for (int d = 0; d < D; ++d) eta += (double)m.X[i * Dp + d] * (double)cr[d];
-            if (LOGIT) {
-                const float s = (float)(1.0 / (1.0 + exp(-eta)));
-                cs = make_float2((float)(-1.4426950408889634 * eta), s);
-                res = (double)m.y[i] - (double)s;
-            } else {
-                res = ((double)m.y[i] - eta) / (m.h0 * m.h0);
-            }
-        }
+    if (t < D) cr[t] = widen(a.c_centre[(int64_t)r * dk + t]);
+    __syncthreads();
+    double res = 0.0;
+    float2 cs = make_float2(0.0f, 0.5f);
+    if (i < m.n) {
+        double eta = 0.0;
+        for (int d = 0; d < D; ++d) eta += widen(m.X[i * Dp + d]) * cr[d];
         if (LOGIT) {
-            // an observation pair's values as (c0, c1, s0, s1): the
-            // epilogue's packed FMAs take each pair from adjacent registers
-            float* fr = reinterpret_cast<float*>(a.c_refs + ((int64_t)c * R + r) * CC);
-            fr[4 * (t >> 1) + (t & 1)] = cs.x;
-            fr[4 * (t >> 1) + 2 + (t & 1)] = cs.y;
+            const float s = (float)(1.0 / (1.0 + exp(-eta)));
+            cs = make_float2((float)(-1.4426950408889634 * eta), s);
+            res = (double)m.y[i] - (double)s;
+        } else {
+            res = ((double)m.y[i] - eta) / (m.h0 * m.h0);
         }
-        rr[t] = res;
-        __syncthreads();
-        if (t < dk) {
-            double g = 0.0;
-            if (t < D) {
-                const int rows = (int)((int64_t)m.n - (int64_t)c * CC < CC ? (int64_t)m.n - (int64_t)c * CC : CC);
-                for (int o = 0; o < rows; ++o) g += (double)m.X[((int64_t)c * CC + o) * Dp + t] * rr[o];
-            }
-            a.c_part[((int64_t)c * R + r) * dk + t] = g;
+    }
+    if (LOGIT) {
+        // an observation pair's values as (c0, c1, s0, s1): the epilogue's
+        // packed FMAs take each pair from adjacent registers
+        float* fr = reinterpret_cast<float*>(a.c_refs + ((int64_t)c * R + r) * CC);
+        fr[4 * (t >> 1) + (t & 1)] = cs.x;
+        fr[4 * (t >> 1) + 2 + (t & 1)] = cs.y;
+    }
+    rr[t] = res;
+    __syncthreads();
+    if (t < dk) {
+        double g = 0.0;
+        if (t < D) {
+            const int rows = (int)((int64_t)m.n - (int64_t)c * CC < CC ? (int64_t)m.n - (int64_t)c * CC : CC);
+            for (int o = 0; o < rows; ++o) g += widen(m.X[((int64_t)c * CC + o) * Dp + t]) * rr[o];
         }
-        __syncthreads();
+        a.c_part[((int64_t)c * R + r) * dk + t] = g;
     }
 }
 
@@ -1023,7 +1037,10 @@ cudaError_t launch_centred(const DevModel& m, const TrajArgs& a, cudaStream_t s)
     // stage then carries the reference pairs of its own run only
     if (R > 1 && (!a.c_tiles || !a.c_perm || !a.c_padoff || !a.c_pcnt || a.c_ntiles < 1))
         return cudaErrorInvalidValue;
-    const CLayout L = c_layout(m.dk, m.Dp, LOGIT ? 1 : 0, R);
+    const int64_t tiles = a.c_tiles ? a.c_ntiles : (a.N + CP - 1) / CP;
+    TrajArgs a2 = a;
+    a2.c_split = centred_split(m, tiles);
+    const CLayout L = c_layout(m.dk, m.Dp, LOGIT ? 1 : 0, R, a2.c_split == 1);
     if (L.total > C_SMEM_MAX) return cudaErrorInvalidValue;
     if (a.c_tiles) {
         const int64_t nblk = (a.N + 1023) / 1024;
@@ -1032,13 +1049,10 @@ cudaError_t launch_centred(const DevModel& m, const TrajArgs& a, cudaStream_t s)
         k_part_scatter<<<(unsigned)nblk, 1024, 0, s>>>(a, nblk);
     }
     k_centre_mean<<<dim3((unsigned)R, (unsigned)m.dk), 256, 0, s>>>(a, m.D, m.dk);
-    k_centre_obs<LOGIT><<<(unsigned)m.n_tiles128, 128, 0, s>>>(m, a);
+    k_centre_obs<LOGIT><<<dim3((unsigned)m.n_tiles128, (unsigned)R), 128, 0, s>>>(m, a);
     k_centre_grad<<<(unsigned)R, 128, 0, s>>>(a, m.dk, m.n_tiles128);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int64_t tiles = a.c_tiles ? a.c_ntiles : (a.N + CP - 1) / CP;
-    TrajArgs a2 = a;
-    a2.c_split = centred_split(m, tiles);
     auto kern = traj_centred_kernel<LOGIT>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
     if (e != cudaSuccess) return e;
