@@ -306,18 +306,98 @@ __device__ unsigned long long lookback_prefix(TileDesc* tiles, int64_t g, int64_
 // its range slot by slot is the whole launch.
 constexpr unsigned int EMIT_SHORT = 8, EMIT_BLOCK = 2048;
 
+struct EmitList {
+    unsigned int lo[SCAN_TILE], hi[SCAN_TILE];   // a tile's long output ranges
+    int i[SCAN_TILE];
+    int n;
+};
+
+// Inclusive prefixes of this thread's SCAN_ITEMS consecutive values (zero past
+// n); returns the exclusive prefix of the thread within the tile and, in
+// tile_agg, the tile's total.
+__device__ __forceinline__ unsigned long long tile_scan(const unsigned long long* q, int64_t base, int64_t n,
+                                                        unsigned long long (&v)[SCAN_ITEMS], unsigned long long* wsum,
+                                                        unsigned long long& tile_agg) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    unsigned long long acc = 0ull;
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) {
+        const int64_t i = base + (int64_t)tid * SCAN_ITEMS + k;
+        acc += i < n ? q[i] : 0ull;
+        v[k] = acc;
+    }
+    unsigned long long x = acc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    unsigned long long before = 0ull;
+    tile_agg = 0ull;
+#pragma unroll
+    for (int w = 0; w < SCAN_THREADS / 32; ++w) {
+        before += w < wid ? wsum[w] : 0ull;
+        tile_agg += wsum[w];
+    }
+    return before + (x - acc);
+}
+
+// Systematic resampling of a tile: particle i (run-local) owns the output slots
+// [cnt(C_{i-1}), cnt(C_i)), C its inclusive prefix off + v.  list.n is zero
+// and all threads are past a barrier since then.
+__device__ __forceinline__ void emit_systematic(const unsigned long long (&v)[SCAN_ITEMS], unsigned long long off,
+                                                int64_t base, int64_t n, unsigned long long T, unsigned long long U,
+                                                int32_t* anc, int32_t* src, int32_t src0, EmitList& list) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned long long N = (unsigned long long)n;
+    const float rT = 1.0f / (float)T;
+    // a particle's range ends where the next one's begins: one count per particle
+    unsigned int lo = (unsigned int)systematic_count(off, N, T, U, rT);
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) {
+        const int64_t i = base + (int64_t)tid * SCAN_ITEMS + k;
+        if (i >= n) break;
+        const unsigned int hi = (unsigned int)systematic_count(off + v[k], N, T, U, rT);
+        if (hi - lo > EMIT_SHORT && hi > lo) {
+            const int e = atomicAdd(&list.n, 1);   // the list's order does not matter: disjoint ranges
+            list.lo[e] = lo;
+            list.hi[e] = hi;
+            list.i[e] = (int)i;
+        } else {
+            for (unsigned int o = lo; o < hi; ++o) {
+                anc[o] = (int32_t)i;
+                if (src) src[o] = src0 + (int32_t)i;
+            }
+        }
+        lo = hi;
+    }
+    __syncthreads();
+    const int nl = list.n;
+    for (int e = 0; e < nl; ++e) {
+        const unsigned int l = list.lo[e], h = list.hi[e];
+        const int32_t i = list.i[e];
+        const bool by_block = h - l >= EMIT_BLOCK;
+        if (!by_block && (e % (SCAN_THREADS / 32)) != wid) continue;
+        const unsigned int step = by_block ? SCAN_THREADS : 32u;
+        for (unsigned int o = l + (by_block ? (unsigned)tid : (unsigned)lane); o < h; o += step) {
+            anc[o] = i;
+            if (src) src[o] = src0 + i;
+        }
+    }
+}
+
 __global__ void __launch_bounds__(SCAN_THREADS) k_resample_scan(StepBufs b) {
     __shared__ unsigned int tile_s;
     __shared__ unsigned long long wsum[SCAN_THREADS / 32];
     __shared__ unsigned long long excl_s;
     __shared__ int failed_s;
-    __shared__ unsigned int long_lo[SCAN_TILE], long_hi[SCAN_TILE];   // the tile's long output ranges
-    __shared__ int long_i[SCAN_TILE];
-    __shared__ int n_long;
+    __shared__ EmitList list;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid == 0) {
         tile_s = atomicAdd(b.counter, 1u);
-        n_long = 0;
+        list.n = 0;
     }
     __syncthreads();
     const int64_t g = tile_s;
@@ -336,44 +416,15 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_resample_scan(StepBufs b) {
         return;
     }
     const unsigned int epoch = b.counter[1] & 0x3fffffffu;
-    const unsigned long long N = (unsigned long long)rp.n, T = st.T;
+    const unsigned long long T = st.T;
     if (T == 0ull) {                 // no mass at all: degenerate
         if (tid == 0) st.status = -4;
         return;
     }
     const unsigned long long U = __umul64hi(st.r64, T);
 
-    // thread-local inclusive prefix of SCAN_ITEMS consecutive elements
-    unsigned long long v[SCAN_ITEMS];
-    unsigned long long acc = 0ull;
-#pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; ++k) {
-        const int64_t i = base + (int64_t)tid * SCAN_ITEMS + k;
-        const unsigned long long x = i < rp.n ? b.q[rp.off + i] : 0ull;
-        acc += x;
-        v[k] = acc;
-    }
-    // block exclusive scan of the per-thread totals
-    unsigned long long x = acc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        unsigned long long w = lane < SCAN_THREADS / 32 ? wsum[lane] : 0ull;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        if (lane < SCAN_THREADS / 32) wsum[lane] = w;
-    }
-    __syncthreads();
-    const unsigned long long thread_excl = (x - acc) + (wid > 0 ? wsum[wid - 1] : 0ull);
-    const unsigned long long tile_agg = wsum[SCAN_THREADS / 32 - 1];
+    unsigned long long v[SCAN_ITEMS], tile_agg;
+    const unsigned long long thread_excl = tile_scan(b.q + rp.off, base, rp.n, v, wsum, tile_agg);
 
     // look-back over predecessor tiles of the same run
     if (wid == 0) {
@@ -410,42 +461,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_resample_scan(StepBufs b) {
         }
         return;
     }
-    const float rT = 1.0f / (float)T;
-    int32_t* const anc = b.anc + rp.off;
-    int32_t* const src = b.src ? b.src + rp.off : nullptr;
-    // a particle's range ends where the next one's begins: one count per particle
-    unsigned int lo = (unsigned int)systematic_count(off, N, T, U, rT);
-#pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; ++k) {
-        const int64_t i = base + (int64_t)tid * SCAN_ITEMS + k;
-        if (i >= rp.n) break;
-        const unsigned int hi = (unsigned int)systematic_count(off + v[k], N, T, U, rT);
-        if (hi - lo > EMIT_SHORT && hi > lo) {
-            const int e = atomicAdd(&n_long, 1);   // the list's order does not matter: disjoint ranges
-            long_lo[e] = lo;
-            long_hi[e] = hi;
-            long_i[e] = (int)i;
-        } else {
-            for (unsigned int o = lo; o < hi; ++o) {
-                anc[o] = (int32_t)i;
-                if (src) src[o] = (int32_t)(rp.off + i);
-            }
-        }
-        lo = hi;
-    }
-    __syncthreads();
-    const int nl = n_long;
-    for (int e = 0; e < nl; ++e) {
-        const unsigned int l = long_lo[e], h = long_hi[e];
-        const int32_t i = long_i[e];
-        const bool by_block = h - l >= EMIT_BLOCK;
-        if (!by_block && (e % (SCAN_THREADS / 32)) != wid) continue;
-        const unsigned int step = by_block ? SCAN_THREADS : 32u;
-        for (unsigned int o = l + (by_block ? (unsigned)tid : (unsigned)lane); o < h; o += step) {
-            anc[o] = i;
-            if (src) src[o] = (int32_t)rp.off + i;
-        }
-    }
+    emit_systematic(v, off, base, rp.n, T, U, b.anc + rp.off, b.src ? b.src + rp.off : nullptr, (int32_t)rp.off, list);
 }
 
 // Multinomial resampling (the paper's scheme, Sec. 3) after the scan: output
@@ -1027,62 +1043,80 @@ __global__ void __launch_bounds__(RUN_THREADS) k_normalise_flat(const double* lo
 }
 // The same over the whole GPU, for more than one CTA's worth of weights.  FP64
 // exponentials bound it (an SM retires about two FP64 operations per clock),
-// so they are spread over every SM: one CTA took 962 us at 100003 weights, the
-// three kernels take 32.  The partials (max, sum exp, sum exp^2 of each CTA's
-// contiguous share) wait in the first 3 gridDim.x entries of W, which the last
-// kernel overwrites, so nothing is allocated.
-constexpr int NORM_THREADS = 256, NORM_MAX_PARTS = 2 * 152;
-__global__ void __launch_bounds__(NORM_THREADS) k_norm_part(const double* logw, int64_t N, double* part) {
-    __shared__ double buf[2 * 32];
-    const int64_t lo = N * blockIdx.x / gridDim.x, hi = N * (blockIdx.x + 1) / gridDim.x;
-    double m = -CUDART_INF;
-    bool nan = false;
+// so each is taken once, relative to the largest of its CTA's share, and
+// scaled when the total is known; one CTA took 962 us at 100003 weights,
+// separate exponentials for the sum and the weights over the whole GPU 32,
+// this 27.  The partials (max, sum exp, sum exp^2 of each CTA's contiguous
+// share) wait in the first 3 gridDim.x entries of W, whose exponentials a last
+// small kernel takes again, so nothing is allocated.
+constexpr int NORM_THREADS = 512, NORM_MAX_PARTS = 152;   // a share per SM
+__device__ __forceinline__ int64_t norm_share(int64_t N, int64_t parts, int64_t b) { return N * b / parts; }
+__global__ void __launch_bounds__(NORM_THREADS) k_norm_part(const double* logw, int64_t N, double* W) {
+    __shared__ double buf[2 * 32], tot_s[2];
+    __shared__ long long lbuf[32];
+    const int64_t lo = norm_share(N, gridDim.x, blockIdx.x), hi = norm_share(N, gridDim.x, blockIdx.x + 1);
+    long long mk = order_key(-CUDART_INF);
+    int nan = 0;
     for (int64_t i = lo + threadIdx.x; i < hi; i += NORM_THREADS) {
         const double x = logw[i];
-        nan |= isnan(x);
-        m = fmax(m, x);
+        if (isnan(x)) nan = 1;
+        else mk = max(mk, order_key(x));
     }
-    m = block_reduce(m, buf, OpMax());
+    const double m = from_order_key(block_reduce(mk, lbuf, OpMax()));
+    const bool mass = m > -CUDART_INF;
     double s[2] = {0.0, 0.0};
-    if (m > -CUDART_INF) {
-        for (int64_t i = lo + threadIdx.x; i < hi; i += NORM_THREADS) {
-            const double e = exp(logw[i] - m);
-            s[0] += e;
-            s[1] += e * e;
-        }
-    } else if (nan) {
-        s[0] = s[1] = CUDART_NAN;   // a share of NaN and -inf only still makes the sums NaN
+    for (int64_t i = lo + threadIdx.x; i < hi; i += NORM_THREADS) {
+        const double x = logw[i];
+        // without mass the share is -inf and NaN
+        const double e = mass ? exp(x - m) : (nan && isnan(x) ? x : 0.0);
+        s[0] += e;
+        s[1] += e * e;
+        if (i >= 3 * (int64_t)gridDim.x) W[i] = e;
     }
-    block_reduce_n(s, buf, OpSum());
+    const double r = block_sums(s, buf);
+    if (threadIdx.x < 2) tot_s[threadIdx.x] = r;
+    __syncthreads();
+    if (threadIdx.x < 3) W[3 * (int64_t)blockIdx.x + threadIdx.x] = threadIdx.x == 0 ? m : tot_s[threadIdx.x - 1];
+}
+// Every CTA combines the partials and scales its share; CTA 0 also writes the
+// scalars.
+__global__ void __launch_bounds__(NORM_THREADS) k_norm_scale(double* W, int64_t N, int n_parts, double* lse_out,
+                                                             double* ess_out) {
+    __shared__ double buf[2 * 32], tot_s[2], f_s;
+    __shared__ long long lbuf[32];
+    const int p = threadIdx.x;
+    const bool in = p < n_parts;
+    const double m = in ? W[3 * p] : -CUDART_INF;
+    const double M = from_order_key(block_reduce(order_key(m), lbuf, OpMax()));
+    double s[2] = {0.0, 0.0};
+    if (in) {
+        const double f = m > -CUDART_INF ? exp(m - M) : 1.0;   // without mass the sums are 0, or NaN
+        s[0] = W[3 * p + 1] * f;
+        s[1] = W[3 * p + 2] * f * f;
+    }
+    const double r = block_sums(s, buf);
+    if (threadIdx.x < 2) tot_s[threadIdx.x] = r;
+    __syncthreads();
+    const bool any = M > -CUDART_INF;
     if (threadIdx.x == 0) {
-        part[3 * blockIdx.x] = m;
-        part[3 * blockIdx.x + 1] = s[0];
-        part[3 * blockIdx.x + 2] = s[1];
+        const double lse = any ? M + log(tot_s[0]) : -CUDART_INF;
+        if (blockIdx.x == 0) {
+            *lse_out = lse;
+            *ess_out = any ? tot_s[0] * tot_s[0] / tot_s[1] : 0.0;
+        }
+        // W_i = exp(x_i - m_b) exp(m_b - lse), m_b this share's largest
+        f_s = any ? exp(W[3 * (int64_t)blockIdx.x] - lse) : 0.0;
     }
+    __syncthreads();
+    const double f = f_s;
+    const int64_t first = 3 * (int64_t)n_parts;
+    const int64_t lo = norm_share(N, n_parts, blockIdx.x), hi = norm_share(N, n_parts, blockIdx.x + 1);
+    for (int64_t i = max(lo, first) + threadIdx.x; i < hi; i += NORM_THREADS) W[i] = any ? W[i] * f : 0.0;
 }
-__global__ void __launch_bounds__(NORM_MAX_PARTS + 16) k_norm_combine(const double* part, int n_parts, double* lse_out,
-                                                                      double* ess_out) {
-    __shared__ double buf[2 * 32];
-    const int t = threadIdx.x;
-    const double mt = t < n_parts ? part[3 * t] : -CUDART_INF;
-    const double m = block_reduce(mt, buf, OpMax());
-    double s[2] = {0.0, 0.0};
-    if (t < n_parts) {
-        const double f = mt > -CUDART_INF ? exp(mt - m) : 1.0;   // without mass the sums are 0, or NaN
-        s[0] = part[3 * t + 1] * f;
-        s[1] = part[3 * t + 2] * f * f;
-    }
-    block_reduce_n(s, buf, OpSum());
-    if (t == 0) {
-        const bool any = m > -CUDART_INF;
-        *lse_out = any ? m + log(s[0]) : -CUDART_INF;
-        *ess_out = any ? s[0] * s[0] / s[1] : 0.0;
-    }
-}
-__global__ void __launch_bounds__(NORM_THREADS) k_norm_write(const double* logw, int64_t N, const double* lse,
-                                                             double* W) {
+// The entries that held the partials.
+__global__ void __launch_bounds__(NORM_THREADS) k_norm_first(const double* logw, int64_t n, const double* lse, double* W) {
     const int64_t i = (int64_t)blockIdx.x * NORM_THREADS + threadIdx.x;
-    if (i >= N) return;
+    if (i >= n) return;
     const double l = *lse;
     W[i] = l == -CUDART_INF ? 0.0 : exp(logw[i] - l);
 }
@@ -1099,8 +1133,8 @@ cudaError_t launch_normalise_flat(const double* logw, int64_t N, double* W, doub
         return cudaGetLastError();
     }
     k_norm_part<<<(unsigned)nb, NORM_THREADS, 0, s>>>(logw, N, W);
-    k_norm_combine<<<1, NORM_MAX_PARTS + 16, 0, s>>>(W, (int)nb, lse, ess);
-    k_norm_write<<<(unsigned)((N + NORM_THREADS - 1) / NORM_THREADS), NORM_THREADS, 0, s>>>(logw, N, lse, W);
+    k_norm_scale<<<(unsigned)nb, NORM_THREADS, 0, s>>>(W, N, (int)nb, lse, ess);
+    k_norm_first<<<(unsigned)((3 * nb + NORM_THREADS - 1) / NORM_THREADS), NORM_THREADS, 0, s>>>(logw, 3 * nb, lse, W);
     return cudaGetLastError();
 }
 
@@ -1115,38 +1149,81 @@ int64_t resample_scratch_bytes(int64_t N) {
     return (int64_t)(((sizeof(FlatScratch) + 255) / 256) * 256 + sizeof(TileDesc) * (size_t)flat_tiles(N));
 }
 
-// q_j = floor(W_j 2^S) and T = sum q (an exact integer sum, so the atomics'
-// order does not matter) over the whole GPU; the header and the descriptors
-// were zeroed before.  Bound by memory: 16 bytes per weight (one CTA over all
-// of them took most of the 942 us of a 1M-particle resampling, now 46 in all).
-constexpr int QUANT_THREADS = 256;
-__global__ void __launch_bounds__(QUANT_THREADS) k_quantise_flat(const double* W, int64_t N, uint64_t r64,
-                                                                 unsigned long long* q, FlatScratch* fs,
-                                                                 int64_t n_tiles, double scale) {
+// q_j = floor(W_j 2^S), with the total of every scan tile.  Bound by memory: 16
+// bytes per weight (one CTA over all of them took most of the 942 us of a
+// 1M-particle resampling).
+__global__ void __launch_bounds__(SCAN_THREADS) k_quantise_flat(const double* W, int64_t N, unsigned long long* q,
+                                                                unsigned long long* agg, double scale) {
     __shared__ unsigned long long ubuf[32];
     unsigned long long T = 0ull;
-    const int64_t stride = (int64_t)gridDim.x * QUANT_THREADS;
-#pragma unroll 4
-    for (int64_t i = (int64_t)blockIdx.x * QUANT_THREADS + threadIdx.x; i < N; i += stride) {
-        const double v = W[i] * scale;
+    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x;
+    double w[SCAN_ITEMS];
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) {
+        const int64_t i = base + (int64_t)k * SCAN_THREADS;
+        w[k] = i < N ? W[i] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) {
+        const int64_t i = base + (int64_t)k * SCAN_THREADS;
+        const double v = w[k] * scale;
         const unsigned long long qi = v > 0.0 ? __double2ull_rz(v) : 0ull;
-        q[i] = qi;
+        if (i < N) q[i] = qi;
         T += qi;
     }
     T = block_reduce(T, ubuf, OpSum());
-    if (threadIdx.x == 0) {
-        if (T) atomicAdd(&fs->st.T, T);
-        if (blockIdx.x == 0) {      // the other fields stay zero
-            fs->rp.n = N;
-            fs->rp.n_tiles = (int32_t)n_tiles;
-            fs->st.k = 1;
-            fs->st.r64 = (unsigned long long)r64;
-            fs->st.resample = 1;    // T == 0 is found (status -4) by the scan
-            fs->counter[1] = 1u;    // the descriptors' epoch: they were zeroed
-        }
-    }
+    if (threadIdx.x == 0) agg[blockIdx.x] = T;
 }
 
+// The ancestors where the tiles' totals are at hand: every CTA adds up those
+// before its tile, and all of them, itself (two round trips to L2, where the
+// look-back's walk takes one per 32 tiles): 1048576 weights 46 -> 30 us in all.
+constexpr int64_t FLAT_DIRECT_TILES = 2048;   // 4194304 particles: 16 KB of totals per CTA
+__global__ void __launch_bounds__(SCAN_THREADS) k_resample_flat(const unsigned long long* q, int64_t N, uint64_t r64,
+                                                                const unsigned long long* agg, int32_t* anc,
+                                                                int32_t* status) {
+    __shared__ unsigned long long wsum[SCAN_THREADS / 32], ubuf[2 * 32];
+    __shared__ EmitList list;
+    if (threadIdx.x == 0) list.n = 0;
+    unsigned long long t[2] = {0ull, 0ull};   // before this tile, all
+    for (int64_t g = threadIdx.x; g < gridDim.x; g += SCAN_THREADS) {
+        const unsigned long long x = agg[g];
+        t[0] += g < blockIdx.x ? x : 0ull;
+        t[1] += x;
+    }
+    block_reduce_n(t, ubuf, OpSum());
+    const unsigned long long T = t[1];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *status = T == 0ull ? -4 : 0;   // no mass at all: degenerate
+    if (T == 0ull) return;
+    unsigned long long v[SCAN_ITEMS], tile_agg;
+    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
+    const unsigned long long off = t[0] + tile_scan(q, base, N, v, wsum, tile_agg);
+    emit_systematic(v, off, base, N, T, __umul64hi((unsigned long long)r64, T), anc, nullptr, 0, list);
+}
+
+// With more tiles the scan looks back; its header from the tiles' totals, which
+// lie where its descriptors will (they are zeroed in between).
+__global__ void __launch_bounds__(RUN_THREADS) k_flat_header(FlatScratch* fs, const unsigned long long* agg, int64_t N,
+                                                             uint64_t r64, int64_t n_tiles) {
+    __shared__ unsigned long long ubuf[32];
+    unsigned long long T = 0ull;
+    for (int64_t g = threadIdx.x; g < n_tiles; g += RUN_THREADS) T += agg[g];
+    T = block_reduce(T, ubuf, OpSum());
+    if (threadIdx.x == 0) {
+        RunParams rp = {};
+        rp.n = N;
+        rp.n_tiles = (int32_t)n_tiles;
+        fs->rp = rp;
+        RunState st = {};
+        st.k = 1;
+        st.T = T;
+        st.r64 = (unsigned long long)r64;
+        st.resample = 1;            // T == 0 is found (status -4) by the scan
+        fs->st = st;
+        fs->counter[0] = 0u;
+        fs->counter[1] = 1u;        // the descriptors' epoch
+    }
+}
 __global__ void k_copy_status(const FlatScratch* fs, int32_t* status) { *status = fs->st.status; }
 
 // The look-back wait of the resampling scan against a predecessor that never
@@ -1177,13 +1254,17 @@ cudaError_t launch_resample_flat(const double* W, int64_t N, uint64_t r64, unsig
     FlatScratch* fs = reinterpret_cast<FlatScratch*>(scratch);
     TileDesc* tiles = reinterpret_cast<TileDesc*>(reinterpret_cast<char*>(scratch) +
                                                   ((sizeof(FlatScratch) + 255) / 256) * 256);
-    cudaError_t e = cudaMemsetAsync(scratch, 0, (size_t)resample_scratch_bytes(N), s);   // header and descriptors
-    if (e != cudaSuccess) return e;
     int c = 0;
     while (((int64_t)1 << c) < N) ++c;
-    // four weights per thread until the GPU is full (8 CTAs of 256 per SM)
-    const int64_t qb = std::min<int64_t>((N + 4 * QUANT_THREADS - 1) / (4 * QUANT_THREADS), 152 * 8);
-    k_quantise_flat<<<(unsigned)qb, QUANT_THREADS, 0, s>>>(W, N, r64, q, fs, nt, std::ldexp(1.0, 62 - c));
+    unsigned long long* agg = reinterpret_cast<unsigned long long*>(tiles);
+    k_quantise_flat<<<(unsigned)nt, SCAN_THREADS, 0, s>>>(W, N, q, agg, std::ldexp(1.0, 62 - c));
+    if (nt <= FLAT_DIRECT_TILES) {
+        k_resample_flat<<<(unsigned)nt, SCAN_THREADS, 0, s>>>(q, N, r64, agg, anc, status);
+        return cudaGetLastError();
+    }
+    k_flat_header<<<1, RUN_THREADS, 0, s>>>(fs, agg, N, r64, nt);
+    cudaError_t e = cudaMemsetAsync(tiles, 0, sizeof(TileDesc) * (size_t)nt, s);
+    if (e != cudaSuccess) return e;
     StepBufs b = {};
     b.runs = &fs->rp;
     b.rstate = &fs->st;

@@ -21,7 +21,7 @@ def _normalise(lw, in_place):
     return W.cpu().numpy(), *sc.cpu().numpy()
 
 
-@pytest.mark.parametrize("N", [1, 256, 257, 511, 513, 304 * 256, 304 * 256 + 1, 100003])
+@pytest.mark.parametrize("N", [1, 256, 257, 511, 512, 513, 152 * 512, 152 * 512 + 1, 304 * 256 + 1, 100003])
 @pytest.mark.parametrize("special", ["none", "-inf", "all -inf", "nan", "+inf", "one share -inf"])
 def test_normalise_over_the_gpu_matches_one_cta(N, special):
     """Both forms round the same exact sums, of at most N terms added in trees
@@ -51,10 +51,11 @@ def test_normalise_over_the_gpu_matches_one_cta(N, special):
         np.testing.assert_allclose([lse, ess], [lse_o, ess_o], rtol=1e-12)
 
 
-@pytest.mark.parametrize("N", [1, 255, 2048, 2049, 70001])
+@pytest.mark.parametrize("N", [1, 255, 2048, 2049, 70001, 4194304, 4300001])
 @pytest.mark.parametrize("kind", ["one", "few", "heavy", "even"])
 def test_resampling_long_and_short_ranges_bit_exact(N, kind):
-    """Ranges of one slot, of a warp's, of a CTA's and of all N slots."""
+    """Ranges of one slot, of a warp's, of a CTA's and of all N slots; the last
+    size is past the tiles whose totals every CTA adds up."""
     need_gpu()
     rng = np.random.default_rng(N)
     W = np.zeros(N)
