@@ -978,7 +978,7 @@ smc_status smc_step(smc_handle* h, smc_stats* stats) {
             cudaEventRecord(h->events[i + 1], s);
             h->n_event_pairs += 1;
             // + the centred form's reference kernels, and its run partition with several runs
-            h->kernel_launches += KERNELS_PER_ITERATION +
+            h->kernel_launches += kernels_per_iteration(b) +
                                   (h->precision == SMC_PREC_BF16C ? (h->n_runs > 1 ? 6 : 3) : 0);
         } else {
             e = h->flow_on ? launch_traj_flow(h->model.m, h->flow, a, h->z0, h->z1, s)

@@ -535,6 +535,66 @@ __global__ void k_sort_scatter(StepBufs b) {
     b.perm[slot] = (int32_t)j;
 }
 
+// Resampling and order of one run that fits a scan tile, in one CTA instead of
+// three kernels of one CTA each (11 us one after the other, now 5): the
+// tile's prefix needs no look-back, and the step histogram is scanned and its
+// slots taken in shared memory.
+constexpr int SMALL_BINS = 4096;
+static bool small_order(const StepBufs& b) { return b.n_runs == 1 && b.n_tiles == 1 && b.max_steps_all < SMALL_BINS; }
+__global__ void __launch_bounds__(SCAN_THREADS) k_resample_order_small(StepBufs b) {
+    __shared__ unsigned long long wsum[SCAN_THREADS / 32];
+    __shared__ EmitList list;
+    __shared__ int slot[SMALL_BINS], wcnt[SCAN_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (tid == 0) list.n = 0;
+    // the first slot of each step count, longest first
+    const int nb = b.max_steps_all + 1, per = (nb + SCAN_THREADS - 1) / SCAN_THREADS;
+    int cnt = 0;
+    for (int i = tid; i < nb; i += SCAN_THREADS) slot[i] = b.hist[i];
+    __syncthreads();
+    for (int i = tid * per; i < min(nb, (tid + 1) * per); ++i) cnt += slot[i];
+    int x = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wcnt[wid] = x;
+    __syncthreads();
+    int first = x - cnt;
+    for (int w = 0; w < wid; ++w) first += wcnt[w];
+    for (int i = tid * per; i < min(nb, (tid + 1) * per); ++i) {
+        const int c = slot[i];
+        slot[i] = first;
+        first += c;
+    }
+    __syncthreads();
+    const int n = (int)b.N;
+    for (int j = tid; j < n; j += SCAN_THREADS) b.perm[warp_agg_inc(slot, b.max_steps_all - b.steps[j])] = j;
+
+    RunState& st = b.rstate[0];
+    const RunParams& rp = b.runs[0];
+    if (!st.resample || st.status != 0) {
+        for (int j = tid; j < n; j += SCAN_THREADS) b.src[j] = j;
+        return;
+    }
+    const unsigned long long T = st.T;
+    __syncthreads();                 // everyone has read the status
+    if (T == 0ull) {                 // no mass at all: degenerate
+        if (tid == 0) st.status = -4;
+        return;
+    }
+    unsigned long long v[SCAN_ITEMS], tile_agg;
+    const unsigned long long off = tile_scan(b.q, 0, n, v, wsum, tile_agg);
+    if (rp.resample_scheme == 1) {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k)
+            if (tid * SCAN_ITEMS + k < n) b.cprefix[tid * SCAN_ITEMS + k] = off + v[k];
+        return;
+    }
+    emit_systematic(v, off, 0, n, T, __umul64hi(st.r64, T), b.anc, b.src, 0, list);
+}
+
 // ============================================================ move statistics
 // Per particle slice (first pass): with the momentum change-of-variable
 // L-kernel the Jacobians cancel and log w += -Delta H (Sec. 3.1); pieces of
@@ -932,11 +992,14 @@ cudaError_t launch_weights_steps(const StepBufs& b, cudaStream_t s) {
     return cudaGetLastError();
 }
 cudaError_t launch_resample_scan(const StepBufs& b, cudaStream_t s) {
-    k_resample_scan<<<(unsigned)b.n_tiles, SCAN_THREADS, 0, s>>>(b);
+    if (small_order(b)) k_resample_order_small<<<1, SCAN_THREADS, 0, s>>>(b);
+    else k_resample_scan<<<(unsigned)b.n_tiles, SCAN_THREADS, 0, s>>>(b);
     if (b.any_multinomial && b.N > 0) k_multinomial_search<<<(unsigned)((b.N + 255) / 256), 256, 0, s>>>(b);
     return cudaGetLastError();
 }
+int kernels_per_iteration(const StepBufs& b) { return small_order(b) ? 5 : 7; }
 cudaError_t launch_sort(const StepBufs& b, cudaStream_t s) {
+    if (small_order(b)) return cudaSuccess;   // with the resampling
     const int bs = 256;
     k_hist_scan<<<1, 1024, 0, s>>>(b);
     k_sort_scatter<<<(unsigned)((b.N + bs - 1) / bs), bs, 0, s>>>(b);

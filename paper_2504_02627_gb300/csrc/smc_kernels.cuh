@@ -83,7 +83,7 @@ cudaError_t launch_resample_scan(const StepBufs& b, cudaStream_t s);
 cudaError_t launch_lookback_wait_check(long long limit, TileDesc* tiles, int* status, cudaStream_t s);
 cudaError_t launch_sort(const StepBufs& b, cudaStream_t s);
 cudaError_t launch_move_stats(const StepBufs& b, cudaStream_t s);
-constexpr int KERNELS_PER_ITERATION = 7;   // kernels launched by one smc_step
+int kernels_per_iteration(const StepBufs& b);   // launched by one smc_step, the trajectories among them
 constexpr int MAX_CHEES_DIM = 256;         // D handled by the fused ChEES statistics
 
 // Kernel-level entry points (stand-alone buffers).
