@@ -713,29 +713,28 @@ __global__ void __launch_bounds__(SLICE) k_move_stats(StepBufs b) {
                     a1[h][u] = in ? t1[o + jj[u]] : 0.0f;
                 }
             }
+            f2sum v[4];                                  // FP32 pairs (about 48 bits): d before, after, d2 before, after
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int dd = h ? d2 : d;
-                f2sum v0{0.0f, 0.0f}, v1{0.0f, 0.0f};    // FP32 pairs (about 48 bits)
+                f2sum v0{0.0f, 0.0f}, v1{0.0f, 0.0f};
 #pragma unroll
                 for (int u = 0; u < PL; ++u) {
                     if (jj[u] < 0) continue;
                     v0 = f2_add_f(v0, a0[h][u]);
                     v1 = f2_add_f(v1, a1[h][u]);
                 }
-                v0 = warp_sum_f2(v0);
-                v1 = warp_sum_f2(v1);
-                if (lane == 0 && dd < D) {
-                    b.colsum[(int64_t)c * 2 * D + dd] = f2_to_double(v0);
-                    b.colsum[(int64_t)c * 2 * D + D + dd] = f2_to_double(v1);
-                }
+                v[2 * h] = v0;
+                v[2 * h + 1] = v1;
             }
+            const f2sum t = warp_sum4_f2(v, lane);
+            const int w = lane >> 3, dd = (w & 2) ? d2 : d;
+            if ((lane & 7) == 0 && dd < D) b.colsum[(int64_t)c * 2 * D + ((w & 1) ? D : 0) + dd] = f2_to_double(t);
         }
     }
 }
 
 // Bound by FP64 (an exponential is some 25 instructions) and by the pair sums
-// over the dimensions: 64 hierarchical runs, 278k particles, 129 -> 83 us; one
+// over the dimensions: 64 hierarchical runs, 278k particles, 129 -> 60 us; one
 // run of 256 particles 13 -> 8 us.
 //
 // Second pass: ChEES gradient estimates g_j = l_j (|t1_j - mean t1|^2 -
@@ -744,7 +743,7 @@ __global__ void __launch_bounds__(SLICE) k_move_stats(StepBufs b) {
 // evidence, log-weights' ESS, Adam ascent on log L, Lbar, the freeze at
 // M_warmup, statistics, and the weight decision of the next iteration.  One run of
 // 256 particles: 34 -> 13 us, nearly all of it the FP64 latency of the last
-// slice's chain.
+// slice's chain; 64 hierarchical runs: 115 -> 88 us, the pair arithmetic.
 __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
     __shared__ double buf[7 * 32], tot_s[7], res_s[4];
     __shared__ long long lbuf[2 * 32];
@@ -805,9 +804,9 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
                     if (d >= D) break;
                     const f2sum e0 = f2_add_f(f2sum{mean_s[d], mean_s[2 * D + d]}, v0[u]);
                     const f2sum e1 = f2_add_f(f2sum{mean_s[D + d], mean_s[3 * D + d]}, v1[u]);
-                    sq0 = f2_add(sq0, f2_mul(e0, e0));
-                    sq1 = f2_add(sq1, f2_mul(e1, e1));
-                    proj = f2_add(proj, f2_mul(e1, f2sum{vp[u], 0.0f}));
+                    f2_dot(sq0, e0, e0);
+                    f2_dot(sq1, e1, e1);
+                    f2_dot(proj, e1, f2sum{vp[u], 0.0f});
                 }
             }
             const double h = jitter_h(rp.jitter, rp.seed, x.i, st.k, rp.n, rp.n_iters, b.primes);
