@@ -279,6 +279,11 @@ __device__ __forceinline__ double from_order_key(long long k) {
     return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
 }
 
+// log(1 + e^x) = max(x, 0) + log(1 + e^-|x|): one exponential and one logarithm
+// for either sign (the two-sided form as a branch runs both sides in a warp;
+// the value is the same bit for bit).
+__device__ __forceinline__ float softplus(float x) { return (x > 0.0f ? x : 0.0f) + log1pf(expf(-fabsf(x))); }
+
 // ---------------------------------------------------------------- FP32 pairs
 // An unevaluated pair hi + lo of FP32 values carries about 48 significant
 // bits.  Sums use Knuth's TwoSum and products the FMA form of Dekker's

@@ -977,9 +977,9 @@ smc_status smc_step(smc_handle* h, smc_stats* stats) {
                            : launch_traj(h->model.m, a, h->precision, s);
             cudaEventRecord(h->events[i + 1], s);
             h->n_event_pairs += 1;
-            // + the centred form's reference kernels, and its run partition with several runs
+            // + the centred form's reference kernels and end-point energies, and its run partition with several runs
             h->kernel_launches += kernels_per_iteration(b) +
-                                  (h->precision == SMC_PREC_BF16C ? (h->n_runs > 1 ? 6 : 3) : 0);
+                                  (h->precision == SMC_PREC_BF16C ? (h->n_runs > 1 ? 7 : 4) : 0);
         } else {
             e = h->flow_on ? launch_traj_flow(h->model.m, h->flow, a, h->z0, h->z1, s)
                            : launch_traj(h->model.m, a, h->precision, s);

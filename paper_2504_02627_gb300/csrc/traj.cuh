@@ -195,6 +195,9 @@ bool traj_stream_supported(const DevModel& m);
 cudaError_t launch_traj_stream(const DevModel& m, const TrajArgs& a, int np, cudaStream_t s);
 // centred tensor-core path (traj_centred.cu): any n, D <= 128, precision 4;
 // the caller provides the TrajArgs::c_* arrays (sizes below)
+// end-point energies of the regressions (traj_energy.cu): log pi, and from H_0 in
+// dH, Delta H and alpha, for kernels that leave them out
+cudaError_t launch_regression_energy(const DevModel& m, const TrajArgs& a, cudaStream_t s);
 bool traj_centred_supported(const DevModel& m);
 int64_t centred_refs_elems(const DevModel& m, int n_runs);
 int64_t centred_part_elems(const DevModel& m, int n_runs);

@@ -22,7 +22,8 @@
 // reference rather than reusing the cached one), so each trajectory is a
 // volume-preserving, reversible composition of shears; the end-point energy
 // that enters the importance weight is recomputed with the FP32 data and
-// FP64 accumulation, as in every other kernel.
+// FP64 accumulation, as in every other path, by a launch of its own
+// (traj_energy.cu), for which this kernel leaves H_0 in dH.
 //
 // Layout.  One CTA holds 128 particles (MMA M = 128).  X streams through a
 // ring of up to four stages (as many as fit in shared memory next to the
@@ -87,17 +88,14 @@ constexpr int C_SMEM_MAX = 232448;
 constexpr float C_X_MAX = 60.0f;           // clamp of the exponent: two factors 1 + 2^x multiply without overflow
 
 struct CLayout {
-    int atoms, tile_bytes, ref_bytes, stage_bytes, stages, xbufs;
-    int off_d, off_stage, off_gx, off_emisc, off_cref, off_bar, off_state, total;
+    int atoms, tile_bytes, ref_bytes, stage_bytes, stages;
+    int off_d, off_stage, off_gx, off_cref, off_bar, off_state, total;
 };
 
 // Byte layout of the dynamic shared memory (from a 1024-aligned base) with
-// `stages` X tile stages.  The end-point pass reuses [0, off_cref), the
-// pipeline's memory, for theta^T, two FP32 X chunks, the partial sums and
-// its kinetic / prior / likelihood parts, so off_cref covers both uses.
-__host__ __device__ inline CLayout c_layout_n(int dk, int Dp, int n_ref, int n_run, int stages, int xbufs) {
+// `stages` X tile stages.
+__host__ __device__ inline CLayout c_layout_n(int dk, int n_ref, int n_run, int stages) {
     CLayout L;
-    L.xbufs = xbufs;
     L.atoms = (dk + 63) / 64;
     L.tile_bytes = L.atoms * C_ATOM;
     L.ref_bytes = n_ref * CC * 8;                         // (c, s) pairs per run, a multiple of 1024
@@ -106,15 +104,9 @@ __host__ __device__ inline CLayout c_layout_n(int dk, int Dp, int n_ref, int n_r
     L.off_d = 0;
     L.off_stage = L.atoms * C_DATOM;
     L.off_gx = L.off_stage + stages * L.stage_bytes;     // [dk][128] f32 partial gradient of this CTA
-    const int pipe = L.off_gx + dk * CP * 4;
-    // the end point reuses the pipeline's memory: theta^T, one or two FP32
-    // X chunks of CC observations and per-warp parts, then its kin, sq:
-    // [4][128] f64 and ll: [128] f64 (the prologue keeps its kinetic parts in
-    // the first stage, idle until the copies start)
-    const int endp = dk * CP * 4 + xbufs * CC * Dp * 4 + C_EPI_WARPS * CP * 8;
-    L.off_emisc = (endp + 1023) & ~1023;
-    const int endx = L.off_emisc + 9 * CP * 8;
-    L.off_cref = ((pipe > endx ? pipe : endx) + 1023) & ~1023;
+    // (the prologue keeps its kinetic parts in the first stage, idle until the
+    // copies start)
+    L.off_cref = (L.off_gx + dk * CP * 4 + 1023) & ~1023;
     L.off_bar = L.off_cref + 2 * n_run * dk * 4;          // reference points, reference gradients [runs][dk]
     L.off_state = 0;
     L.total = L.off_bar + 256 + 1024;                     // + alignment slack of the base
@@ -123,16 +115,14 @@ __host__ __device__ inline CLayout c_layout_n(int dk, int Dp, int n_ref, int n_r
     if (L.total < 118 * 1024) L.total = 118 * 1024;
     return L;
 }
-// The most X stages that fit (4, 3 or 2) with a double-buffered end point,
-// else two stages with a single end-point buffer.  A CTA that is not part of a
+// The most X stages that fit (4, 3 or 2).  A CTA that is not part of a
 // cluster also keeps the move's theta and p there ([dk][128] each) when they
 // fit next to the stages: the update at a pass's end then waits for no L2
 // round trip (ten runs of 4096 particles, n = 1000, D = 25: a move of about
 // 375 steps 9.80 -> 9.48 ms).
-__host__ __device__ inline CLayout c_layout(int dk, int Dp, int n_ref, int n_run, bool alone) {
-    CLayout L = c_layout_n(dk, Dp, n_ref, n_run, C_NS_MAX, 2);
-    for (int st = C_NS_MAX - 1; st >= 2 && L.total > C_SMEM_MAX; --st) L = c_layout_n(dk, Dp, n_ref, n_run, st, 2);
-    if (L.total > C_SMEM_MAX) L = c_layout_n(dk, Dp, n_ref, n_run, 2, 1);
+__host__ __device__ inline CLayout c_layout(int dk, int n_ref, int n_run, bool alone) {
+    CLayout L = c_layout_n(dk, n_ref, n_run, C_NS_MAX);
+    for (int st = C_NS_MAX - 1; st >= 2 && L.total > C_SMEM_MAX; --st) L = c_layout_n(dk, n_ref, n_run, st);
     const int state = L.off_bar + 256;
     if (alone && state + 2 * dk * CP * 4 + 1024 <= C_SMEM_MAX) {
         L.off_state = state;
@@ -157,7 +147,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
     // 1024-aligned base by pointer arithmetic on the shared array, so that
     // accesses through it stay shared-space loads and stores
     unsigned char* sm = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
-    const CLayout L = c_layout(m.dk, m.Dp, LOGIT ? 1 : 0, a.c_runs, a.c_split == 1);
+    const CLayout L = c_layout(m.dk, LOGIT ? 1 : 0, a.c_runs, a.c_split == 1);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int D = m.D, dk = m.dk, nch_all = m.n_tiles128;
     const int64_t ld = a.ld;
@@ -193,9 +183,6 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
     int* smax_s = reinterpret_cast<int*>(tmem_s + 1);
     volatile int* abort_s = smax_s + 1;
     double* kin0_s = reinterpret_cast<double*>(sm + L.off_stage);    // prologue: [4][128] |p_0|^2 parts
-    double* kin_s = reinterpret_cast<double*>(sm + L.off_emisc);     // end point: [4][128] |p|^2 parts
-    double* sq_s = kin_s + 4 * CP;                                   // [4][128] |theta|^2 parts
-    double* ll_s = sq_s + 4 * CP;                                    // [128] log-likelihood
     const uint32_t s_base = tc::smem_u32(sm);
     float* gx = reinterpret_cast<float*>(sm + L.off_gx);             // [dk][128] this CTA's partial gradient
     const uint32_t gx_base = s_base + (uint32_t)L.off_gx, dev_base = s_base + (uint32_t)L.off_d;
@@ -248,9 +235,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
     const int ds = 32 * q;                             // first state dimension of this thread
     const int bq = q >> 1, half = q & 1;
     const float inv_tau2 = LOGIT ? (float)(1.0 / (m.h0 * m.h0)) : (float)(1.0 / (m.h1 * m.h1));
-    const double inv_tau2_d = LOGIT ? 1.0 / (m.h0 * m.h0) : 1.0 / (m.h1 * m.h1);
     const float inv_s2 = LOGIT ? 0.0f : (float)(1.0 / (m.h0 * m.h0));
-    const float inv_s = LOGIT ? 0.0f : (float)(1.0 / m.h0);
     const bool evalm = a.eval_only != 0;
     // the state is kept by slot: in shared memory, else in c_sth / c_sp
     const bool smst = L.off_state > 0 && !evalm;
@@ -347,10 +332,10 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
     tc::fence_after_sync();
     if (epi && S > 0) atomicMax(smax_s, S);
     tc::cluster_sync();   // barriers of every CTA of the cluster initialised before any remote arrive
-    double H0 = 0.0;
-    if (epi && q == 0 && j >= 0 && !evalm)
-        H0 = 0.5 * (kin0_s[prow] + kin0_s[CP + prow] + kin0_s[2 * CP + prow] + kin0_s[3 * CP + prow]) -
-             a.logpi_in[src];
+    // H_0, for the end-point energies' launch
+    if (rank == 0 && epi && q == 0 && j >= 0 && !evalm && a.dH)
+        a.dH[j] = 0.5 * (kin0_s[prow] + kin0_s[CP + prow] + kin0_s[2 * CP + prow] + kin0_s[3 * CP + prow]) -
+                  a.logpi_in[src];
     __syncthreads();
     const uint32_t tmem = *tmem_s;
     const int smax = *smax_s;
@@ -699,159 +684,21 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
         }
     }
 
-    // ---------------------------------------------------------------- end point energy
-    // eta = X theta in FP32 from the FP32 data (register tile of 4
-    // observations x 4 particles per thread, X chunks double-buffered in
-    // shared memory by cp.async), a thread's four terms of a particle summed in
-    // FP32, then FP64 accumulation of the log-likelihood.
+    // ---------------------------------------------------------------- final state
     if (tid == 0) {
         volatile int ignore_abort = 0;   // these drain waits run even after an abort
         tc::mbar_wait_timed(fin1, 0u, err, &ignore_abort, 4000000000ull);
         tc::mbar_wait_timed(fin2, 0u, err, &ignore_abort, 4000000000ull);
     }
-    __syncthreads();
-    tc::cluster_sync();   // every CTA of the cluster has written its units of the final state
-    const int Dp = m.Dp, n = m.n;
-    // this CTA's share of the CC-observation chunks of the end point (the
-    // same split as its X tiles)
-    const int e_lo = c_lo, e_hi = c_hi;
-    const int XB = L.xbufs;
-    float* thT = reinterpret_cast<float*>(sm);                  // [dk][128]
-    float* xs = thT + dk * CP;                                  // [XB][CC][Dp]
-    double* llp = reinterpret_cast<double*>(xs + XB * CC * Dp);   // [16][128]
-    if (epi) {
-        double sq = 0.0, kin = 0.0;
+    __syncthreads();   // every warp of the CTA has written its units
+    // from the slots to the particle's outputs, by the CTA that owns the unit
+    if (epi && slotst && j >= 0) {
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
             const int d = ds + e;
-            float tvv = 0.0f;
-            if (j >= 0 && d < D) {
-                tvv = evalm ? a.theta_in[(int64_t)d * ld + src] : thb[(int64_t)d * sld + si];
-                if (!evalm) {
-                    const float pvf = pb[(int64_t)d * sld + si];
-                    const double pv = pvf;
-                    kin += pv * pv;
-                    // the final state from the slot-ordered buffers to the
-                    // particle's outputs, by the CTA that owns the unit
-                    if (slotst && (d >> 3) >= u_lo && (d >> 3) < u_hi) {
-                        a.theta_out[(int64_t)d * ld + j] = tvv;
-                        a.p_out[(int64_t)d * ld + j] = pvf;
-                    }
-                }
-            }
-            if (d < dk) thT[d * CP + prow] = tvv;
-            sq += (double)tvv * (double)tvv;
-        }
-        sq_s[q * CP + prow] = sq;
-        kin_s[q * CP + prow] = kin;
-    }
-    auto issue_x = [&](int c, int buf) {
-        const int64_t row0 = (int64_t)c * CC;
-        const int64_t left = (int64_t)n - row0;
-        const int rows = left < CC ? (int)left : CC;
-        const int nvec = rows * Dp / 4;
-        float* dst = xs + buf * CC * Dp;
-        const float* srcx = m.X + row0 * Dp;
-        for (int v = tid; v < nvec; v += C_THREADS) tc::cp_async16(dst + 4 * v, srcx + 4 * v);
-        tc::cp_async_commit();
-    };
-    if (e_lo < e_hi) issue_x(e_lo, 0);
-    {
-        // warps 0-15 compute 8 observations each for 4 particles per lane
-        // (a register tile of 8 x 4: every theta^T load serves 8
-        // observations), warps 16-18 only copy
-        const int pg = lane, og = wid;
-        double ll[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int c = e_lo; c < e_hi; ++c) {
-            const int buf = (c - e_lo) % XB;
-            if (XB == 2) {
-                if (c + 1 < e_hi) issue_x(c + 1, buf ^ 1);
-                else tc::cp_async_commit();
-                tc::cp_async_wait<1>();
-            } else {
-                tc::cp_async_wait<0>();
-            }
-            __syncthreads();
-            if (og < C_EPI_WARPS) {
-                const float* xc = xs + buf * CC * Dp + og * 8 * Dp;
-                float acc[8][4];
-#pragma unroll
-                for (int o = 0; o < 8; ++o)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[o][k] = 0.0f;
-                // four dimensions per iteration: X rows as float4 (Dp is a
-                // multiple of 4 and zero-padded; theta^T rows past D are zero)
-                const float* tcol = thT + 4 * pg;
-                for (int d = 0; d < Dp; d += 4) {
-                    float4 xv[8];
-#pragma unroll
-                    for (int o = 0; o < 8; ++o) xv[o] = *reinterpret_cast<const float4*>(xc + o * Dp + d);
-#pragma unroll
-                    for (int dd = 0; dd < 4; ++dd) {
-                        const float4 t4 = *reinterpret_cast<const float4*>(tcol + (d + dd) * CP);
-#pragma unroll
-                        for (int o = 0; o < 8; ++o) {
-                            const float x = dd == 0 ? xv[o].x : dd == 1 ? xv[o].y : dd == 2 ? xv[o].z : xv[o].w;
-                            acc[o][0] = fmaf(x, t4.x, acc[o][0]);
-                            acc[o][1] = fmaf(x, t4.y, acc[o][1]);
-                            acc[o][2] = fmaf(x, t4.z, acc[o][2]);
-                            acc[o][3] = fmaf(x, t4.w, acc[o][3]);
-                        }
-                    }
-                }
-                float part[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-                for (int o = 0; o < 8; ++o) {
-                    const int64_t i = (int64_t)c * CC + og * 8 + o;
-                    if (i < n) {
-                        const float yv = __ldg(m.y + i);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const float eta = acc[o][k];
-                            float term;
-                            if (LOGIT) {
-                                const float sp = eta > 0.0f ? eta + log1pf(expf(-eta)) : log1pf(expf(eta));
-                                term = yv * eta - sp;
-                            } else {
-                                const float z = (yv - eta) * inv_s;
-                                term = -0.5f * z * z;
-                            }
-                            part[k] += term;
-                        }
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) ll[k] += (double)part[k];
-            }
-            __syncthreads();
-            if (XB == 1 && c + 1 < e_hi) issue_x(c + 1, 0);
-        }
-        if (og < C_EPI_WARPS)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) llp[og * CP + 4 * pg + k] = ll[k];
-        __syncthreads();
-        if (tid < CP) {
-            double tot = 0.0;
-            for (int w = 0; w < C_EPI_WARPS; ++w) tot += llp[w * CP + tid];   // fixed order
-            ll_s[tid] = tot;
-        }
-    }
-    __syncthreads();
-    tc::cluster_sync();   // every CTA's log-likelihood part is in its shared memory
-    if (rank == 0 && epi && q == 0 && j >= 0) {
-        // the cluster's parts, summed in rank order
-        const uint32_t la = tc::smem_u32(ll_s + prow);
-        double llsum = tc::ld_cluster_f64(tc::map_to_rank(la, 0u));
-        for (int r = 1; r < kc; ++r) llsum += tc::ld_cluster_f64(tc::map_to_rank(la, (uint32_t)r));
-        const double sq = sq_s[prow] + sq_s[CP + prow] + sq_s[2 * CP + prow] + sq_s[3 * CP + prow];
-        const double lp1 = llsum - 0.5 * sq * inv_tau2_d + m.lconst;
-        a.logpi_out[j] = lp1;
-        if (!evalm) {
-            const double kin = kin_s[prow] + kin_s[CP + prow] + kin_s[2 * CP + prow] + kin_s[3 * CP + prow];
-            double dH = (0.5 * kin - lp1) - H0;
-            if (!isfinite(dH)) dH = CUDART_INF;
-            if (a.dH) a.dH[j] = dH;
-            if (a.alpha) a.alpha[j] = dH <= 0.0 ? 1.0 : exp(-dH);
+            if (d >= D || (d >> 3) < u_lo || (d >> 3) >= u_hi) continue;
+            a.theta_out[(int64_t)d * ld + j] = thb[(int64_t)d * sld + si];
+            a.p_out[(int64_t)d * ld + j] = pb[(int64_t)d * sld + si];
         }
     }
     tc::fence_before_sync();
@@ -1002,13 +849,20 @@ __global__ void __launch_bounds__(1024) k_part_scatter(TrajArgs a, int64_t nblk)
     }
 }
 
-// g_ref[r][d] = sum over tiles of the partial sums, in tile order.
-__global__ void __launch_bounds__(128) k_centre_grad(TrajArgs a, int dk, int nch) {
-    const int r = blockIdx.x, d = threadIdx.x, R = a.c_runs;
-    if (d >= dk) return;
-    double g = 0.0;
-    for (int c = 0; c < nch; ++c) g += a.c_part[((int64_t)c * R + r) * dk + d];
-    a.c_gref[(int64_t)r * dk + d] = (float)g;
+// g_ref[r][d] = sum over tiles of the partial sums: eight groups of tiles (tile
+// modulo 8), each in tile order, then the groups (one chain over the 782 tiles
+// of n = 1e5 took 91 us).
+__global__ void __launch_bounds__(1024) k_centre_grad(TrajArgs a, int dk, int nch) {
+    __shared__ double part[8][128];
+    const int r = blockIdx.x, d = threadIdx.x & 127, g = threadIdx.x >> 7, R = a.c_runs;
+    double v = 0.0;
+    if (d < dk)
+        for (int c = g; c < nch; c += 8) v += a.c_part[((int64_t)c * R + r) * dk + d];
+    part[g][d] = v;
+    __syncthreads();
+    if (g != 0 || d >= dk) return;
+    for (int i = 1; i < 8; ++i) v += part[i][d];
+    a.c_gref[(int64_t)r * dk + d] = (float)v;
 }
 
 // CTAs per particle tile: the largest k in {1, 2, 4, 8} with at most two CTAs
@@ -1040,7 +894,7 @@ cudaError_t launch_centred(const DevModel& m, const TrajArgs& a, cudaStream_t s)
     const int64_t tiles = a.c_tiles ? a.c_ntiles : (a.N + CP - 1) / CP;
     TrajArgs a2 = a;
     a2.c_split = centred_split(m, tiles);
-    const CLayout L = c_layout(m.dk, m.Dp, LOGIT ? 1 : 0, R, a2.c_split == 1);
+    const CLayout L = c_layout(m.dk, LOGIT ? 1 : 0, R, a2.c_split == 1);
     if (L.total > C_SMEM_MAX) return cudaErrorInvalidValue;
     if (a.c_tiles) {
         const int64_t nblk = (a.N + 1023) / 1024;
@@ -1050,7 +904,7 @@ cudaError_t launch_centred(const DevModel& m, const TrajArgs& a, cudaStream_t s)
     }
     k_centre_mean<<<dim3((unsigned)R, (unsigned)m.dk), 256, 0, s>>>(a, m.D, m.dk);
     k_centre_obs<LOGIT><<<dim3((unsigned)m.n_tiles128, (unsigned)R), 128, 0, s>>>(m, a);
-    k_centre_grad<<<(unsigned)R, 128, 0, s>>>(a, m.dk, m.n_tiles128);
+    k_centre_grad<<<(unsigned)R, 1024, 0, s>>>(a, m.dk, m.n_tiles128);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     auto kern = traj_centred_kernel<LOGIT>;
@@ -1070,7 +924,7 @@ cudaError_t launch_centred(const DevModel& m, const TrajArgs& a, cudaStream_t s)
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, kern, m, a2);
     if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return launch_regression_energy(m, a, s);
 }
 
 }  // namespace

@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(GM_T, 1) traj_glm_mma_kernel(DevModel m, TrajA
                 const float eta = e0 + e1;
                 float term;
                 if (LOGIT) {
-                    const float sp = eta > 0.0f ? eta + log1pf(expf(-eta)) : log1pf(expf(eta));
+                    const float sp = softplus(eta);
                     term = yv * eta - sp;
                 } else {
                     const float z = (yv - eta) * inv_s;

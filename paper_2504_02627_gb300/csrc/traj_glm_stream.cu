@@ -33,7 +33,7 @@ __device__ __forceinline__ float gs_resid(float y, float eta, float inv_s2) {
 template <bool LOGIT>
 __device__ __forceinline__ float gs_term(float y, float eta, float inv_s) {
     if (LOGIT) {
-        const float sp = eta > 0.0f ? eta + log1pf(expf(-eta)) : log1pf(expf(eta));
+        const float sp = softplus(eta);
         return y * eta - sp;
     }
     const float z = (y - eta) * inv_s;

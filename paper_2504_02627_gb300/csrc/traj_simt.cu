@@ -46,7 +46,7 @@ __device__ __forceinline__ float glm_resid(float y, float eta, float inv_s2) {
 template <bool LOGIT>
 __device__ __forceinline__ float glm_loglik_term(float y, float eta, float inv_s) {
     if (LOGIT) {
-        float sp = eta > 0.0f ? eta + log1pf(expf(-eta)) : log1pf(expf(eta));
+        float sp = softplus(eta);
         return y * eta - sp;
     }
     float z = (y - eta) * inv_s;

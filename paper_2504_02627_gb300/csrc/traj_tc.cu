@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) traj_tc_kernel(DevModel m, Traj
             const float eta = e0 + e1, yv = y_s[i];
             float term;
             if (LOGIT) {
-                const float sp = eta > 0.0f ? eta + log1pf(expf(-eta)) : log1pf(expf(eta));
+                const float sp = softplus(eta);
                 term = yv * eta - sp;
             } else {
                 const float z = (yv - eta) * inv_s;

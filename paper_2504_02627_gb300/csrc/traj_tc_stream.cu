@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(S_THREADS, 1) traj_stream_kernel(DevModel m, T
                             const float eta = acc[o][q];
                             float term;
                             if (LOGIT) {
-                                const float sp = eta > 0.0f ? eta + log1pf(expf(-eta)) : log1pf(expf(eta));
+                                const float sp = softplus(eta);
                                 term = yv * eta - sp;
                             } else {
                                 const float z = (yv - eta) * inv_s;
