@@ -16,14 +16,20 @@ constexpr double LOG_2PI = 1.8378770664093454835606594728112;
 // ============================================================ initial draw
 // theta_0 ~ q_init = N(0, s^2 I) (Eq. for theta_0), or N(m, L L') when the
 // run has a general Gaussian initial distribution, and log q_init(theta_0)
-// parked in logw until the target has been evaluated.
-__global__ void k_init_draw(StepBufs b, float* theta) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= b.N) return;
-    const int r = b.run_of[j];
-    const RunParams rp = b.runs[r];
+// parked in logw until the target has been evaluated.  Bound by FP64 (a pair of
+// normals is some 90 instructions, 64 clocks each in a warp), so a particle's
+// pairs are spread over the INIT_SPLIT warps of a CTA of 32 particles (a thread
+// per particle had 256 particles of 10 dimensions on one SM: the whole run of ten
+// iterations 786 -> 752 us with the split; ten runs of 4096 x 25 155 -> 89 us here).
+constexpr int INIT_SPLIT = 4;
+__global__ void __launch_bounds__(32 * INIT_SPLIT) k_init_draw(StepBufs b, float* theta) {
+    __shared__ double zz_s[INIT_SPLIT][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t j = (int64_t)blockIdx.x * 32 + lane;
+    const bool on = j < b.N;
+    const RunParams rp = b.runs[on ? b.run_of[j] : 0];
     const uint32_t jl = (uint32_t)(j - rp.off);
-    if (rp.init_general) {
+    if (on && rp.init_general && w == 0) {
         // theta_d = m_d + L_d0 z_0 + ... + L_dd z_d in FP64, added column by
         // column (the same order for every d), every product and sum rounded
         // on its own (no contraction), so the result is that of the plain
@@ -47,19 +53,26 @@ __global__ void k_init_draw(StepBufs b, float* theta) {
         }
         for (int64_t d = 0; d < D; ++d) theta[d * b.ld + j] = (float)acc[d];
         b.logw[j] = __dsub_rn(-0.5 * zz, __dadd_rn(__dmul_rn(0.5 * (double)D, LOG_2PI), rp.init_logdet));
-        return;
     }
+    // a particle of a general run is done (its run's other lanes too: every lane
+    // still reaches the barrier)
+    const bool iso = on && !rp.init_general;
     double zz = 0.0;
-    for (int64_t d = 0; d < b.D; d += 2) {
-        double z0, z1;
-        normal_pair(rp.seed, (uint32_t)(d >> 1), jl, 0u, TAG_INIT, z0, z1);
-        theta[d * b.ld + j] = (float)(rp.init_scale * z0);
-        zz += z0 * z0;
-        if (d + 1 < b.D) {
-            theta[(d + 1) * b.ld + j] = (float)(rp.init_scale * z1);
-            zz += z1 * z1;
+    if (iso)
+        for (int64_t d = 2 * w; d < b.D; d += 2 * INIT_SPLIT) {
+            double z0, z1;
+            normal_pair(rp.seed, (uint32_t)(d >> 1), jl, 0u, TAG_INIT, z0, z1);
+            theta[d * b.ld + j] = (float)(rp.init_scale * z0);
+            zz += z0 * z0;
+            if (d + 1 < b.D) {
+                theta[(d + 1) * b.ld + j] = (float)(rp.init_scale * z1);
+                zz += z1 * z1;
+            }
         }
-    }
+    zz_s[w][lane] = zz;
+    __syncthreads();
+    if (!iso || w != 0) return;
+    for (int u = 1; u < INIT_SPLIT; ++u) zz += zz_s[u][lane];
     b.logw[j] = -0.5 * zz - 0.5 * (double)b.D * (LOG_2PI + 2.0 * log(rp.init_scale));
 }
 
@@ -978,8 +991,7 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
 
 // ============================================================ launchers
 cudaError_t launch_init_draw(const StepBufs& b, float* theta, cudaStream_t s) {
-    const int bs = 256;
-    k_init_draw<<<(unsigned)((b.N + bs - 1) / bs), bs, 0, s>>>(b, theta);
+    k_init_draw<<<(unsigned)((b.N + 31) / 32), 32 * INIT_SPLIT, 0, s>>>(b, theta);
     return cudaGetLastError();
 }
 cudaError_t launch_init_finish(const StepBufs& b, const double* logpi, cudaStream_t s) {
