@@ -118,8 +118,8 @@ __host__ __device__ inline CLayout c_layout_n(int dk, int n_ref, int n_run, int 
 // The most X stages that fit (4, 3 or 2).  A CTA that is not part of a
 // cluster also keeps the move's theta and p there ([dk][128] each) when they
 // fit next to the stages: the update at a pass's end then waits for no L2
-// round trip (ten runs of 4096 particles, n = 1000, D = 25: a move of about
-// 375 steps 9.80 -> 9.48 ms).
+// round trip (ten runs of 4096 particles, n = 1000, D = 25: a move of 500 steps
+// 9.80 -> 9.48 ms; such short passes have since gone to two CTAs per SM, below).
 __host__ __device__ inline CLayout c_layout(int dk, int n_ref, int n_run, bool alone) {
     CLayout L = c_layout_n(dk, n_ref, n_run, C_NS_MAX);
     for (int st = C_NS_MAX - 1; st >= 2 && L.total > C_SMEM_MAX; --st) L = c_layout_n(dk, n_ref, n_run, st);
@@ -134,6 +134,37 @@ __host__ __device__ inline CLayout c_layout(int dk, int n_ref, int n_run, bool a
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// The residuals of a pair of observations from their linear predictors, packed.
+// One SFU reciprocal serves both: 1 / q0 = q1 / (q0 q1), 1 / q1 = q0 / (q0 q1),
+// with the exponents clamped so that q0 q1 < 2^121 (a sigmoid below 2^-60 is
+// then taken as 2^-60, i.e. zero here).  cs holds the pair's (c0, c1, s0, s1);
+// the exponents, 1 + 2^x and the residuals are packed pair operations (each
+// lane rounded as its scalar form), the sum taken as (q1, q0) so that it
+// multiplies -1 / (q0 q1) into (r0, r1) as is.
+template <bool LOGIT>
+__device__ __forceinline__ uint32_t residual_pair(uint32_t e0, uint32_t e1, const float4& cs, float inv_s2) {
+    constexpr float kneg = -1.4426950408889634f;
+    const float v0f = __uint_as_float(e0), v1f = __uint_as_float(e1);
+    float r0, r1;
+    if (LOGIT) {
+        float x0, x1;
+        tc::f32x2_unpack(
+            tc::f32x2_fma(tc::f32x2_pack(kneg, kneg), tc::f32x2_pack(v0f, v1f), tc::f32x2_pack(cs.x, cs.y)), x0, x1);
+        x0 = fminf(x0, C_X_MAX);
+        x1 = fminf(x1, C_X_MAX);
+        const uint64_t q10 =
+            tc::f32x2_add(tc::f32x2_pack(tc::ex2_approx(x1), tc::ex2_approx(x0)), tc::f32x2_pack(1.0f, 1.0f));
+        float q1, q0;
+        tc::f32x2_unpack(q10, q1, q0);
+        const float rp = tc::rcp_approx(q0 * q1);
+        tc::f32x2_unpack(tc::f32x2_fma(q10, tc::f32x2_pack(-rp, -rp), tc::f32x2_pack(cs.z, cs.w)), r0, r1);
+    } else {
+        r0 = -inv_s2 * v0f;
+        r1 = -inv_s2 * v1f;
+    }
+    return pack_bf16(r0, r1);
 }
 
 // Named hardware barrier of `count` threads (ids 1.. are free: 0 is __syncthreads).
@@ -444,7 +475,6 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
         // ------------------------------------------------------------ residuals and state (warps 0-15)
         const uint32_t lane_base = (uint32_t)(32 * quarter) << 16;
         const float hf = 0.5f * ef;
-        const float kneg = -1.4426950408889634f;
         const float* gref = gref_s + run * dk;
         // a residual thread's observation pairs: 8 mm + 2 tig (+1)
         const int tig = lane & 3;
@@ -466,37 +496,6 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
                     const uint32_t rcol = tmem + lane_base + C_COL_R + (uint32_t)(bq * (CC / 2) + 32 * half);
                     const unsigned char* refs0 =
                         sm + L.off_stage + st * L.stage_bytes + L.tile_bytes + half * (64 * 8);
-                    // One SFU reciprocal serves both observations of a pair:
-                    // 1 / q0 = q1 / (q0 q1), 1 / q1 = q0 / (q0 q1), with the
-                    // exponents clamped so that q0 q1 < 2^121 (a sigmoid below
-                    // 2^-60 is then taken as 2^-60, i.e. zero here).  cs holds
-                    // the pair's (c0, c1, s0, s1); the exponents, 1 + 2^x and
-                    // the residuals are packed pair operations (each lane
-                    // rounded as its scalar form), the sum taken as (q1, q0)
-                    // so that it multiplies -1 / (q0 q1) into (r0, r1) as is.
-                    auto res_pair = [&](uint32_t e0, uint32_t e1, const float4& cs) -> uint32_t {
-                        const float v0f = __uint_as_float(e0), v1f = __uint_as_float(e1);
-                        float r0, r1;
-                        if (LOGIT) {
-                            float x0, x1;
-                            tc::f32x2_unpack(tc::f32x2_fma(tc::f32x2_pack(kneg, kneg), tc::f32x2_pack(v0f, v1f),
-                                                           tc::f32x2_pack(cs.x, cs.y)),
-                                             x0, x1);
-                            x0 = fminf(x0, C_X_MAX);
-                            x1 = fminf(x1, C_X_MAX);
-                            const uint64_t q10 = tc::f32x2_add(
-                                tc::f32x2_pack(tc::ex2_approx(x1), tc::ex2_approx(x0)), tc::f32x2_pack(1.0f, 1.0f));
-                            float q1, q0;
-                            tc::f32x2_unpack(q10, q1, q0);
-                            const float rp = tc::rcp_approx(q0 * q1);
-                            tc::f32x2_unpack(tc::f32x2_fma(q10, tc::f32x2_pack(-rp, -rp), tc::f32x2_pack(cs.z, cs.w)),
-                                             r0, r1);
-                        } else {
-                            r0 = -inv_s2 * v0f;
-                            r1 = -inv_s2 * v1f;
-                        }
-                        return pack_bf16(r0, r1);
-                    };
                     // this thread forms the residuals of the quarter's lanes
                     // g4, g4 + 8 (first group) and g4 + 16, g4 + 24 (second)
                     // for the observation pairs 8 mm + 2 tig (+1), mm = 0..7,
@@ -512,8 +511,8 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
 #pragma unroll
                         for (int mm = 0; mm < 8; ++mm) {
                             const float4 cs = LOGIT ? f[4 * mm + tig] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                            const uint32_t a0 = res_pair(v[4 * mm], v[4 * mm + 1], cs);
-                            const uint32_t a1 = res_pair(v[4 * mm + 2], v[4 * mm + 3], cs);
+                            const uint32_t a0 = residual_pair<LOGIT>(v[4 * mm], v[4 * mm + 1], cs, inv_s2);
+                            const uint32_t a1 = residual_pair<LOGIT>(v[4 * mm + 2], v[4 * mm + 3], cs, inv_s2);
                             v[2 * mm] = a0;
                             v[2 * mm + 1] = a1;
                         }
@@ -705,6 +704,401 @@ __global__ void __launch_bounds__(C_THREADS, 1) traj_centred_kernel(DevModel m, 
     tc::cluster_sync();   // no CTA leaves while another may still read its shared memory
     tc::fence_after_sync();
     if (wid == 0) tc::tmem_dealloc(tmem, C_TMEM_COLS);
+}
+
+// ---------------------------------------------------------------- two CTAs per SM
+// The same trajectories for 64 particles per CTA, two CTAs to an SM, for moves
+// whose tiles fill the GPU without a cluster (c_split = 1), D <= 64.  A pass over
+// few observation tiles is mostly its end -- the last product, the update, the
+// first product of the next pass, one after the other -- and the SM idles through
+// it unless another CTA, at another point of its own pass, forms residuals
+// meanwhile.  Ten runs of 4096 particles, n = 1000, D = 25, two iterations: 15.41
+// -> 12.80 ms a run, of which these moves were 14.4.  Still bound by latency
+// (issue 53%, the SFU 33% of their peaks), no longer by the ends of the passes.
+//
+// A particle is the MMA row 32 (r / 16) + r % 16: the 16 lanes of each TMEM
+// quarter that the residuals' 16-lane shapes read at once; the other rows are
+// zero in the deviations and never read from the results.  TMEM: G [0, 64), eta
+// [64, 192), d_r [192, 256), half of the SM's columns; one buffer of each, the
+// next product runs while the residuals are formed.  Warps 0-7 form residuals
+// (warp w: the 16 particles of quarter w % 4, half w / 4 of the observations) and
+// update the state, which stays in shared memory; warp 8 issues the copies, warp
+// 9 both products.  A row's products and sums are those of the 128-particle
+// kernel in the same order.
+constexpr int HP = 64;                      // particles per CTA
+constexpr int H_EPI_WARPS = 8, H_PRODUCER_WARP = 8, H_MMA_WARP = 9;
+constexpr int H_THREADS = 320;
+constexpr int H_DK_MAX = 64;                // one 64-dimension atom
+// Observation tiles up to which it is the faster one: a tile's waits are shared by
+// half of the residuals.  38912 particles, us a move of 40 steps here / there, D =
+// 25: 390 / 601 at n = 250, 930 / 1034 at 1000, 1618 / 1606 at 2000, 2992 / 2754
+// at 4000; D = 60: 1085 / 1301 at 1000, 3397 / 3218 at 4000.
+constexpr int H_TILES_MAX = 12;
+constexpr uint32_t H_TMEM_COLS = 256, H_COL_G = 0, H_COL_ETA = 64, H_COL_R = 192;
+constexpr int H_SMEM_MAX = 113 * 1024;      // half of an SM's
+
+struct HLayout {
+    int ref_bytes, stage_bytes, stages, off_stage, off_state, off_ref, off_bar, total;
+};
+__host__ __device__ inline HLayout h_layout(int dk, bool logit) {
+    HLayout L;
+    L.ref_bytes = logit ? CC * 8 : 0;
+    L.stage_bytes = C_ATOM + L.ref_bytes;
+    L.off_stage = C_DATOM;                                          // the deviations come first
+    const int rest = 2 * dk * HP * 4 + 2 * dk * 4 + 256 + 1024;     // state, reference, barriers, alignment slack
+    L.stages = C_NS_MAX;
+    while (L.stages > 2 && L.off_stage + L.stages * L.stage_bytes + rest > H_SMEM_MAX) L.stages -= 1;
+    L.off_state = L.off_stage + L.stages * L.stage_bytes;
+    L.off_ref = L.off_state + 2 * dk * HP * 4;
+    L.off_bar = L.off_ref + 2 * dk * 4;
+    L.total = L.off_bar + 256 + 1024;
+    return L;
+}
+
+template <bool LOGIT>
+__global__ void __launch_bounds__(H_THREADS, 2) traj_centred_half_kernel(DevModel m, TrajArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* sm = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
+    const HLayout L = h_layout(m.dk, LOGIT);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int D = m.D, dk = m.dk, nch = m.n_tiles128, NS = L.stages, nunit = dk / 8;
+    const int64_t ld = a.ld;
+    const int64_t tile = blockIdx.x >> 1;
+    int trun = 0;
+    int64_t slot0 = tile * CP;
+    if (a.c_tiles) {
+        const int2 tt = a.c_tiles[tile];
+        trun = tt.x;
+        slot0 = tt.y;
+    }
+    slot0 += HP * (int64_t)(blockIdx.x & 1);
+    uint64_t* full = reinterpret_cast<uint64_t*>(sm + L.off_bar);   // [NS] stage filled
+    uint64_t* empty = full + C_NS_MAX;                               // [NS] stage consumed by both products
+    uint64_t* eta_full = empty + C_NS_MAX;                           // first product done
+    uint64_t* eta_empty = eta_full + 1;                              // eta read by the residual warps
+    uint64_t* r_full = eta_empty + 1;                                // d_r written
+    uint64_t* r_empty = r_full + 1;                                  // second product done with d_r
+    uint64_t* g_full = r_empty + 1;                                  // pass's gradient complete
+    uint64_t* th_full = g_full + 1;                                  // next pass's deviations written
+    uint64_t* fin = th_full + 1;                                     // every product issued has completed
+    uint32_t* tmem_s = reinterpret_cast<uint32_t*>(fin + 1);
+    int* smax_s = reinterpret_cast<int*>(tmem_s + 1);
+    volatile int* abort_s = smax_s + 1;
+    float* const cref = reinterpret_cast<float*>(sm + L.off_ref);    // the run's reference point, reference gradient
+    float* const gref = cref + dk;
+    float* const th_s = reinterpret_cast<float*>(sm + L.off_state);  // [dk][64], columns of odd units swapped by 16
+    float* const p_s = th_s + dk * HP;
+    const uint32_t s_base = tc::smem_u32(sm);
+    int* err = a.dev_err;
+
+    if (tid == 0) {
+        for (int i = 0; i < NS; ++i) {
+            tc::mbar_init(&full[i], 1);
+            tc::mbar_init(&empty[i], 1);
+        }
+        tc::mbar_init(eta_full, 1);
+        tc::mbar_init(eta_empty, H_EPI_WARPS);
+        tc::mbar_init(r_full, H_EPI_WARPS);
+        tc::mbar_init(r_empty, 1);
+        tc::mbar_init(g_full, 1);
+        tc::mbar_init(th_full, H_EPI_WARPS);
+        tc::mbar_init(fin, 1);
+        tc::fence_mbar_init();
+        *smax_s = 0;
+        *abort_s = 0;
+    }
+    if (wid == 0) {
+        tc::tmem_alloc(tmem_s, H_TMEM_COLS);
+        tc::tmem_relinquish();
+    }
+    for (int i = tid; i < dk; i += H_THREADS) {
+        cref[i] = a.c_centre[(int64_t)trun * dk + i];
+        gref[i] = a.c_gref[(int64_t)trun * dk + i];
+    }
+    for (int i = tid; i < C_DATOM / 16; i += H_THREADS) reinterpret_cast<uint4*>(sm)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+
+    // ---------------------------------------------------------------- particle state (warps 0-7)
+    // A thread keeps the units 2 p + lane / 16 of particle 16 (w % 4) + lane % 16
+    // for the unit pairs p = w / 4, w / 4 + 2.
+    const bool epi = wid < H_EPI_WARPS;
+    const int quarter = wid & 3, half = (wid >> 2) & 1, upper = lane >> 4;
+    const int prow = 16 * quarter + (lane & 15);
+    const int mrow = 32 * quarter + (lane & 15);                      // its MMA row
+    const int scol = prow ^ (upper << 4);                             // its column in th_s / p_s (its units are all odd or all even)
+    const float inv_tau2 = LOGIT ? (float)(1.0 / (m.h0 * m.h0)) : (float)(1.0 / (m.h1 * m.h1));
+    const float inv_s2 = LOGIT ? 0.0f : (float)(1.0 / (m.h0 * m.h0));
+    int64_t j = -1, src = -1;
+    int S = 0;
+    float ef = 0.0f;
+    auto write_unit = [&](int unit, const float (&tv)[8]) {
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int d = 8 * unit + e;
+            v[e] = (j >= 0 && d < D) ? tv[e] - cref[d] : 0.0f;
+        }
+        *reinterpret_cast<uint4*>(sm + mrow * 128 + ((unit ^ (mrow & 7)) << 4)) =
+            make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+    };
+    if (epi) {
+        const int64_t t = slot0 + prow;
+        uint64_t seed = 0;
+        uint32_t kk = 0, jl = 0;
+        if (a.c_tiles) j = a.c_perm[t];                               // -1 in a pad slot
+        else if (t < a.N) j = a.perm ? a.perm[t] : t;
+        if (j >= 0) {
+            src = a.src ? a.src[j] : j;
+            S = a.steps[j];
+            double eps;
+            int run;
+            particle_run(a, j, run, eps, seed, kk, jl);
+            ef = (float)eps;
+        }
+#pragma unroll 1
+        for (int pr = half; 2 * pr < nunit; pr += 2) {
+            const int unit = 2 * pr + upper;
+            float tv[8];
+#pragma unroll
+            for (int e = 0; e < 8; e += 2) {
+                const int d = 8 * unit + e;
+                float pv[2] = {0.0f, 0.0f};
+                tv[e] = tv[e + 1] = 0.0f;
+                if (j >= 0 && d < D) {
+                    const bool two = d + 1 < D;
+                    tv[e] = a.theta_in[(int64_t)d * ld + src];
+                    if (two) tv[e + 1] = a.theta_in[(int64_t)(d + 1) * ld + src];
+                    // momentum (given, or Philox + Box-Muller); the first half
+                    // kick waits for the gradient of pass 0
+                    if (a.p_in) {
+                        pv[0] = a.p_in[(int64_t)d * ld + j];
+                        if (two) pv[1] = a.p_in[(int64_t)(d + 1) * ld + j];
+                    } else {
+                        double z0, z1;
+                        normal_pair(seed, (uint32_t)(d >> 1), jl, kk, TAG_MOM, z0, z1);
+                        pv[0] = (float)z0;
+                        pv[1] = two ? (float)z1 : 0.0f;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    th_s[(d + u) * HP + scol] = tv[e + u];
+                    p_s[(d + u) * HP + scol] = pv[u];
+                }
+            }
+            write_unit(unit, tv);
+        }
+    }
+    tc::fence_proxy_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (epi && S > 0) atomicMax(smax_s, S);
+    // H_0, for the end-point energies' launch: the dimensions in order, in groups of 32
+    if (epi && half == 0 && upper == 0 && j >= 0 && a.dH) {
+        double kin[2] = {0.0, 0.0};
+        for (int d = 0; d < D; ++d) {
+            const double v = widen(p_s[d * HP + (prow ^ (((d >> 3) & 1) << 4))]);
+            kin[d >> 5] += v * v;
+        }
+        a.dH[j] = 0.5 * (kin[0] + kin[1]) - a.logpi_in[src];
+    }
+    __syncthreads();
+    const uint32_t tmem = *tmem_s;
+    const int npass = *smax_s + 1;                                    // pass 0: gradient at the start point
+
+    if (wid == H_PRODUCER_WARP) {
+        // ------------------------------------------------------------ producer
+        if (lane == 0) {
+            const uint32_t bytes = (uint32_t)L.stage_bytes;
+            const int64_t total = (int64_t)npass * nch;
+            int st = 0, c = 0;
+            uint32_t ph = 0;
+            for (int64_t it = 0; it < total; ++it) {
+                tc::mbar_wait_timed(&empty[st], ph ^ 1u, err, abort_s);
+                tc::mbar_arrive_expect_tx(&full[st], bytes);
+                unsigned char* dst = sm + L.off_stage + st * L.stage_bytes;
+                tc::bulk_g2s(dst, m.xc_img + (int64_t)c * (C_ATOM / 2), (uint32_t)C_ATOM, &full[st]);
+                if (LOGIT)
+                    tc::bulk_g2s(dst + C_ATOM, a.c_refs + ((int64_t)c * a.c_runs + trun) * CC, (uint32_t)L.ref_bytes,
+                                 &full[st]);
+                if (++c == nch) c = 0;
+                if (++st == NS) {
+                    st = 0;
+                    ph ^= 1u;
+                }
+            }
+            // every copy has landed before the CTA exits
+            const int64_t first = total > NS ? total - NS : 0;
+            for (int64_t it = first; it < total; ++it)
+                tc::mbar_wait_timed(&full[(int)(it % NS)], (uint32_t)((it / NS) & 1), err, abort_s);
+        }
+    } else if (wid == H_MMA_WARP) {
+        // ------------------------------------------------------------ both products
+        if (lane == 0) {
+            const uint32_t IDESC1 = tc::idesc_bf16_f32(CP, CC);
+            const uint32_t IDESC2 = tc::idesc_bf16_f32(CP, (uint32_t)dk) | (1u << 16);   // B MN-major
+            const int ksteps1 = dk / 16;
+            int s1 = 0, s2 = 0;                 // stages of the next first and second product
+            uint32_t ph = 0, e1 = 0, e2 = 0;    // phases: of stage s1, of eta, of d_r
+            // d_eta = dev . X_c^T of the next tile
+            auto first = [&]() {
+                tc::mbar_wait_timed(&full[s1], ph, err, abort_s);
+                tc::mbar_wait_timed(eta_empty, e1 ^ 1u, err, abort_s);
+                tc::fence_after_sync();
+                const uint32_t xt = s_base + L.off_stage + s1 * L.stage_bytes;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                    if (kk < ksteps1)
+                        tc::mma_bf16(tmem + H_COL_ETA, tc::smem_desc(s_base + kk * 32, 16, 1024, tc::SWZ_128B),
+                                     tc::smem_desc(xt + kk * 32, 16, 1024, tc::SWZ_128B), IDESC1, kk > 0 ? 1u : 0u);
+                tc::mma_commit(eta_full);
+                if (++s1 == NS) {
+                    s1 = 0;
+                    ph ^= 1u;
+                }
+                e1 ^= 1u;
+            };
+            for (int s = 0; s < npass; ++s) {
+                if (s >= 1) tc::mbar_wait_timed(th_full, (uint32_t)((s - 1) & 1), err, abort_s);
+                first();
+                for (int c = 0; c < nch; ++c) {
+                    if (c + 1 < nch) first();
+                    // G += d_r^T . X_c
+                    tc::mbar_wait_timed(r_full, e2, err, abort_s);
+                    tc::fence_after_sync();
+                    const uint32_t xt = s_base + L.off_stage + s2 * L.stage_bytes;
+#pragma unroll
+                    for (int kk = 0; kk < CC / 16; ++kk)
+                        tc::mma_bf16_ta(tmem + H_COL_G, tmem + H_COL_R + (uint32_t)(kk * 8),
+                                        tc::smem_desc(xt + kk * 2048, C_ATOM, 1024, tc::SWZ_128B), IDESC2,
+                                        (c > 0 || kk > 0) ? 1u : 0u);
+                    tc::mma_commit(r_empty);
+                    tc::mma_commit(&empty[s2]);
+                    if (c == nch - 1) tc::mma_commit(g_full);
+                    if (++s2 == NS) s2 = 0;
+                    e2 ^= 1u;
+                }
+            }
+            tc::mma_commit(fin);
+        }
+    } else {
+        // ------------------------------------------------------------ residuals and state (warps 0-7)
+        const uint32_t lane_base = (uint32_t)(32 * quarter) << 16;
+        const uint32_t ecol = tmem + lane_base + H_COL_ETA + (uint32_t)(64 * half);
+        const uint32_t rcol = tmem + lane_base + H_COL_R + (uint32_t)(32 * half);
+        const float hf = 0.5f * ef;
+        const int tig = lane & 3;
+        int st = 0;
+        uint32_t sph = 0, ph = 0;
+        for (int s = 0; s < npass; ++s) {
+            for (int c = 0; c < nch; ++c) {
+                // one thread waits for the tile; the others sleep on a hardware
+                // barrier instead of polling
+                if (tid == 0) {
+                    tc::mbar_wait_timed(eta_full, ph, err, abort_s);
+                    tc::mbar_wait_timed(&full[st], sph, err, abort_s);
+                }
+                named_sync(1u, 32u * H_EPI_WARPS);
+                tc::fence_after_sync();
+                uint32_t v[32];
+                tc::tmem_ld16x256_x8_nowait(ecol, v);
+                tc::tmem_wait_ld();
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(eta_empty);
+                // lanes g4, g4 + 8 of the quarter, observation pairs 8 mm + 2 tig
+                // (+1) of the half, packed over consumed registers (the order of
+                // the 16x128b store)
+                const float4* f = reinterpret_cast<const float4*>(sm + L.off_stage + st * L.stage_bytes + C_ATOM +
+                                                                  half * (64 * 8));
+#pragma unroll
+                for (int mm = 0; mm < 8; ++mm) {
+                    const float4 cs = LOGIT ? f[4 * mm + tig] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    const uint32_t a0 = residual_pair<LOGIT>(v[4 * mm], v[4 * mm + 1], cs, inv_s2);
+                    const uint32_t a1 = residual_pair<LOGIT>(v[4 * mm + 2], v[4 * mm + 3], cs, inv_s2);
+                    v[2 * mm] = a0;
+                    v[2 * mm + 1] = a1;
+                }
+                // the previous residuals have been read by the second product
+                if (lane == 0) tc::mbar_wait_timed(r_empty, ph ^ 1u, err, abort_s);
+                __syncwarp();
+                tc::fence_after_sync();
+                tc::tmem_st16x128_x8_nowait(rcol, v);
+                tc::tmem_wait_st();
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(r_full);
+                ph ^= 1u;
+                if (++st == NS) {
+                    st = 0;
+                    sph ^= 1u;
+                }
+            }
+            // the pass's gradient g_ref + G - theta / tau^2, then the leapfrog update
+            if (tid == 0) tc::mbar_wait_timed(g_full, (uint32_t)(s & 1), err, abort_s);
+            named_sync(1u, 32u * H_EPI_WARPS);
+            tc::fence_after_sync();
+            const bool live = j >= 0 && s <= S, more = s + 1 < npass;
+#pragma unroll 1
+            for (int pr = half; 2 * pr < nunit; pr += 2) {
+                // the pair's columns of the quarter's first 16 lanes; the upper
+                // lanes take the second unit
+                uint32_t g0[8], g1[8];
+                tc::tmem_ld8_nowait(tmem + lane_base + H_COL_G + (uint32_t)(16 * pr), g0);
+                tc::tmem_ld8_nowait(tmem + lane_base + H_COL_G + (uint32_t)(16 * pr + 8), g1);
+                tc::tmem_wait_ld();
+                const int unit = 2 * pr + upper;
+                float tv[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t o = __shfl_sync(0xffffffffu, g1[e], lane & 15);
+                    const float gs = __uint_as_float(upper ? o : g0[e]);
+                    const int d = 8 * unit + e;
+                    tv[e] = 0.0f;
+                    if (live && d < D) {
+                        float t0 = th_s[d * HP + scol], pv = p_s[d * HP + scol];
+                        const float g = gref[d] + gs - t0 * inv_tau2;
+                        if (s == S) a.grad_out[(int64_t)d * ld + j] = g;
+                        if (s >= 1) pv = fmaf(hf, g, pv);
+                        if (s < S) {
+                            pv = fmaf(hf, g, pv);
+                            t0 = fmaf(ef, pv, t0);
+                            th_s[d * HP + scol] = t0;
+                        }
+                        p_s[d * HP + scol] = pv;
+                        tv[e] = t0;
+                    }
+                }
+                if (more) write_unit(unit, tv);
+            }
+            if (more) {
+                tc::fence_proxy_async_smem();
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(th_full);
+            }
+        }
+        // the final state, kept by this thread
+        if (j >= 0)
+            for (int pr = half; 2 * pr < nunit; pr += 2) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int d = 8 * (2 * pr + upper) + e;
+                    if (d >= D) continue;
+                    a.theta_out[(int64_t)d * ld + j] = th_s[d * HP + scol];
+                    a.p_out[(int64_t)d * ld + j] = p_s[d * HP + scol];
+                }
+            }
+    }
+    if (tid == 0) {
+        volatile int ignore_abort = 0;   // this drain wait runs even after an abort
+        tc::mbar_wait_timed(fin, 0u, err, &ignore_abort, 4000000000ull);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (wid == 0) tc::tmem_dealloc(tmem, H_TMEM_COLS);
 }
 
 // ---------------------------------------------------------------- reference point and quantities
@@ -907,6 +1301,17 @@ cudaError_t launch_centred(const DevModel& m, const TrajArgs& a, cudaStream_t s)
     k_centre_grad<<<(unsigned)R, 1024, 0, s>>>(a, m.dk, m.n_tiles128);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    // no cluster and short passes: two CTAs per SM
+    if (a2.c_split == 1 && !a.eval_only && m.dk <= H_DK_MAX && m.n_tiles128 <= H_TILES_MAX) {
+        const HLayout H = h_layout(m.dk, LOGIT);
+        auto half = traj_centred_half_kernel<LOGIT>;
+        e = cudaFuncSetAttribute(half, cudaFuncAttributeMaxDynamicSharedMemorySize, H.total);
+        if (e != cudaSuccess) return e;
+        half<<<(unsigned)(2 * tiles), H_THREADS, H.total, s>>>(m, a2);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        return launch_regression_energy(m, a, s);
+    }
     auto kern = traj_centred_kernel<LOGIT>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
     if (e != cudaSuccess) return e;
