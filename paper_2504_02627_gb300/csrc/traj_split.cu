@@ -50,6 +50,15 @@ __device__ __forceinline__ void banana_grad(float a, float b, float inva, float 
     g0 = -xo * inva + 2.0f * b * u * xo;
     g1 = -u;
 }
+// A pair's part of log pi.  Which of its two products is rounded on its own is
+// written out, so that the value does not vary with what the compiler contracts in
+// an instance of the kernel: the second, and for a single pair the first, as a
+// thread that holds the whole particle has it.
+__device__ __forceinline__ float banana_term(float a, float b, float half_inva, float xo, float xe, bool single) {
+    const float u = xe - b * (xo * xo - a);
+    const float s = __fmul_rn(-half_inva, xo), t = __fmul_rn(0.5f, u);
+    return single ? fmaf(-t, u, __fmul_rn(s, xo)) : fmaf(s, xo, -__fmul_rn(t, u));
+}
 
 // A warp holds 32 consecutive slots; the PW warps of a slot group share the
 // particles' pairs, warp w taking pairs w, w + PW, ..., NPT of them side by
@@ -121,8 +130,7 @@ __global__ void __launch_bounds__(256) traj_banana_kernel(DevModel m, TrajArgs a
             const int i = w + k * pw;
             if (i >= np) continue;
             const int64_t o = (int64_t)(2 * i) * a.ld + x.j;
-            const float u = xe[k] - fb * (xo[k] * xo[k] - fa);
-            slp[i * 32 + lane] = -half_inva * xo[k] * xo[k] - 0.5f * u * u;
+            slp[i * 32 + lane] = banana_term(fa, fb, half_inva, xo[k], xe[k], np == 1);
             a.grad_out[o] = g0[k];
             a.grad_out[o + a.ld] = g1[k];
             if (a.eval_only) continue;

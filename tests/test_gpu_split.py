@@ -66,6 +66,30 @@ def test_banana_pairs_are_independent_of_their_neighbours(D):
     dm.close()
 
 
+@pytest.mark.parametrize("D", [2, 4, 8, 16, 18, 64])
+def test_banana_log_density_is_its_written_fp32_form(D):
+    """The FP32 terms to the last bit (an FMA of FP32 values is exact in FP64 but
+    for its rounding), their FP64 sum up to its order."""
+    need_gpu()
+    dm = B.DevModel(B.ModelData(B.BANANA, D, hyper=(10.0, 0.1)), stream())
+    n = 500
+    th = torch.as_tensor(np.random.default_rng(D).standard_normal((D, n)).astype(np.float32)).cuda()
+    gr, lp = torch.zeros(D, n, device="cuda"), torch.zeros(n, dtype=torch.float64, device="cuda")
+    B.check(B.lib().smc_k_target(dm.h, ptr(th), n, n, ptr(lp), ptr(gr), 0, stream()), "target")
+    f = np.float32
+    fma = lambda x, y, z: (x.astype(np.float64) * y.astype(np.float64) + z.astype(np.float64)).astype(f)
+    xo, xe = th.cpu().numpy()[0::2], th.cpu().numpy()[1::2]
+    full = lambda v: np.full_like(xo, f(v))
+    u = fma(full(-0.1), fma(xo, xo, full(-10.0)), xe)
+    s, t = f(-0.05) * xo, f(0.5) * u
+    terms = fma(-t, u, s * xo) if D == 2 else fma(s, xo, -(t * u))
+    want = terms.astype(np.float64).sum(axis=0)
+    got = lp.cpu().numpy()
+    const = np.median(got - want)                       # the normalising constant
+    assert np.all(np.abs(got - want - const) <= 1e-13 * (np.abs(terms).sum(axis=0) + abs(const)))
+    dm.close()
+
+
 @pytest.mark.parametrize("kind,D,n,N", [("gauss", 100, 0, 3100), ("gauss", 40, 0, 20011), ("logistic", 25, 1000, 515),
                                         ("logistic", 40, 3000, 130)])
 @pytest.mark.parametrize("precision", [0, 1])
