@@ -94,18 +94,21 @@ cudaError_t launch_order_steps(const int32_t* steps, int64_t N, int32_t* perm, c
 }
 
 // Ordering pays where the particles of a tile share the longest trajectory and a
-// step of the launch takes about a microsecond or more (some 5e7 operations):
-// below that the move is over in the time that ordering takes.  Counts uniform
-// on 1 .. S: the n = 1000, D = 25 regression, 4096 particles, S = 40, 617 ->
-// 326 us; the 100-d Gaussian in BF16x3, 8191 particles, S = 50, 150 -> 122 us.
+// step of the launch takes about a microsecond or more (some 5e7 operations, 1e8
+// on the matrix units): below that the move is over in the time that ordering
+// takes.  Counts uniform on 1 .. S: the n = 1000, D = 25 regression, 4096 particles, S = 40, 617 ->
+// 326 us; the 100-d Gaussian in BF16x3, 8191 particles, S = 50, 150 -> 122 us, 6000
+// particles, S = 30, 69 -> 62 us (a move of 30 steps each: 70 -> 72); in 40 and 64
+// dimensions, 16384 particles, 49 -> 51 and 64 -> 65 us (30 steps each 60 -> 68, the
+// scattered reads of the state): left in the particles' order.
 // The centred and
 // the other tcgen05 kernels keep state at the particles' indices and read it
 // every step, coalesced only in the particles' own order.
 bool order_pays(const DevModel& m, int32_t precision, int64_t N) {
     double per = 0.0;   // operations of one particle's gradient
-    if (m.kind == GAUSS_DENSE && m.D > 32 && precision <= 2) per = 2.0 * m.D * m.D;
+    if (m.kind == GAUSS_DENSE && m.D > (precision == 0 ? 32 : 64) && precision <= 2) per = 2.0 * m.D * m.D;
     if ((m.kind == LOGISTIC || m.kind == LINEAR_GAUSS) && precision == 0) per = 4.0 * m.n * m.D;
-    return per * (double)N >= 5e7;
+    return per * (double)N >= (precision == 0 ? 5e7 : 1e8);
 }
 
 }  // namespace smc
