@@ -65,8 +65,9 @@ smc_status smc_k_resample_noalloc(const double* W, int64_t N, uint64_t r64, uint
         fprintf(stderr, "smc_k_resample_noalloc: cudaGetSymbolAddress failed: %s\n", cudaGetErrorString(e));
         return SMC_E_CUDA;
     }
-    // launch_resample_flat clears the tile descriptors and writes the header
-    // before the scan reads them, so leftovers of an earlier call are harmless.
+    // launch_resample_flat writes all that it reads of the scratch (the tiles'
+    // totals, or the header and cleared descriptors of the look-back), so
+    // leftovers of an earlier call are harmless.
     e = smc::launch_resample_flat(W, N, r64, reinterpret_cast<unsigned long long*>(q), ancestors, status_out,
                                   scratch, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) {
