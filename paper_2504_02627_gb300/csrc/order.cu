@@ -98,9 +98,9 @@ cudaError_t launch_order_steps(const int32_t* steps, int64_t N, int32_t* perm, c
 // on the matrix units): below that the move is over in the time that ordering
 // takes.  Counts uniform on 1 .. S: the n = 1000, D = 25 regression, 4096 particles, S = 40, 617 ->
 // 326 us; the 100-d Gaussian in BF16x3, 8191 particles, S = 50, 150 -> 122 us, 6000
-// particles, S = 30, 69 -> 62 us (a move of 30 steps each: 70 -> 72); in 40 and 64
-// dimensions, 16384 particles, 49 -> 51 and 64 -> 65 us (30 steps each 60 -> 68, the
-// scattered reads of the state): left in the particles' order.
+// particles, S = 30, 69 -> 62 us (a move of 30 steps each: 70 -> 72); in 64
+// dimensions, 16384 particles, 69 -> 65 us (30 steps each 66 -> 68), in 40 as much
+// as it costs: left in the particles' order.
 // The centred and
 // the other tcgen05 kernels keep state at the particles' indices and read it
 // every step, coalesced only in the particles' own order.

@@ -71,8 +71,13 @@ __device__ __forceinline__ float gg_sq4(const float (&pp)[2][4], int h) {
 // state elements (u, 2 h + v), u, h, v in {0, 1}: particle gq + 8 h of the
 // CTA, dimension 16 w + 8 u + 2 tq + v -- the m16n8 accumulator layout of
 // n-tile 2 w + u.
+// Resident CTAs that the registers are capped for: where the kernel runs many
+// waves they count (D = 64, 16384 particles, 30 steps: 60 us with four CTAs, 66 with
+// three, for which a few registers more suffice).
+constexpr int gg_ctas(int ks) { return ks <= 3 ? 6 : ks == 4 ? 4 : ks == 5 ? 3 : 2; }
+
 template <int KS, bool X3>
-__global__ void __launch_bounds__(32 * KS, 2) traj_gauss_mma_kernel(DevModel m, TrajArgs a) {
+__global__ void __launch_bounds__(32 * KS, gg_ctas(KS)) traj_gauss_mma_kernel(DevModel m, TrajArgs a) {
     constexpr int NTH = 32 * KS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int D = m.D;
