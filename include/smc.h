@@ -208,7 +208,10 @@ smc_status smc_init_batch(smc_handle** out, int64_t n_runs, const smc_config* cf
 /* One SMC iteration (the loop body of Algorithm 3): normalise, ESS test,
  * systematic resampling, jittered ChEES-HMC move of every particle, reweight
  * by -Delta H, ChEES adaptation.  stats (n_runs entries) may be NULL; when
- * non-NULL the call synchronises the stream and copies the statistics. */
+ * non-NULL the call synchronises the stream and copies the statistics.  An
+ * iteration that fails after its first launch cannot be tried again (its
+ * counts have been added to): every later step returns SMC_E_STATE until
+ * smc_reset, which serves after SMC_E_NOMEM but not after SMC_E_CUDA. */
 smc_status smc_step(smc_handle* h, smc_stats* stats);
 
 /* n_iters calls of smc_step; per_iter (n_iters * n_runs, iteration-major) may

@@ -937,7 +937,24 @@ smc_status smc_step(smc_handle* h, smc_stats* stats) {
     if (h->sticky) return SMC_E_STATE;
     cudaStream_t s = h->stream;
     StepBufs b = make_bufs(h);
-    cudaError_t e = launch_weights_steps(b, s);
+    // From the first kernel on, the step histogram and the weights' total hold
+    // this iteration's counts.  A second attempt would add to them, and the
+    // launch order's slots would run past its end: whatever stops an iteration
+    // that has begun, the handle waits for smc_reset, which empties both.
+    // (A captured iteration has not begun.)
+    bool begun = false;
+    auto broken = [&](cudaError_t err, const char* where) {
+        const smc_status st = cuda_fail(h, err, where);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        (void)cudaStreamIsCapturing(s, &cap);
+        if (begun && cap == cudaStreamCaptureStatusNone) h->sticky = st;
+        return st;
+    };
+    cudaError_t e = cudaGetLastError();   // an earlier call's error, which the launch would report as its own
+    if (e == cudaSuccess) {
+        e = launch_weights_steps(b, s);
+        begun = e == cudaSuccess;
+    }
     if (e == cudaSuccess) e = launch_resample_scan(b, s);
     if (e == cudaSuccess) e = launch_sort(b, s);
     if (e == cudaSuccess && flow_trains_at(h, h->iters_done + 1)) e = flow_train(h, s);
@@ -969,7 +986,7 @@ smc_status smc_step(smc_handle* h, smc_stats* stats) {
             while (h->events.size() < i + 2) {
                 cudaEvent_t ev;
                 e = cudaEventCreate(&ev);
-                if (e != cudaSuccess) return cuda_fail(h, e, "smc_step profiling");
+                if (e != cudaSuccess) return broken(e, "smc_step profiling");
                 h->events.push_back(ev);
             }
             cudaEventRecord(h->events[i], s);
@@ -986,7 +1003,7 @@ smc_status smc_step(smc_handle* h, smc_stats* stats) {
         }
     }
     if (e == cudaSuccess) e = launch_move_stats(b, s);
-    if (e != cudaSuccess) return cuda_fail(h, e, "smc_step launch");
+    if (e != cudaSuccess) return broken(e, "smc_step launch");
     h->cur = 1 - h->cur;
     h->iters_done += 1;
     if (stats) return read_stats(h, stats);
