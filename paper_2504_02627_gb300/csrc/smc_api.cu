@@ -100,6 +100,17 @@ struct OrderRoom {
     unsigned long long stream_id = 0;
     bool any = false;
     std::mutex mu;
+    // Whether that launch has finished.  An event query in the thread's own
+    // mode would break a capture that another thread has under way in the
+    // global mode; the event is never recorded inside a capture, so the
+    // relaxed mode is safe.
+    bool finished() const {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+        const bool done = cudaEventQuery(used) == cudaSuccess;
+        (void)cudaThreadExchangeStreamCaptureMode(&mode);   // as it was
+        return done;
+    }
 };
 
 struct smc_dev_model {
@@ -1460,7 +1471,7 @@ smc_status smc_k_leapfrog(const smc_dev_model* m, float* theta, float* p, float*
     unsigned long long id = 0;
     bool mine = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
                 cudaStreamGetId(s, &id) == cudaSuccess;
-    if (mine && room.any && id != room.stream_id) mine = cudaEventQuery(room.used) == cudaSuccess;
+    if (mine && room.any && id != room.stream_id) mine = room.finished();
     if (!mine) {
         (void)cudaGetLastError();   // cudaErrorNotReady is no error of this call
         return kstatus(launch_traj(m->m, a, precision, s));

@@ -54,6 +54,9 @@ void host_cuda_foreign_capture(int on) {
     foreign_broken = false;
 }
 int host_cuda_foreign_capture_broken() { return foreign_broken; }
+int host_cuda_mode() { return (int)mode; }
+int host_cuda_last_error() { return (int)last; }
+void host_cuda_capture(int on) { capturing = on != 0; }
 void host_cuda_event_busy(int on) { event_busy = on != 0; }
 
 // ---- what nvcc's host code calls

@@ -1,0 +1,60 @@
+"""Which stage-level moves take the launch order, and what the call does beside
+other streams' work and captures, on the host's CUDA runtime (no kernel runs;
+test_gpu_ordered_moves.py has the results on the GPU)."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import host_cuda
+import paper_2504_02627_gb300 as g
+from paper_2504_02627_gb300 import _binding as B
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return host_cuda.load(tmp_path_factory.mktemp("host_cuda"))
+
+
+def _model(lib, D=100):
+    md = B.ModelData(B.GAUSS_DENSE, D, mu=np.zeros(D), prec=np.eye(D))
+    m = C.c_void_p()
+    assert lib.smc_model_create(C.byref(m), C.byref(md.struct), None) == 0
+    host_cuda.launches(lib)
+    return m
+
+
+def _ordered(lib, m, stream, N=6007, precision=0):
+    """Whether a move on this stream was ordered."""
+    room = C.c_void_p(4096)                       # never read: no kernel runs
+    assert lib.smc_k_leapfrog(m, room, room, room, room, room, 0.1, N, N, precision, C.c_void_p(stream)) == 0
+    names = host_cuda.launches(lib)
+    assert any("traj" in n for n in names)
+    return any("k_order_steps" in n for n in names)
+
+
+def test_a_capture_of_another_thread_is_left_whole(lib):
+    m = _model(lib)
+    lib.host_cuda_foreign_capture(0)
+    assert _ordered(lib, m, 16)
+    lib.host_cuda_foreign_capture(1)
+    assert _ordered(lib, m, 32)                   # the room's last move ran on another stream, and has ended
+    assert not lib.host_cuda_foreign_capture_broken()
+    lib.host_cuda_foreign_capture(0)
+    assert lib.host_cuda_mode() == 0              # as the thread had it: global
+    lib.smc_model_destroy(m)
+
+
+def test_a_move_without_the_room_runs_in_the_particles_order(lib):
+    m = _model(lib)
+    assert _ordered(lib, m, 16)
+    lib.host_cuda_event_busy(1)
+    assert _ordered(lib, m, 16)                   # behind its own stream's move
+    assert not _ordered(lib, m, 32)               # that move may still read the room
+    lib.host_cuda_event_busy(0)
+    assert _ordered(lib, m, 32)
+    lib.host_cuda_capture(1)
+    assert not _ordered(lib, m, 32)               # a replay could overlap later calls
+    lib.host_cuda_capture(0)
+    assert lib.host_cuda_last_error() == 0        # the busy event is no error of the caller's
+    lib.smc_model_destroy(m)
