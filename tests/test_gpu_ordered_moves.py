@@ -9,6 +9,9 @@ from paper_2504_02627_gb300 import _binding as B
 
 pytestmark = pytest.mark.gpu
 D, N = 100, 6007
+# particles and precision of dense Gaussians in D dimensions that are ordered
+# (test_host_ordered_moves.py holds them against the rule); 97 are not
+ORDERED = [(N, 0), (N, 1), (N, 2), (5003, 1), (16411, 2)]
 
 
 def _gauss(s):
@@ -70,4 +73,28 @@ def test_moves_beside_captures_and_busy_streams():
         for k in (1, 2, 3):
             for u, v in zip(x[0], x[k]):
                 assert torch.equal(u, v)
+    dm.close()
+
+
+@pytest.mark.parametrize("n,precision", ORDERED)
+def test_ordered_moves_of_every_precision(n, precision):
+    """Ragged, equal and zero step counts, against the same particles in
+    launches of 97, which are not ordered.  The gradients are not those of the
+    positions: a particle without steps keeps the one it came with."""
+    need_gpu()
+    s = torch.cuda.current_stream()
+    dm = _gauss(s)
+    start = _state(n, n)
+    rng = np.random.default_rng(n)
+    for counts in (rng.integers(0, 9, size=n), np.full(n, 3), rng.integers(0, 2000, size=n) // 400, np.zeros(n, int)):
+        S = dev(counts.astype(np.int32))
+        whole = [t.clone() for t in start]
+        _move(dm, whole, S, s, precision)
+        for lo in range(0, n, 97):
+            part = [t[..., lo:lo + 97].clone(memory_format=torch.contiguous_format) for t in start]
+            _move(dm, part, S[lo:lo + 97].clone(), s, precision)
+            for u, v in zip(part, whole):
+                assert torch.equal(u, v[..., lo:lo + 97])
+        still = S == 0
+        assert torch.equal(whole[2][:, still], start[2][:, still])
     dm.close()

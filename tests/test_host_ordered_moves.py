@@ -7,8 +7,8 @@ import numpy as np
 import pytest
 
 import host_cuda
-import paper_2504_02627_gb300 as g
 from paper_2504_02627_gb300 import _binding as B
+from test_gpu_ordered_moves import D, ORDERED
 
 
 @pytest.fixture(scope="module")
@@ -16,7 +16,7 @@ def lib(tmp_path_factory):
     return host_cuda.load(tmp_path_factory.mktemp("host_cuda"))
 
 
-def _model(lib, D=100):
+def _model(lib):
     md = B.ModelData(B.GAUSS_DENSE, D, mu=np.zeros(D), prec=np.eye(D))
     m = C.c_void_p()
     assert lib.smc_model_create(C.byref(m), C.byref(md.struct), None) == 0
@@ -57,4 +57,12 @@ def test_a_move_without_the_room_runs_in_the_particles_order(lib):
     assert not _ordered(lib, m, 32)               # a replay could overlap later calls
     lib.host_cuda_capture(0)
     assert lib.host_cuda_last_error() == 0        # the busy event is no error of the caller's
+    lib.smc_model_destroy(m)
+
+
+@pytest.mark.parametrize("n,precision", ORDERED)
+def test_the_gpu_tests_cases_are_ordered(lib, n, precision):
+    m = _model(lib)
+    assert _ordered(lib, m, 16, n, precision)
+    assert not _ordered(lib, m, 16, 97, precision)
     lib.smc_model_destroy(m)
