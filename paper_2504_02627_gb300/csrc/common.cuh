@@ -7,6 +7,7 @@
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
+#include "pairs.cuh"
 
 namespace smc {
 
@@ -284,67 +285,10 @@ __device__ __forceinline__ double from_order_key(long long k) {
 // the value is the same bit for bit).
 __device__ __forceinline__ float softplus(float x) { return (x > 0.0f ? x : 0.0f) + log1pf(expf(-fabsf(x))); }
 
-// ---------------------------------------------------------------- FP32 pairs
-// An unevaluated pair hi + lo of FP32 values carries about 48 significant
-// bits.  Sums use Knuth's TwoSum and products the FMA form of Dekker's
-// TwoProduct (both error-free transformations); pair + pair follows the
-// accurate double-double addition of Hida, Li and Bailey.  On this GPU FP64
-// runs at about 1/64 of the FP32 rate, so the statistics kernels accumulate
-// in pairs and convert to FP64 once per partial sum.
-struct f2sum {
-    float hi, lo;
-};
-__device__ __forceinline__ f2sum two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-__device__ __forceinline__ f2sum quick_two_sum(float a, float b) {   // needs |a| >= |b| or a = 0
-    const float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ f2sum f2_add(f2sum x, f2sum y) {
-    f2sum s = two_sum(x.hi, y.hi);
-    const f2sum t = two_sum(x.lo, y.lo);
-    s = quick_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
-    return quick_two_sum(s.hi, __fadd_rn(s.lo, t.lo));
-}
-__device__ __forceinline__ f2sum f2_add_f(f2sum x, float y) {
-    const f2sum s = two_sum(x.hi, y);
-    return quick_two_sum(s.hi, __fadd_rn(s.lo, x.lo));
-}
-__device__ __forceinline__ f2sum f2_mul(f2sum x, f2sum y) {           // lo * lo dropped
-    const float p = __fmul_rn(x.hi, y.hi);
-    const float e = __fmaf_rn(x.hi, y.hi, -p);                          // exact error of p
-    return quick_two_sum(p, __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, e)));
-}
-// s += x y: the product's error joins the running error terms, which are added
-// in FP32 (the compensated dot product of Ogita, Rump and Oishi: as accurate as
-// if summed in twice FP32's precision, 12 operations instead of 27).
-__device__ __forceinline__ void f2_dot(f2sum& s, f2sum x, f2sum y) {
-    const float p = __fmul_rn(x.hi, y.hi);
-    const float e = __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, __fmaf_rn(x.hi, y.hi, -p)));
-    const f2sum t = two_sum(s.hi, p);
-    s.hi = t.hi;
-    s.lo = __fadd_rn(s.lo, __fadd_rn(t.lo, e));
-}
-__device__ __forceinline__ double f2_to_double(f2sum x) { return (double)x.hi + (double)x.lo; }
-__device__ __forceinline__ f2sum f2_from_double(double v) {
-    const float hi = __double2float_rn(v);
-    return {hi, __double2float_rn(v - (double)hi)};
-}
-// butterfly sum over the warp (pair addition is commutative bit for bit)
-__device__ __forceinline__ f2sum warp_sum_f2(f2sum v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const f2sum w{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-        v = f2_add(v, w);
-    }
-    return v;
-}
-
-// Four such sums at once, value (lane >> 3) & 3 on return, by a reduce-scatter
-// over the first two levels: the same pairs are added, 6 additions instead of 20.
+// ---------------------------------------------------------------- FP32 pairs (pairs.cuh) over a warp
+// Four sums over the warp at once, value (lane >> 3) & 3 on return: a
+// reduce-scatter over the first two levels, then a butterfly (pair addition is
+// commutative bit for bit); 6 additions instead of 20.
 __device__ __forceinline__ f2sum warp_sum4_f2(f2sum (&v)[4], int lane) {
 #pragma unroll
     for (int h = 2; h >= 1; h >>= 1) {

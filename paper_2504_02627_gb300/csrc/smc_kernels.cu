@@ -798,8 +798,8 @@ __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
             const int64_t j0 = b.chees0 ? x.j : src;
             const float* t0 = b.chees0 ? b.chees0 : b.theta_prev;
             const float* t1 = b.chees1 ? b.chees1 : b.theta_new;
-            // |t - mean|^2 and the projection accumulated in FP32 pairs
-            f2sum sq0{0.0f, 0.0f}, sq1{0.0f, 0.0f}, proj{0.0f, 0.0f};
+            // |t - mean|^2 and the projection, sums of products of FP32 pairs
+            f2dot sq0{0.0f, 0.0f, 0.0f}, sq1{0.0f, 0.0f, 0.0f}, proj{0.0f, 0.0f, 0.0f};
             constexpr int BD = 8;
             for (int d0 = 0; d0 < D; d0 += BD) {
                 float v0[BD], v1[BD], vp[BD];
