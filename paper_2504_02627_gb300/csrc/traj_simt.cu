@@ -56,7 +56,7 @@ __device__ __forceinline__ float glm_loglik_term(float y, float eta, float inv_s
 template <int DP, int G, bool LOGIT, int PP = 1, int NT = GLM_THREADS, int DR = DP>
 __global__ void __launch_bounds__(NT, 1) traj_glm_kernel(DevModel m, TrajArgs a) {
     constexpr int NW = NT / 32, PG = G / PP, SL = NT / PG;
-    static_assert(G <= 32 && (32 % G) == 0 && DP <= 32 && NW <= 32, "G must divide 32; a lane per dimension and per warp");
+    static_assert(G <= 32 && (32 % G) == 0 && NW >= 3, "G must divide 32; three warps for the end point's sums");
     static_assert(PG * PP == G && DR <= DP, "PP must divide G; DR <= DP");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = m.n, D = m.D;
@@ -68,8 +68,8 @@ __global__ void __launch_bounds__(NT, 1) traj_glm_kernel(DevModel m, TrajArgs a)
     float* g_s = p_s + DP * G;
     float* red = g_s + DP * G;
     double* H0_s = reinterpret_cast<double*>(red + NW * DP * G);
-    double* lp_s = H0_s + G;
-    double* red64 = lp_s + G;
+    double* ll_s = H0_s + G;
+    double* red64 = ll_s + G;
     int* S_s = reinterpret_cast<int*>(red64 + NW * G);
     int* smax_s = S_s + G;
 
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(NT, 1) traj_glm_kernel(DevModel m, TrajArgs a)
     const int64_t slot0 = (int64_t)blockIdx.x * G;
     __shared__ int64_t j_s[G], src_s[G];
     __shared__ float eps_s[G];
-    __shared__ double kin_s[G];
+    __shared__ double end_s[2][G];   // |theta|^2, |p|^2
     __shared__ uint64_t seed_s[G];
     __shared__ uint32_t k_s[G], jl_s[G];
     if (tid < G) {
@@ -155,16 +155,18 @@ __global__ void __launch_bounds__(NT, 1) traj_glm_kernel(DevModel m, TrajArgs a)
         }
         __syncthreads();
     }
-    // FP64 sums over the dimensions, here and at the end: a warp per particle, a
-    // dimension per lane, then a fixed tree (an FP64 instruction takes a warp 64
-    // clocks: by one thread per particle the move of 4096 particles, n = 1000, D = 25
-    // took 323 us, so 319)
-    if (!a.eval_only)
-        for (int q = wid; q < G; q += NW) {
-            const double v = lane < D ? widen(p_s[lane * G + q]) : 0.0;
-            const double kin = warp_sum(v * v);
-            if (lane == 0) H0_s[q] = j_s[q] >= 0 ? 0.5 * kin - a.logpi_in[src_s[q]] : 0.0;
+    // FP64 sums over the dimensions, here and at the end: a lane per particle, and
+    // a warp (of another scheduler) for each sum, since an FP64 instruction takes
+    // its warp 64 clocks.  By trees over the lanes, a warp per particle, they took
+    // the small regressions 4 of 21 us (n = 100, D = 3, 15 steps).
+    if (!a.eval_only && tid < G) {
+        double kin = 0.0;
+        for (int d = 0; d < D; ++d) {
+            const double v = widen(p_s[d * G + tid]);
+            kin += v * v;
         }
+        H0_s[tid] = j_s[tid] >= 0 ? 0.5 * kin - a.logpi_in[src_s[tid]] : 0.0;
+    }
     __syncthreads();   // H0 reads p_s before the first half kick below rewrites it
     const int smax = *smax_s;
 
@@ -301,15 +303,17 @@ __global__ void __launch_bounds__(NT, 1) traj_glm_kernel(DevModel m, TrajArgs a)
 #pragma unroll
             for (int k = 0; k < PP; ++k) red64[wid * G + pl + k * PG] = ll[k];
         __syncthreads();
-        for (int q = wid; q < G; q += NW) {
-            // the slices' sums and the prior, the kinetic energy beside it
-            const double s = warp_sum(lane < NW ? red64[lane * G + q] : 0.0);
-            const double v = lane < D ? widen(th_s[lane * G + q]) : 0.0, p = lane < D ? widen(p_s[lane * G + q]) : 0.0;
-            const double sq = warp_sum(v * v), kin = warp_sum(p * p);
-            if (lane == 0) {
-                lp_s[q] = s - 0.5 * sq * inv_tau2_d + m.lconst;
-                kin_s[q] = kin;
-            }
+        if (lane < G && wid < 3) {
+            // the slices' sums; the prior; the kinetic energy
+            double s = 0.0;
+            if (wid == 0)
+                for (int w = 0; w < NW; ++w) s += red64[w * G + lane];
+            else if (wid == 1 || !a.eval_only)
+                for (int d = 0; d < D; ++d) {
+                    const double v = widen((wid == 1 ? th_s : p_s)[d * G + lane]);
+                    s += v * v;
+                }
+            (wid == 0 ? ll_s : end_s[wid - 1])[lane] = s;
         }
         __syncthreads();
     }
@@ -325,10 +329,10 @@ __global__ void __launch_bounds__(NT, 1) traj_glm_kernel(DevModel m, TrajArgs a)
     }
     if (tid < G && j_s[tid] >= 0) {
         const int64_t j = j_s[tid];
-        const double lp1 = lp_s[tid];
+        const double lp1 = ll_s[tid] - 0.5 * end_s[0][tid] * inv_tau2_d + m.lconst;
         a.logpi_out[j] = lp1;
         if (!a.eval_only) {
-            double dH = (0.5 * kin_s[tid] - lp1) - H0_s[tid];
+            double dH = (0.5 * end_s[1][tid] - lp1) - H0_s[tid];
             if (!isfinite(dH)) dH = CUDART_INF;
             if (a.dH) a.dH[j] = dH;
             if (a.alpha) a.alpha[j] = dH <= 0.0 ? 1.0 : exp(-dH);
