@@ -186,6 +186,16 @@ __global__ void __launch_bounds__(32 * KS, gg_ctas(KS)) traj_gauss_mma_kernel(De
                 pp[u][e] = pv;
             }
         }
+    // a trajectory without steps keeps its gradient (the steps of those beside it
+    // overwrite the registers)
+    if (!a.eval_only && (S[0] == 0 || S[1] == 0))
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int d = 16 * wid + 8 * u + 2 * tq + (e & 1);
+                if (S[e >> 1] == 0 && jq[e >> 1] >= 0 && d < D) a.grad_out[(int64_t)d * a.ld + jq[e >> 1]] = gr[u][e];
+            }
     if (!a.p_in && !a.eval_only) {
         // momentum p ~ N(0, I) from the (seed, i, j, k, MOM) Philox stream: this
         // thread's dimensions 2 i, 2 i + 1 are one pair, i = 8 wid + 4 u + tq
@@ -280,8 +290,7 @@ __global__ void __launch_bounds__(32 * KS, gg_ctas(KS)) traj_gauss_mma_kernel(De
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
-            for (int e = 0; e < 4; ++e)   // a trajectory without steps keeps its gradient
-                if (a.eval_only || s <= S[e >> 1]) gr[u][e] = -(acc[u][e] + cor[u][e]);
+            for (int e = 0; e < 4; ++e) gr[u][e] = -(acc[u][e] + cor[u][e]);
         // ---- closing half kick of step s; opening kick + drift of step s + 1
         //      and its A operand into the other buffer (its readers, step
         //      s - 1, finished at the previous barrier)
@@ -406,7 +415,7 @@ __global__ void __launch_bounds__(32 * KS, gg_ctas(KS)) traj_gauss_mma_kernel(De
             const int64_t j = jq[e >> 1];
             if (j < 0 || d >= D) continue;
             if (!a.eval_only) a.theta_out[(int64_t)d * a.ld + j] = th[u][e];
-            a.grad_out[(int64_t)d * a.ld + j] = gr[u][e];
+            if (a.eval_only || S[e >> 1] > 0) a.grad_out[(int64_t)d * a.ld + j] = gr[u][e];
             if (a.p_out && !a.eval_only) a.p_out[(int64_t)d * a.ld + j] = pp[u][e];
         }
 }
