@@ -16,7 +16,9 @@
 // of P per thread in registers and loading the deviations as broadcasts feeds one
 // (the same 10.6 us); 8 x 8 feeds four but leaves one warp a scheduler with
 // nothing to hide its chains behind (12.5 us).  The 8 x 4 tile here: 20 steps of
-// 8192 particles at D = 100 in 169 instead of 221 us, with the caller's copies.
+// 8192 particles at D = 100 in 158 instead of 221 us, with the caller's copies (170 with the
+// FP64 sums as trees over a warp per particle).
+#include <algorithm>
 #include <type_traits>
 #include <math_constants.h>
 #include "tc_ptx.cuh"
@@ -26,6 +28,7 @@ namespace smc {
 namespace {
 
 constexpr int DENSE_MAX_THREADS = 256;   // 16 row groups x 16 particle groups
+constexpr int DENSE_SHARES = 8;          // parts of an FP64 sum over the dimensions
 
 // Shared memory, in floats: P^T [D][RP] (RP = rows padded to the tile), deviations
 // [2][D][G], theta [RP][G], the final gradients [RP][G].
@@ -50,7 +53,7 @@ __global__ void __launch_bounds__(DENSE_MAX_THREADS) traj_dense_kernel(DevModel 
     constexpr int NPG = G / PT, PV = PT < 4 ? PT : 4;     // particle groups; particles per vector access
     static_assert(RT % 4 == 0 && (PT == 2 || PT % 4 == 0), "vector accesses");
     extern __shared__ __align__(16) float sm[];
-    const int D = m.D, NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = NT >> 5;
+    const int D = m.D, NT = blockDim.x, tid = threadIdx.x;
     const DenseLayout L(D, RT, G);
     const int RP = L.rp, NRG = L.nrg;
     float* const Pt = sm;
@@ -62,7 +65,7 @@ __global__ void __launch_bounds__(DENSE_MAX_THREADS) traj_dense_kernel(DevModel 
     __shared__ float eps_s[G];
     __shared__ uint64_t seed_s[G];
     __shared__ uint32_t k_s[G], jl_s[G];
-    __shared__ double e_s[3][G];
+    __shared__ double part_s[3][DENSE_SHARES][G], e_s[3][G];   // |p_0|^2, (theta - mu)' grad, |p|^2
 
     for (int e = tid; e < D * RP; e += NT) {
         const int r = e / D, k = e - r * D;               // reads of a row of P
@@ -129,17 +132,20 @@ __global__ void __launch_bounds__(DENSE_MAX_THREADS) traj_dense_kernel(DevModel 
         }
     }
     __syncthreads();
-    // FP64 sums over the dimensions, here and at the end: a warp per particle,
-    // each lane its dimensions in order, then a fixed tree
-    for (int q = wid; q < G; q += nw) {
-        double kin = 0.0;
-        for (int d = lane; d < D; d += 32) {
-            const double v = widen(p_st[d * G + q]);
-            kin += v * v;
+    // FP64 sums over the dimensions, here and at the end: a lane per particle and
+    // share of the dimensions, so that no lane idles and no tree is needed (an FP64
+    // instruction takes its warp 64 clocks whatever the lanes do); the shares are
+    // added in order.  Not unrolled: that cost the step loop 14 registers and 15%
+    if (!a.eval_only)
+        for (int i = tid; i < DENSE_SHARES * G; i += NT) {
+            double kin = 0.0;
+#pragma unroll 1
+            for (int d = i / G; d < D; d += DENSE_SHARES) {
+                const double v = widen(p_st[d * G + i % G]);
+                kin += v * v;
+            }
+            part_s[0][i / G][i % G] = kin;
         }
-        kin = warp_sum(kin);
-        if (lane == 0) e_s[0][q] = kin;
-    }
     const int rg = tid / NPG, pg = tid % NPG;
     const bool on = rg < NRG;
     auto row = [&](int i) { return (i < 4 ? 4 * rg : 4 * NRG + 4 * rg - 4) + i; };
@@ -279,20 +285,26 @@ __global__ void __launch_bounds__(DENSE_MAX_THREADS) traj_dense_kernel(DevModel 
             for (int c = 0; c < PT; ++c)
                 if (row(i) < D) p_st[row(i) * G + part(c)] = p[i][c];
     __syncthreads();
-    for (int q = wid; q < G; q += nw) {
+    for (int i = tid; i < DENSE_SHARES * G; i += NT) {
+        const int q = i % G;
         double q2 = 0.0, kin = 0.0;
-        for (int d = lane; d < D; d += 32) {
-            const double dv = widen(th_s[d * G + q]) - widen(m.mu[d]);
-            q2 += dv * widen(g_s[d * G + q]);
+#pragma unroll 1
+        for (int d = i / G; d < D; d += DENSE_SHARES) {
+            q2 += (widen(th_s[d * G + q]) - widen(m.mu[d])) * widen(g_s[d * G + q]);
+            if (a.eval_only) continue;
             const double v = widen(p_st[d * G + q]);
             kin += v * v;
         }
-        q2 = warp_sum(q2);
-        kin = warp_sum(kin);
-        if (lane == 0) {
-            e_s[1][q] = q2;
-            e_s[2][q] = kin;
-        }
+        part_s[1][i / G][q] = q2;
+        part_s[2][i / G][q] = kin;
+    }
+    __syncthreads();
+    for (int i = tid; i < 3 * G; i += NT) {
+        double t = 0.0;
+        if (!a.eval_only || i / G == 1)
+#pragma unroll 1
+            for (int h = 0; h < DENSE_SHARES; ++h) t += part_s[i / G][h][i % G];
+        e_s[i / G][i % G] = t;
     }
     __syncthreads();
     for (int q = tid; q < G; q += NT) {
@@ -327,19 +339,29 @@ cudaError_t launch_dense(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const int64_t grid = (a.N + G - 1) / G;
     if (grid == 0) return cudaSuccess;
-    return launch_ordered(kern, grid, (L.nrg * (G / PT) + 31) / 32 * 32, sm, s, m, a);
+    // four warps at least: the product needs fewer for small tiles, what comes
+    // before and after it does not
+    return launch_ordered(kern, grid, std::max((L.nrg * (G / PT) + 31) / 32 * 32, 128), sm, s, m, a);
 }
 
 }  // namespace
 
-// The largest tile whose CTAs still reach most SMs: fewer particles take smaller
-// tiles, which load more per FMA but leave no SM idle (64 particles a CTA from
-// 96 such CTAs on, 32 from 96 of those, else 8).
+// From 96 CTAs of 64 particles on a large tile, where its threads fill the CTA:
+// 8 x 4 above 96 dimensions, 4 x 4 between 48 and 64.  Otherwise smaller tiles, which
+// load more per FMA but put more threads to work and leave no SM idle.  us for 15
+// steps in tiles of 8 x 4 x 64 particles / 4 x 4 x 64 / 4 x 2 x 16 / 4 x 2 x 8:
+//   D = 128, 16384 particles 284 / - / 340 / 476   3500 particles 149 / - / 102 / 139
+//   D = 100,  8192 particles 116 / - / 124 / 134   1500 particles 121 / - / 46 / 51
+//   D = 80,  16384 particles 209 / - / 132 / 170   3500 particles 108 / - / 50 / 49
+//   D = 64,  16384 particles 95 / 89 / 107 / 131   3500 particles 76 / 60 / 38 / 37
+//   D = 48,  16384 particles 75 / 62 / 58 / 81     3500 particles 62 / 50 / 28 / 27
 cudaError_t launch_traj_dense(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     if (m.D > 128) return cudaErrorInvalidValue;
-    if (a.N >= 64 * 96) return launch_dense<8, 4, 64>(m, a, s);
-    if (a.N >= 32 * 96) return launch_dense<8, 4, 32>(m, a, s);
-    return launch_dense<4, 2, 8>(m, a, s);
+    if (a.N >= 64 * 96) {
+        if (m.D > 96) return launch_dense<8, 4, 64>(m, a, s);
+        return m.D > 48 && m.D <= 64 ? launch_dense<4, 4, 64>(m, a, s) : launch_dense<4, 2, 16>(m, a, s);
+    }
+    return m.D > 64 && a.N >= 32 * 96 ? launch_dense<4, 2, 16>(m, a, s) : launch_dense<4, 2, 8>(m, a, s);
 }
 
 }  // namespace smc
