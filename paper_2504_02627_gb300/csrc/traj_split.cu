@@ -45,6 +45,12 @@ __device__ __forceinline__ void finish(const TrajArgs& a, int64_t j, double lp1,
 
 // ============================================================ banana
 // Banana pairs (Sec. 4, Rosenbrock): x_o ~ N(0, a), x_e ~ N(b (x_o^2 - a), 1).
+// Its constants come from the host: two FP64 divisions, in every warp of a kernel
+// that spreads a particle over warps, were half of a gradient evaluation (D = 2:
+// 6.2 us a call, D = 32, 100000 particles 37.2).
+struct BananaC {
+    float a, b, inva, half_inva;
+};
 __device__ __forceinline__ void banana_grad(float a, float b, float inva, float xo, float xe, float& g0, float& g1) {
     float u = xe - b * (xo * xo - a);
     g0 = -xo * inva + 2.0f * b * u * xo;
@@ -71,7 +77,7 @@ __device__ __forceinline__ float banana_term(float a, float b, float half_inva, 
 // 8192 particles, up to 100 steps 59.6 -> 38.9 us with the caller's copies (24
 // of them this kernel; a thread per particle filled 64 CTAs).
 template <int NPT>
-__global__ void __launch_bounds__(256) traj_banana_kernel(DevModel m, TrajArgs a, int pw) {
+__global__ void __launch_bounds__(256) traj_banana_kernel(DevModel m, TrajArgs a, BananaC c, int pw) {
     extern __shared__ __align__(16) float sm[];
     const int D = m.D, np = D / 2;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -82,7 +88,7 @@ __global__ void __launch_bounds__(256) traj_banana_kernel(DevModel m, TrajArgs a
     float* sp1 = sp0 + 32 * D;                              // [D][32] momenta after
     float* slp = sp1 + 32 * D;                              // [np][32] log pi terms
     double* se = reinterpret_cast<double*>(slp + 32 * np);   // [3][32] log pi, p'p before and after
-    const float fa = (float)m.h0, fb = (float)m.h1, inva = (float)(1.0 / m.h0), half_inva = (float)(0.5 / m.h0);
+    const float fa = c.a, fb = c.b, inva = c.inva, half_inva = c.half_inva;
     Slot x{};
     double lp0 = 0.0;
     // a group of one warp needs no other
@@ -178,7 +184,8 @@ cudaError_t launch_banana_n(const DevModel& m, const TrajArgs& a, int pw, int ng
         if (e != cudaSuccess) return e;
     }
     const int64_t grid = (a.N + 32 * ngrp - 1) / (32 * ngrp);
-    kern<<<(unsigned)grid, 32 * pw * ngrp, sm, s>>>(m, a, pw);
+    const BananaC c{(float)m.h0, (float)m.h1, (float)(1.0 / m.h0), (float)(0.5 / m.h0)};
+    kern<<<(unsigned)grid, 32 * pw * ngrp, sm, s>>>(m, a, c, pw);
     return cudaGetLastError();
 }
 
@@ -283,8 +290,7 @@ cudaError_t launch_rows(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-// The launch variants of the banana (the autotuner's; 0 for the stage-level
-// calls) differ in the slot groups per CTA only.
+// All launch plans of the banana are this one launch.
 cudaError_t launch_traj_banana(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     if (m.D > 64) return cudaErrorInvalidValue;
     const int np = m.D / 2;
@@ -293,7 +299,9 @@ cudaError_t launch_traj_banana(const DevModel& m, const TrajArgs& a, cudaStream_
     // two pairs per thread where one each would put more than four warps on a
     // scheduler (D = 16, 16384 particles, 30 steps: 12.5 us with one)
     if (np <= 2 * (pw / 2) && (a.N + 31) / 32 * pw > 152 * 4 * 4) pw /= 2;
-    const int ngrp = std::max(1, std::min(8 / pw, a.tile % 4 == 1 ? 2 : a.tile % 4 == 2 ? 4 : 8 / pw));
+    // CTAs of four warps where a particle's pairs take fewer: an FP64 sum per
+    // scheduler (eight warps: D = 2, 1500 particles, 15 steps 3.5 us, so 3.3)
+    const int ngrp = std::max(1, 4 / pw);
     switch ((np + pw - 1) / pw) {
         case 1: return launch_banana_n<1>(m, a, pw, ngrp, s);
         case 2: return launch_banana_n<2>(m, a, pw, ngrp, s);
