@@ -166,7 +166,7 @@ int32_t traj_tile_count(const DevModel& m, int32_t precision);
 // several threads per particle (traj_split.cu): the banana by pairs, the
 // dense Gaussian D <= 32 by rows where N particles alone do not fill the GPU
 cudaError_t launch_traj_banana(const DevModel& m, const TrajArgs& a, cudaStream_t s);
-bool gauss_rows_supported(const DevModel& m, int64_t N);
+bool gauss_rows_supported(const DevModel& m, const TrajArgs& a);
 cudaError_t launch_traj_gauss_rows(const DevModel& m, const TrajArgs& a, cudaStream_t s);
 // dense Gaussian 32 < D <= 128, FP32 (traj_dense.cu)
 cudaError_t launch_traj_dense(const DevModel& m, const TrajArgs& a, cudaStream_t s);

@@ -197,27 +197,76 @@ cudaError_t launch_banana_n(const DevModel& m, const TrajArgs& a, int pw, int ng
 // thread that holds the whole particle).  Bound by the step's chain (exchange
 // and one row's sum): the 10-d Gaussian's move of 256 particles, up to about 100
 // steps, takes 9 instead of 30.5 us.
+//
+// The FP64 sums of the end point (log pi, p'p before and after: FP32 terms, added
+// in the order of the dimensions) go to one warp of the CTA, a lane per particle
+// and sum: an FP64 instruction takes its warp 64 clocks however few of its lanes
+// need it (three lanes per particle in its own warp: D = 32, 8192 particles, 15
+// steps 27.6 us instead of 21.7, 256 particles 7.0 instead of 6.8).
 template <int G>
 __global__ void __launch_bounds__(128) traj_gauss_rows_kernel(DevModel m, TrajArgs a) {
     constexpr int PPC = 128 / G;                       // particles per CTA
-    __shared__ __align__(16) float dl_s[PPC][G];
+    __shared__ __align__(16) float P_s[G][G + 4], dl_s[PPC][G];
     __shared__ float p0_s[PPC][G], p1_s[PPC][G], q_s[PPC][G];
-    const int D = m.D, r = threadIdx.x % G, pi = threadIdx.x / G;
+    __shared__ double e_s[3][PPC], lp0_s[PPC];
+    __shared__ int64_t j_s[PPC];
+    const int D = m.D, tid = threadIdx.x, r = tid % G, pi = tid / G;
     const int64_t t = (int64_t)blockIdx.x * PPC + pi;
     // the lanes of one particle; all of them take every branch together
-    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << (G % 32)) - 1u) << ((threadIdx.x & 31) / G * G);
-    if (t >= a.N) return;
-    const bool in = r < D;
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << (G % 32)) - 1u) << ((tid & 31) / G * G);
+    const bool on = t < a.N, in = on && r < D;
+    // P once per CTA: a lane's row straight from global memory is a sector per
+    // lane and column
+    float pv[(G * G + 127) / 128];
+#pragma unroll
+    for (int k = 0; k < (G * G + 127) / 128; ++k) {
+        const int i = tid + 128 * k, row = i / G, c = i % G;
+        pv[k] = (row < D && c < D) ? m.P[row * D + c] : 0.0f;
+    }
+    Slot x{};
+    float mu = 0.0f, th = 0.0f, p = 0.0f, g = 0.0f;
+    if (on) {
+        x = slot_of(a, t);
+        if (r == 0) {
+            j_s[pi] = x.j;
+            lp0_s[pi] = a.eval_only ? 0.0 : a.logpi_in[x.src];
+        }
+    }
+    const int64_t o = (int64_t)r * a.ld;
+    if (in) {
+        mu = m.mu[r];
+        th = a.theta_in[o + x.src];
+        if (!a.eval_only) {
+            g = a.grad_in[o + x.src];
+            if (a.p_in) {
+                p = a.p_in[o + x.j];
+            } else {   // both lanes of a pair draw it
+                float z0, z1;
+                normal_pair_f32(x.seed, (uint32_t)(r >> 1), x.jl, x.kk, TAG_MOM, z0, z1);
+                p = (r & 1) ? z1 : z0;
+            }
+        }
+    } else {
+        dl_s[pi][r] = 0.0f;   // and stays zero
+    }
+#pragma unroll
+    for (int k = 0; k < (G * G + 127) / 128; ++k) {
+        const int i = tid + 128 * k;
+        if (G * G >= 128 || i < G * G) P_s[i / G][i % G] = pv[k];
+    }
+    __syncthreads();
     float P[G];
 #pragma unroll
-    for (int b = 0; b < G; ++b) P[b] = (in && b < D) ? m.P[r * D + b] : 0.0f;
-    const float mu = in ? m.mu[r] : 0.0f;
-    const Slot x = slot_of(a, t);
-    const int64_t o = (int64_t)r * a.ld;
-    float th = in ? a.theta_in[o + x.src] : 0.0f, p = 0.0f, g = 0.0f;
+    for (int b = 0; b < G; b += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(&P_s[r][b]);
+        P[b] = v.x;
+        P[b + 1] = v.y;
+        P[b + 2] = v.z;
+        P[b + 3] = v.w;
+    }
     // grad log pi = -P (theta - mu), this lane's row
     auto grad = [&]() {
-        dl_s[pi][r] = th - mu;
+        if (in) dl_s[pi][r] = th - mu;
         __syncwarp(gmask);
         float acc = 0.0f;
 #pragma unroll
@@ -233,53 +282,45 @@ __global__ void __launch_bounds__(128) traj_gauss_rows_kernel(DevModel m, TrajAr
         __syncwarp(gmask);
         return -acc;
     };
-    if (a.eval_only) {
-        g = grad();
-    } else {
+    if (on) {
+        if (a.eval_only) {
+            g = grad();
+        } else {
+            p0_s[pi][r] = p;
+            const float ef = (float)x.eps, he = (float)(0.5 * x.eps);
+            for (int s = 0; s < x.S; ++s) {
+                p = fmaf(he, g, p);
+                th = fmaf(ef, p, th);
+                g = grad();
+                p = fmaf(he, g, p);
+            }
+            p1_s[pi][r] = p;
+        }
+        q_s[pi][r] = (th - mu) * g;
         if (in) {
-            g = a.grad_in[o + x.src];
-            if (a.p_in) {
-                p = a.p_in[o + x.j];
-            } else {   // both lanes of a pair draw it
-                float z0, z1;
-                normal_pair_f32(x.seed, (uint32_t)(r >> 1), x.jl, x.kk, TAG_MOM, z0, z1);
-                p = (r & 1) ? z1 : z0;
+            a.grad_out[o + x.j] = g;
+            if (!a.eval_only) {
+                a.theta_out[o + x.j] = th;
+                if (a.p_out) a.p_out[o + x.j] = p;
             }
         }
-        p0_s[pi][r] = p;
-        const float ef = (float)x.eps, he = (float)(0.5 * x.eps);
-        for (int s = 0; s < x.S; ++s) {
-            p = fmaf(he, g, p);
-            th = fmaf(ef, p, th);
-            g = grad();
-            p = fmaf(he, g, p);
-        }
-        p1_s[pi][r] = p;
     }
-    q_s[pi][r] = (th - mu) * g;
-    if (in) {
-        a.grad_out[o + x.j] = g;
-        if (!a.eval_only) {
-            a.theta_out[o + x.j] = th;
-            if (a.p_out) a.p_out[o + x.j] = p;
-        }
-    }
-    __syncwarp(gmask);
-    // log pi = c + 1/2 (theta - mu)' g: FP32 products, FP64 accumulation in
-    // the order of the dimensions, as are the kinetic energies; lanes 0, 1 and
-    // 2 take one of the three sums each, in the same instructions
-    double sum = 0.0;
-    if (r < 3 && (r == 0 || !a.eval_only)) {
-        const float* v = r == 0 ? q_s[pi] : r == 1 ? p0_s[pi] : p1_s[pi];
+    __syncthreads();
+    // log pi = c + 1/2 (theta - mu)' g
+    const int e = tid / PPC, k = tid % PPC;
+    if (e < (a.eval_only ? 1 : 3)) {
+        const float* v = e == 0 ? q_s[k] : e == 1 ? p0_s[k] : p1_s[k];
+        double sum = 0.0;
         for (int d = 0; d < D; ++d) {
-            const double e = widen(v[d]);
-            sum = fma(e, r == 0 ? 1.0 : e, sum);
+            const double w = widen(v[d]);
+            sum = fma(w, e == 0 ? 1.0 : w, sum);
         }
+        e_s[e][k] = sum;
     }
-    const double kin0 = __shfl_sync(gmask, sum, 1, G), kin1 = __shfl_sync(gmask, sum, 2, G);
-    if (r != 0) return;
-    const double lp0 = a.eval_only ? 0.0 : a.logpi_in[x.src];
-    finish(a, x.j, m.lconst + 0.5 * sum, 0.5 * kin0 - lp0, kin1);
+    __syncthreads();
+    if (tid < PPC && (int64_t)blockIdx.x * PPC + tid < a.N)
+        finish(a, j_s[tid], m.lconst + 0.5 * e_s[0][tid], a.eval_only ? 0.0 : 0.5 * e_s[1][tid] - lp0_s[tid],
+               a.eval_only ? 0.0 : e_s[2][tid]);
 }
 
 template <int G>
@@ -310,12 +351,19 @@ cudaError_t launch_traj_banana(const DevModel& m, const TrajArgs& a, cudaStream_
     }
 }
 
-bool gauss_rows_supported(const DevModel& m, int64_t N) {
-    // up to a few warps per scheduler in all (1245184 rows); beyond that the GPU
-    // is full with a particle per thread, which needs fewer instructions for
-    // each (no exchange, no idle lanes).  Below five dimensions there is
-    // nothing to split.
-    return m.kind == GAUSS_DENSE && m.D > 4 && m.D <= 32 && N * m.D <= (int64_t)152 * 2048 * 4;
+// A particle per thread needs fewer instructions for each (no exchange, no idle
+// lanes), but its chain is long and its launch starts late: where N particles
+// leave most of the GPU idle the rows are faster.  us by rows / by particles, 15
+// steps: D = 8, 8192 particles 4.8 / 9.3, 32768 9.4 / 10.2, 65536 14.5 / 13.0; D = 16,
+// 16384 13.0 / 21.0, 32768 22.0 / 22.7, 65536 39.8 / 29.9; D = 32, 16384 39 / 89, 65536
+// 138 / 192 (one step: 27.6 / 17.3 and 92 / 38).  Gradients alone cross at 131072
+// lanes: D = 8, 16384 particles 3.0 / 3.0, D = 16, 8192 4.0 / 4.2, D = 32, 8192 10.7 / 7.6.
+// Below five dimensions there is nothing to split.
+bool gauss_rows_supported(const DevModel& m, const TrajArgs& a) {
+    if (m.kind != GAUSS_DENSE || m.D <= 4 || m.D > 32) return false;
+    const int64_t lanes = m.D <= 8 ? 8 : m.D <= 16 ? 16 : 32;
+    if (a.eval_only) return a.N * lanes <= 131072;
+    return m.D <= 16 ? a.N <= 32768 : a.N * m.D <= 1245184;
 }
 
 cudaError_t launch_traj_gauss_rows(const DevModel& m, const TrajArgs& a, cudaStream_t s) {

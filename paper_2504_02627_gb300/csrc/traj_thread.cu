@@ -374,7 +374,7 @@ cudaError_t launch_traj_thread(const DevModel& m, const TrajArgs& a, cudaStream_
     switch (m.kind) {
         case GAUSS_DENSE:
             if (m.D > 32) return cudaErrorInvalidValue;
-            return a.tile == 0 && gauss_rows_supported(m, a.N) ? launch_traj_gauss_rows(m, a, s)
+            return a.tile == 0 && gauss_rows_supported(m, a) ? launch_traj_gauss_rows(m, a, s)
                                                                : dispatch_thread<GaussDenseM>(m, a, s);
         case BANANA: return launch_traj_banana(m, a, s);
         case HIER_NORMAL: return dispatch_thread_wide<HierM>(m, a, s);

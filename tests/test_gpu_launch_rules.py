@@ -33,3 +33,31 @@ def _check(dm, D, n, larger, eps):
 def test_dense_gaussian_tiles(D):
     need_gpu()
     _check(_gauss(D), D, 61, (3071, 3072, 6143, 6144, 6205), 0.02)
+
+
+@pytest.mark.parametrize("D", [5, 7, 8, 9, 15, 16, 17, 31, 32])
+def test_gaussian_rows_and_particles(D):
+    """Moves: 32768 particles up to 16 dimensions, else 1245184 values; gradients
+    alone: 131072 lanes."""
+    need_gpu()
+    lanes = 8 if D <= 8 else 16 if D <= 16 else 32
+    move = 32768 if D <= 16 else 1245184 // D
+    _check(_gauss(D), D, 301, (131072 // lanes, 131072 // lanes + 1, move, move + 1), 0.02)
+
+
+def test_rows_of_a_diverged_particle():
+    """Deviations that overflow stay infinite where the row sums do: the lanes past
+    D add nothing to them (5 of 8 lanes; all elements of P positive)."""
+    need_gpu()
+    D = 5
+    mu = np.zeros(D)
+    mu[0] = -3e38
+    dm = B.DevModel(B.ModelData(B.GAUSS_DENSE, D, mu=mu, prec=0.5 * np.eye(D) + 0.5), stream())
+    th = torch.zeros(D, 1, device="cuda")
+    th[0] = 3e38                                   # the deviation is infinite, the position is not
+    p, gr, lp = torch.zeros_like(th), torch.zeros_like(th), torch.zeros(1, dtype=torch.float64, device="cuda")
+    S = dev(np.array([2], np.int32))
+    B.check(B.lib().smc_k_leapfrog(dm.h, ptr(th), ptr(p), ptr(gr), ptr(lp), ptr(S), 0.1, 1, 1, 0, stream()), "leapfrog")
+    torch.cuda.synchronize()
+    assert torch.all(th == -np.inf) and torch.all(gr == np.inf)
+    dm.close()
