@@ -26,7 +26,8 @@ template <int DM>
 struct GaussDenseM {
     static constexpr bool ENERGY_FROM_GRAD = true;
     static constexpr int CTAS = DM > 16 ? 3 : 4;   // resident CTAs of 128 that the registers are capped for
-    static constexpr int LD = (DM + 3) / 4 * 4;    // row stride of P in shared memory
+    static constexpr int VW = DM <= 2 ? 2 : 4;     // elements of P per shared load
+    static constexpr int LD = (DM + VW - 1) / VW * VW;   // row stride of P in shared memory
     static size_t smem_bytes(const DevModel&) { return (size_t)(DM * LD + LD) * sizeof(float); }
     __device__ static void load(const DevModel& m, float* sm) {
         for (int i = threadIdx.x; i < DM * LD; i += blockDim.x) {
@@ -36,7 +37,9 @@ struct GaussDenseM {
         for (int i = threadIdx.x; i < LD; i += blockDim.x) sm[DM * LD + i] = i < m.D ? m.mu[i] : 0.0f;
     }
     // grad log pi = -P (theta - mu); a row's sum runs over the padded width
-    // (zero times zero adds nothing), four elements of P per shared load
+    // (zero times zero adds nothing), VW elements of P per shared load.  Up to
+    // four dimensions the rows past D run too: a branch per row costs more
+    // (D = 2, 300 particles, up to 30 steps 6.8 us with it, 5.7 without)
     template <class F>
     __device__ static void grad_each(const DevModel& m, const float* sm, const float (&th)[DM], F&& f) {
         const float* mu = sm + DM * LD;
@@ -45,17 +48,23 @@ struct GaussDenseM {
         for (int d = 0; d < LD; ++d) dl[d] = d < DM ? th[d < DM ? d : 0] - mu[d] : 0.0f;
 #pragma unroll
         for (int a = 0; a < DM; ++a) {
-            if (a >= m.D) break;
+            if (DM > 4 && a >= m.D) break;
             float acc = 0.0f;
 #pragma unroll
-            for (int b = 0; b < LD; b += 4) {
-                const float4 v = *reinterpret_cast<const float4*>(sm + a * LD + b);
-                acc = fmaf(v.x, dl[b], acc);
-                acc = fmaf(v.y, dl[b + 1], acc);
-                acc = fmaf(v.z, dl[b + 2], acc);
-                acc = fmaf(v.w, dl[b + 3], acc);
+            for (int b = 0; b < LD; b += VW) {
+                if constexpr (VW == 2) {
+                    const float2 v = *reinterpret_cast<const float2*>(sm + a * LD + b);
+                    acc = fmaf(v.x, dl[b], acc);
+                    acc = fmaf(v.y, dl[b + 1], acc);
+                } else {
+                    const float4 v = *reinterpret_cast<const float4*>(sm + a * LD + b);
+                    acc = fmaf(v.x, dl[b], acc);
+                    acc = fmaf(v.y, dl[b + 1], acc);
+                    acc = fmaf(v.z, dl[b + 2], acc);
+                    acc = fmaf(v.w, dl[b + 3], acc);
+                }
             }
-            f(a, -acc);
+            if (DM > 4 || a < m.D) f(a, -acc);
         }
     }
     // log pi = c - 1/2 (theta - mu)' P (theta - mu) = c + 1/2 (theta - mu)' g
