@@ -26,6 +26,7 @@ template <int DM>
 struct GaussDenseM {
     static constexpr bool ENERGY_FROM_GRAD = true;
     static constexpr int CTAS = DM > 16 ? 3 : 4;   // resident CTAs of 128 that the registers are capped for
+    static constexpr int FEW = CTAS;               // the same in launches of two CTAs an SM at most
     static constexpr int VW = DM <= 2 ? 2 : 4;     // elements of P per shared load
     static constexpr int LD = (DM + VW - 1) / VW * VW;   // row stride of P in shared memory
     static size_t smem_bytes(const DevModel&) { return (size_t)(DM * LD + LD) * sizeof(float); }
@@ -85,6 +86,7 @@ template <int DM>
 struct HierM {
     static constexpr bool ENERGY_FROM_GRAD = false;
     static constexpr int CTAS = DM > 52 ? 3 : 4;   // resident CTAs of 128 that the registers are capped for
+    static constexpr int FEW = 2;                  // the same in launches of two CTAs an SM at most (no spills)
     // shared memory: (ybar_g, n_g / sigma^2) pairs for the gradient (one 8-byte
     // load per group), then n_g and the within-group sums of squares
     static size_t smem_bytes(const DevModel& m) { return (size_t)4 * m.n * sizeof(float); }
@@ -150,7 +152,8 @@ struct HierM {
 
 // The move of the particle in slot t (Algorithm 1 for its S_j steps, the
 // end-point energy and Delta H), the model's data already in shared memory.
-template <template <int> class MT, int DM>
+// ROOM: the registers hold a gradient beside theta and p.
+template <template <int> class MT, int DM, bool ROOM>
 __device__ __forceinline__ void particle_move(const DevModel& m, const TrajArgs& a, const float* sm, int64_t t) {
     using M = MT<DM>;
     const int64_t j = a.perm ? a.perm[t] : t;
@@ -189,6 +192,15 @@ __device__ __forceinline__ void particle_move(const DevModel& m, const TrajArgs&
             if (d + 1 < DM) p[d + 1] = d + 1 < D ? z1 : 0.0f;
         }
     }
+    // the cached gradient, GB loads in flight at a time (zeros past D, where p and
+    // theta are zero too); with room in the registers all of it, behind nothing
+    constexpr int GB = ROOM ? DM : 16;
+    float g[GB];
+    auto load_grad = [&](int d0) {
+#pragma unroll
+        for (int u = 0; u < GB; ++u) g[u] = d0 + u < D ? a.grad_in[(int64_t)(d0 + u) * a.ld + src] : 0.0f;
+    };
+    if (ROOM) load_grad(0);
     double kin0 = 0.0;
 #pragma unroll
     for (int d = 0; d < DM; ++d)
@@ -204,11 +216,15 @@ __device__ __forceinline__ void particle_move(const DevModel& m, const TrajArgs&
     if (S > 0) {
         // the first half kick and drift from the cached gradient
 #pragma unroll
-        for (int d = 0; d < DM; ++d)
-            if (d < D) {
-                p[d] = fmaf(he, a.grad_in[(int64_t)d * a.ld + src], p[d]);
-                th[d] = fmaf(ef, p[d], th[d]);
-            }
+        for (int d0 = 0; d0 < DM; d0 += GB) {
+            if (!ROOM) load_grad(d0);
+#pragma unroll
+            for (int u = 0; u < GB; ++u)
+                if (d0 + u < DM) {
+                    p[d0 + u] = fmaf(he, g[u], p[d0 + u]);
+                    th[d0 + u] = fmaf(ef, p[d0 + u], th[d0 + u]);
+                }
+        }
         // a step's gradient closes its kick, opens the next and drifts
         for (int s = 1; s < S; ++s)
             M::grad_each(m, sm, th, [&](int d, float g) {
@@ -259,7 +275,7 @@ __global__ void __launch_bounds__(NT, MINB) traj_thread_kernel(DevModel m, TrajA
     MT<DM>::load(m, sm);
     __syncthreads();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < a.N) particle_move<MT, DM>(m, a, sm, t);
+    if (t < a.N) particle_move<MT, DM, (NT * MINB <= 256)>(m, a, sm, t);
 }
 
 // Persistent form: as many CTAs as fit on the GPU at once, each loading the
@@ -278,12 +294,23 @@ __global__ void __launch_bounds__(NT, MINB) traj_thread_persist_kernel(DevModel 
         __syncthreads();   // every thread has the tile before the next one is taken
         if (tile >= ntiles) break;
         const int64_t t = tile * NT + threadIdx.x;
-        if (t < a.N) particle_move<MT, DM>(m, a, sm, t);
+        if (t < a.N) particle_move<MT, DM, (NT * MINB <= 256)>(m, a, sm, t);
     }
 }
 
 
 namespace {
+
+int sm_count() {
+    static int sms = 0;
+    if (sms == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+            sms = 1;
+    }
+    return sms;
+}
 
 template <template <int> class MT, int DM, int NT, int MINB>
 cudaError_t launch_thread_v(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
@@ -309,13 +336,7 @@ cudaError_t launch_thread_persist(const DevModel& m, const TrajArgs& a, cudaStre
     }
     const int64_t ntiles = (a.N + NT - 1) / NT;
     if (ntiles == 0) return cudaSuccess;
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-            sms = 1;
-    }
+    const int sms = sm_count();
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, sm);
     if (e != cudaSuccess) return e;
@@ -347,8 +368,13 @@ cudaError_t launch_thread(const DevModel& m, const TrajArgs& a, cudaStream_t s) 
             case 5: return launch_thread_persist<MT, DM, 64, 2 * C>(m, a, s);
             case 6: return launch_thread_persist<MT, DM, 256, 2>(m, a, s);
             case 7: return launch_thread_persist<MT, DM, 128, O>(m, a, s);
-            default: return launch_thread_v<MT, DM, 128, C>(m, a, s);
+            default: break;
         }
+        // while two CTAs an SM hold all particles, more registers for each beat more
+        // CTAs: 52-d hierarchical normal, 300 or 8192 particles, 15 steps 46 -> 41 us,
+        // one step 29 -> 25
+        return a.N <= 2 * 128 * (int64_t)sm_count() ? launch_thread_v<MT, DM, 128, MT<DM>::FEW>(m, a, s)
+                                                    : launch_thread_v<MT, DM, 128, C>(m, a, s);
     } else {
         return launch_thread_v<MT, DM, 128, 1>(m, a, s);
     }

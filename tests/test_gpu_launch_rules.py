@@ -45,6 +45,17 @@ def test_gaussian_rows_and_particles(D):
     _check(_gauss(D), D, 301, (131072 // lanes, 131072 // lanes + 1, move, move + 1), 0.02)
 
 
+@pytest.mark.parametrize("G", [15, 20, 32, 50, 51, 62])
+def test_hierarchical_normal_register_caps(G):
+    """Two CTAs of 128 particles an SM, and more."""
+    need_gpu()
+    rng = np.random.default_rng(G)
+    md = B.ModelData(B.HIER_NORMAL, G + 2, G, group_mean=rng.standard_normal(G), group_n=np.full(G, 20.0),
+                     group_ss=np.full(G, 19.0), hyper=(1.0,))
+    few = 2 * 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    _check(B.DevModel(md, stream()), G + 2, 301, (few, few + 1), 0.01)
+
+
 def test_rows_of_a_diverged_particle():
     """Deviations that overflow stay infinite where the row sums do: the lanes past
     D add nothing to them (5 of 8 lanes; all elements of P positive)."""
