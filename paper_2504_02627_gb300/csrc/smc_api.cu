@@ -1032,12 +1032,15 @@ static smc_status capture_two_steps(smc_handle* h) {
     cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(h, e, "smc_run capture");
     cudaStream_t user = h->stream;
+    const int cur = h->cur;
+    const int64_t done = h->iters_done;
     h->stream = s;
     smc_status st = smc_step(h, nullptr);
     if (st == SMC_OK) st = smc_step(h, nullptr);
     h->stream = user;
     e = cudaStreamEndCapture(s, &graph);
-    h->iters_done -= 2;   // captured, not executed
+    h->cur = cur;         // captured, not executed, whether one step or both
+    h->iters_done = done;
     if (st != SMC_OK) {
         if (graph) cudaGraphDestroy(graph);
         return st;

@@ -68,3 +68,18 @@ def test_a_step_that_never_began_may_be_tried_again(lib):
     assert lib.smc_run(h, 4, None) == 0
     assert host_cuda.launches(lib).count("graph") == 2
     lib.smc_destroy(h)
+
+
+def test_a_capture_that_failed_leaves_the_buffers_in_place(lib):
+    """The second of the two captured steps fails: the particles are still where
+    the last step that ran left them, and the next run starts from there."""
+    h = _handle(lib)
+    lib.host_cuda_fail(b"move_stats", host_cuda.NOMEM, 1)
+    assert lib.smc_run(h, 4, None) == host_cuda.E_NOMEM
+    lib.host_cuda_fail(b"", 0, 0)
+    host_cuda.launches(lib)
+    assert lib.smc_run(h, 4, None) == 0
+    names = host_cuda.launches(lib)
+    assert names.count("graph") == 2
+    assert sum("k_weights_steps" in n for n in names) == 2     # captured; none to align the buffers
+    lib.smc_destroy(h)
