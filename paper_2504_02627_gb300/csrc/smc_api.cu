@@ -90,9 +90,10 @@ struct CentredScratch {
 };
 
 // Room for the launch order of the stage-level moves on a model (smc_model_create
-// only; 1 MB).  Calls may come from several threads and streams: a call takes
-// the room when the last one that used it ran on the same stream or has
-// finished, and otherwise goes without (the order changes speed only).
+// only; 1 MB, where any of its moves is ordered).  Calls may come from several
+// threads and streams: a call takes the room when the last one that used it ran
+// on the same stream or has finished, and otherwise goes without (the order
+// changes speed only).
 struct OrderRoom {
     static constexpr int64_t CAP = 262144;   // particles
     int32_t* perm = nullptr;
@@ -1360,11 +1361,13 @@ smc_status smc_model_create(smc_dev_model** out, const smc_model* model, void* s
         delete m;
         return SMC_E_INVAL;
     }
-    if (cudaEventCreateWithFlags(&m->order.used, cudaEventDisableTiming) == cudaSuccess) {
+    bool ordered = false;   // at any size that the room serves
+    for (int32_t p : {SMC_PREC_FP32, SMC_PREC_BF16X3, SMC_PREC_BF16}) ordered |= order_pays(m->m, p, OrderRoom::CAP);
+    if (ordered && cudaEventCreateWithFlags(&m->order.used, cudaEventDisableTiming) == cudaSuccess) {
         m->order.perm = m->mem.get<int32_t>((size_t)OrderRoom::CAP);
         cudaStreamSynchronize(m->mem.s);   // calls on other streams may use it from now on
     }
-    if (!m->order.perm) (void)cudaGetLastError();   // moves then run in the particles' order
+    if (ordered && !m->order.perm) (void)cudaGetLastError();   // moves then run in the particles' order
     *out = m;
     return SMC_OK;
 }

@@ -26,6 +26,7 @@ struct Config {
     void* stream;
 };
 std::vector<Config> configs;
+long long allocated = 0;                       // bytes, over all calls
 
 cudaError_t ret(cudaError_t e) {
     if (e != cudaSuccess) last = e;
@@ -54,6 +55,7 @@ void host_cuda_foreign_capture(int on) {
     foreign_broken = false;
 }
 int host_cuda_foreign_capture_broken() { return foreign_broken; }
+long long host_cuda_allocated() { return allocated; }
 int host_cuda_mode() { return (int)mode; }
 int host_cuda_last_error() { return (int)last; }
 void host_cuda_capture(int on) { capturing = on != 0; }
@@ -106,7 +108,10 @@ cudaError_t cudaGetSymbolAddress(void** p, const void*) {
     static char room[65536];
     return *p = room, cudaSuccess;
 }
-cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return *p = calloc(1, n), cudaSuccess; }
+cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) {
+    allocated += (long long)n;
+    return *p = calloc(1, n), cudaSuccess;
+}
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return free(p), cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return memcpy(d, s, n), cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {

@@ -38,6 +38,7 @@ def load(folder):
         f = getattr(lib, name)
         f.restype, f.argtypes = res, args
     lib.host_cuda_launched.restype = C.c_char_p
+    lib.host_cuda_allocated.restype = C.c_longlong
     lib.host_cuda_fail.argtypes = [C.c_char_p, C.c_int, C.c_int]
     return lib
 

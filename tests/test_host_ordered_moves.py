@@ -66,3 +66,19 @@ def test_the_gpu_tests_cases_are_ordered(lib, n, precision):
     assert _ordered(lib, m, 16, n, precision)
     assert not _ordered(lib, m, 16, 97, precision)
     lib.smc_model_destroy(m)
+
+
+def test_only_models_whose_moves_are_ordered_keep_room_for_the_order(lib):
+    rng = np.random.default_rng(0)
+    def room(md):
+        m = C.c_void_p()
+        before = lib.host_cuda_allocated()
+        assert lib.smc_model_create(C.byref(m), C.byref(md.struct), None) == 0
+        lib.smc_model_destroy(m)
+        return lib.host_cuda_allocated() - before
+    gauss = lambda D: B.ModelData(B.GAUSS_DENSE, D, mu=np.zeros(D), prec=np.eye(D))
+    assert room(B.ModelData(B.BANANA, 50, hyper=(10.0, 0.1))) < 1 << 16
+    assert room(gauss(32)) < 1 << 16                  # never ordered, at any particle count
+    assert room(gauss(33)) > 1 << 20
+    assert room(B.ModelData(B.LOGISTIC, 25, 1000, X=rng.standard_normal((1000, 25)), y=np.zeros(1000),
+                            hyper=(1.0,))) > 1 << 20
