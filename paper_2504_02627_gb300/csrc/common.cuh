@@ -312,13 +312,6 @@ __device__ __forceinline__ T warp_sum(T v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-template <typename T>
-__device__ __forceinline__ T warp_max(T v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
 // Warp sums of 16 values per lane: on return each lane holds the total over
 // the 32 lanes of value (lane >> 1) & 15.  A reduce-scatter butterfly: at
 // each level a lane keeps half of its values and adds the partner's copy of

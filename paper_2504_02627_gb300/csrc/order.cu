@@ -12,7 +12,7 @@ constexpr int ORDER_CTAS = 8, ORDER_THREADS = 1024, ORDER_BINS = 512;
 // One cluster: every CTA takes a contiguous share of the particles; the range of
 // the counts, then per-bin counts, then each share's slots per bin go through
 // distributed shared memory.  Counts that span more than ORDER_BINS values
-// share bins (an order within a fiftieth of a warp's length is enough), and
+// share bins (an order within a five-hundredth of the range is enough), and
 // equal counts come in any order: no result depends on it.  The kernel that
 // reads the order may start at once (programmatic launch): it waits for this
 // one's end before it reads it, and by then has loaded the model's data.

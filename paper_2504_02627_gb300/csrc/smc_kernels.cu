@@ -628,12 +628,6 @@ __device__ __forceinline__ SliceIdx slice_idx(const StepBufs& b) {
     return x;
 }
 
-// (max, sum exp) pair of a block; returns (M, S) with S = sum exp(a - M).
-__device__ __forceinline__ void block_lse(double a, double* buf, double& M, double& S) {
-    M = block_reduce(a, buf, OpMax());
-    S = block_reduce(M > -CUDART_INF ? exp(a - M) : 0.0, buf, OpSum());
-}
-
 __global__ void __launch_bounds__(SLICE) k_move_stats(StepBufs b) {
     __shared__ double buf[5 * 32];
     __shared__ long long lbuf[2 * 32];
