@@ -749,8 +749,9 @@ __global__ void __launch_bounds__(SLICE) k_move_stats(StepBufs b) {
 // then the last slice of each run combines every slice in a fixed order:
 // evidence, log-weights' ESS, Adam ascent on log L, Lbar, the freeze at
 // M_warmup, statistics, and the weight decision of the next iteration.  One run of
-// 256 particles: 34 -> 13 us, nearly all of it the FP64 latency of the last
-// slice's chain; 64 hierarchical runs: 115 -> 88 us, the pair arithmetic.
+// 256 particles: 34 -> 20 us alone and cold, the FP64 latency of the last slice's
+// chain and the fetch of the unrolled sums; 64 hierarchical runs: 115 -> 103 us,
+// the pair arithmetic.
 __global__ void __launch_bounds__(SLICE) k_chees_finish(StepBufs b) {
     __shared__ double buf[7 * 32], tot_s[7], res_s[4];
     __shared__ long long lbuf[2 * 32];

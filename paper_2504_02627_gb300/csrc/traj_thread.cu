@@ -8,9 +8,11 @@
 // What bounds them is the FMA pipe and, before that, the registers: a
 // gradient component is used up as it is formed (it closes its dimension's
 // kick, opens the next one and drifts the position at once), so no gradient
-// array lives next to theta and p.  The 52-d hierarchical normal then fits
-// 128 registers, four CTAs an SM (223, or 168 with 2 KB of spills, before):
-// 64 runs, 278k particles, three iterations 8.73 -> 6.53 ms.
+// array lives next to theta and p during the steps.  The 52-d hierarchical normal
+// then runs four CTAs an SM on 128 registers with 324 bytes of spills (223
+// registers, or 168 with 2 KB of spills, before): 64 runs, 278k particles, three
+// iterations 8.73 -> 5.87 ms.  Launches of up to two CTAs an SM take 255 registers
+// and spill nothing.
 #include <algorithm>
 #include <cstdio>
 #include <math_constants.h>
