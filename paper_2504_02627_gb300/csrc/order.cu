@@ -93,22 +93,37 @@ cudaError_t launch_order_steps(const int32_t* steps, int64_t N, int32_t* perm, c
     return cudaGetLastError();
 }
 
-// Ordering pays where the particles of a tile share the longest trajectory and a
-// step of the launch takes about a microsecond or more (some 5e7 operations, 1e8
-// on the matrix units): below that the move is over in the time that ordering
-// takes.  Counts uniform on 1 .. S: the n = 1000, D = 25 regression, 4096 particles, S = 40, 617 ->
-// 326 us; the 100-d Gaussian in BF16x3, 8191 particles, S = 50, 150 -> 122 us, 6000
-// particles, S = 30, 69 -> 62 us (a move of 30 steps each: 70 -> 72); in 64
-// dimensions, 16384 particles, 69 -> 65 us (30 steps each 66 -> 68), in 40 as much
-// as it costs: left in the particles' order.
-// The centred and
-// the other tcgen05 kernels keep state at the particles' indices and read it
-// every step, coalesced only in the particles' own order.
+// Ordering pays where the particles of a tile share the longest trajectory, a step
+// of the launch takes about a microsecond or more (some 5e7 operations, 1e8 on
+// the matrix units; the move is over in the time that ordering takes below that)
+// and there are more tiles than SMs: otherwise the longest tile is the launch,
+// ordered or not, and only slower when all of its particles run on.  us in order
+// / in the particles' own order, counts uniform on 0 .. 30, then all 15:
+//   regression, n = 1000, D = 25, 16 particles a tile: 4096 particles 228 / 442, 242 / 237;
+//     1000 particles 228 / 222
+//   regression, n = 300, D = 64, 64 a tile: 12000 2620 / 3261; 4096 2366 / 2207
+//   Gaussian in FP32, D = 100: 5000 123 / 163, 97 / 93; 10000 199 / 360; 8192, 128 tiles of
+//     64, 199 / 183; D = 40, 20011 76 / 108, 68 / 63
+// On tensor cores a tile's 16 lanes gather their particles, which short moves
+// hardly repay: D = 80, 16384 particles in BF16x3, to 30 steps 84 / 84, to 100 158 / 228; in
+// BF16 70 / 62 and 111 / 135; D = 64 to 30 69 / 65, D = 40 as much as it costs.
+// The centred and the other tcgen05 kernels keep state at the particles' indices
+// and read it every step, coalesced only in the particles' own order.
 bool order_pays(const DevModel& m, int32_t precision, int64_t N) {
-    double per = 0.0;   // operations of one particle's gradient
-    if (m.kind == GAUSS_DENSE && m.D > (precision == 0 ? 32 : 64) && precision <= 2) per = 2.0 * m.D * m.D;
-    if ((m.kind == LOGISTIC || m.kind == LINEAR_GAUSS) && precision == 0) per = 4.0 * m.n * m.D;
-    return per * (double)N >= (precision == 0 ? 5e7 : 1e8);
+    const double n = (double)N;
+    if (m.kind == GAUSS_DENSE && (precision == 1 || precision == 2)) return m.D > 64 && 2.0 * m.D * m.D * n >= 1e8;
+    if (precision != 0) return false;
+    int64_t tile;
+    if (m.kind == GAUSS_DENSE && m.D > 32) {
+        if (2.0 * m.D * m.D * n < 5e7) return false;
+        tile = dense_tile(m, N);
+    } else if (m.kind == LOGISTIC || m.kind == LINEAR_GAUSS) {
+        if (4.0 * m.n * m.D * n < 5e7) return false;
+        tile = glm_tile(m);
+    } else {
+        return false;
+    }
+    return (N + tile - 1) / tile > sm_count();
 }
 
 }  // namespace smc

@@ -145,6 +145,10 @@ cudaError_t launch_ordered(K kern, int64_t grid, int block, size_t smem, cudaStr
     return cudaLaunchKernelEx(&c, kern, m, a);
 }
 
+int sm_count();                                              // of the device (traj_thread.cu)
+int64_t dense_tile(const DevModel& m, int64_t N);            // particles per CTA of traj_dense.cu
+int64_t glm_tile(const DevModel& m);                         // ... of the FP32 regressions
+constexpr int GLM_STREAM_TILE = 64;                          // ... with streamed data
 // order.cu: perm = the particles by descending steps (any order within a
 // five-hundredth of the counts' range), and where that is worth a launch
 cudaError_t launch_order_steps(const int32_t* steps, int64_t N, int32_t* perm, cudaStream_t s);

@@ -355,13 +355,18 @@ cudaError_t launch_dense(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
 //   D = 80,  16384 particles 209 / - / 132 / 170   3500 particles 108 / - / 50 / 49
 //   D = 64,  16384 particles 95 / 89 / 107 / 131   3500 particles 76 / 60 / 38 / 37
 //   D = 48,  16384 particles 75 / 62 / 58 / 81     3500 particles 62 / 50 / 28 / 27
+int64_t dense_tile(const DevModel& m, int64_t N) {
+    if (N >= 64 * 96) return m.D > 96 || (m.D > 48 && m.D <= 64) ? 64 : 16;
+    return m.D > 64 && N >= 32 * 96 ? 16 : 8;
+}
+
 cudaError_t launch_traj_dense(const DevModel& m, const TrajArgs& a, cudaStream_t s) {
     if (m.D > 128) return cudaErrorInvalidValue;
-    if (a.N >= 64 * 96) {
-        if (m.D > 96) return launch_dense<8, 4, 64>(m, a, s);
-        return m.D > 48 && m.D <= 64 ? launch_dense<4, 4, 64>(m, a, s) : launch_dense<4, 2, 16>(m, a, s);
+    switch (dense_tile(m, a.N)) {
+        case 64: return m.D > 96 ? launch_dense<8, 4, 64>(m, a, s) : launch_dense<4, 4, 64>(m, a, s);
+        case 16: return launch_dense<4, 2, 16>(m, a, s);
+        default: return launch_dense<4, 2, 8>(m, a, s);
     }
-    return m.D > 64 && a.N >= 32 * 96 ? launch_dense<4, 2, 16>(m, a, s) : launch_dense<4, 2, 8>(m, a, s);
 }
 
 }  // namespace smc

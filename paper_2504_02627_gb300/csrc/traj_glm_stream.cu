@@ -20,7 +20,7 @@
 namespace smc {
 namespace {
 
-constexpr int GS_P = 64;           // particles per CTA
+constexpr int GS_P = GLM_STREAM_TILE;   // particles per CTA
 constexpr int GS_T = 256;          // threads per CTA
 constexpr int GS_C = 64;           // observations per chunk
 

@@ -374,6 +374,8 @@ bool glm_shape_ok(const DevModel& m) {
 
 }  // namespace
 
+int64_t glm_tile(const DevModel& m) { return glm_shape_ok(m) ? 16 : GLM_STREAM_TILE; }
+
 bool traj_supported(const DevModel& m, int32_t precision) {
     if (precision == 1 || precision == 2) {
         if (m.kind == GAUSS_DENSE) return traj_gauss_mma_supported(m);

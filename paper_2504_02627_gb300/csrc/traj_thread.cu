@@ -301,8 +301,6 @@ __global__ void __launch_bounds__(NT, MINB) traj_thread_persist_kernel(DevModel 
 }
 
 
-namespace {
-
 int sm_count() {
     static int sms = 0;
     if (sms == 0) {
@@ -313,6 +311,8 @@ int sm_count() {
     }
     return sms;
 }
+
+namespace {
 
 template <template <int> class MT, int DM, int NT, int MINB>
 cudaError_t launch_thread_v(const DevModel& m, const TrajArgs& a, cudaStream_t s) {

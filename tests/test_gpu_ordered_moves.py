@@ -9,19 +9,21 @@ from paper_2504_02627_gb300 import _binding as B
 
 pytestmark = pytest.mark.gpu
 D, N = 100, 6007
-# particles and precision of dense Gaussians in D dimensions that are ordered
-# (test_host_ordered_moves.py holds them against the rule); 97 are not
-ORDERED = [(N, 0), (N, 1), (N, 2), (5003, 1), (16411, 2)]
+# (kind, dimensions, observations, particles, precision) of moves that are ordered
+# (test_host_ordered_moves.py holds them against the rule); 97 particles are not
+ORDERED = [("gauss", D, 0, N, 0), ("gauss", D, 0, 9800, 0), ("gauss", D, 0, N, 1), ("gauss", D, 0, N, 2),
+           ("gauss", 80, 0, 16411, 2), ("gauss", 40, 0, 20011, 0), ("logistic", 25, 1000, 2500, 0), ("logistic", 40, 64, 9800, 0)]
 
 
-def _gauss(s):
+def model(kind, D, n):
     rng = np.random.default_rng(D)
+    if kind == "logistic":
+        return B.ModelData(B.LOGISTIC, D, n, X=rng.standard_normal((n, D)), y=(rng.uniform(size=n) < 0.5), hyper=(1.0,))
     A = rng.standard_normal((D, D))
-    return B.DevModel(B.ModelData(B.GAUSS_DENSE, D, mu=rng.standard_normal(D), prec=A @ A.T / D + np.eye(D)),
-                      s.cuda_stream)
+    return B.ModelData(B.GAUSS_DENSE, D, mu=rng.standard_normal(D), prec=A @ A.T / D + np.eye(D))
 
 
-def _state(seed, n=N):
+def _state(seed, n=N, D=D):
     t = torch.Generator(device="cuda").manual_seed(seed)
     x = [torch.randn(D, n, device="cuda", generator=t) for _ in range(3)]
     return x + [torch.zeros(n, dtype=torch.float64, device="cuda")]
@@ -35,7 +37,7 @@ def _move(dm, x, S, s, precision=0):
 def test_moves_beside_captures_and_busy_streams():
     need_gpu()
     a, b, c = (torch.cuda.Stream() for _ in range(3))
-    dm = _gauss(a)
+    dm = B.DevModel(model("gauss", D, 0), a.cuda_stream)
     S = dev(np.random.default_rng(1).integers(0, 40, size=N).astype(np.int32))
     x = [[t.clone() for t in _state(2)] for _ in range(4)]
     big, S_big = _state(3, 262144), torch.full((262144,), 60, dtype=torch.int32, device="cuda")
@@ -76,15 +78,15 @@ def test_moves_beside_captures_and_busy_streams():
     dm.close()
 
 
-@pytest.mark.parametrize("n,precision", ORDERED)
-def test_ordered_moves_of_every_precision(n, precision):
+@pytest.mark.parametrize("kind,dim,obs,n,precision", ORDERED)
+def test_ordered_moves_of_every_kind(kind, dim, obs, n, precision):
     """Ragged, equal and zero step counts, against the same particles in
     launches of 97, which are not ordered.  The gradients are not those of the
     positions: a particle without steps keeps the one it came with."""
     need_gpu()
     s = torch.cuda.current_stream()
-    dm = _gauss(s)
-    start = _state(n, n)
+    dm = B.DevModel(model(kind, dim, obs), s.cuda_stream)
+    start = _state(n, n, dim)
     rng = np.random.default_rng(n)
     for counts in (rng.integers(0, 9, size=n), np.full(n, 3), rng.integers(0, 2000, size=n) // 400, np.zeros(n, int)):
         S = dev(counts.astype(np.int32))

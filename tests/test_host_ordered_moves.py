@@ -8,7 +8,7 @@ import pytest
 
 import host_cuda
 from paper_2504_02627_gb300 import _binding as B
-from test_gpu_ordered_moves import D, ORDERED
+from test_gpu_ordered_moves import D, ORDERED, model
 
 
 @pytest.fixture(scope="module")
@@ -16,8 +16,8 @@ def lib(tmp_path_factory):
     return host_cuda.load(tmp_path_factory.mktemp("host_cuda"))
 
 
-def _model(lib):
-    md = B.ModelData(B.GAUSS_DENSE, D, mu=np.zeros(D), prec=np.eye(D))
+def _model(lib, md=None):
+    md = md or model("gauss", D, 0)
     m = C.c_void_p()
     assert lib.smc_model_create(C.byref(m), C.byref(md.struct), None) == 0
     host_cuda.launches(lib)
@@ -60,11 +60,22 @@ def test_a_move_without_the_room_runs_in_the_particles_order(lib):
     lib.smc_model_destroy(m)
 
 
-@pytest.mark.parametrize("n,precision", ORDERED)
-def test_the_gpu_tests_cases_are_ordered(lib, n, precision):
-    m = _model(lib)
+@pytest.mark.parametrize("kind,dim,obs,n,precision", ORDERED)
+def test_the_gpu_tests_cases_are_ordered(lib, kind, dim, obs, n, precision):
+    m = _model(lib, model(kind, dim, obs))
     assert _ordered(lib, m, 16, n, precision)
     assert not _ordered(lib, m, 16, 97, precision)
+    lib.smc_model_destroy(m)
+
+
+@pytest.mark.parametrize("kind,dim,obs,n,precision", [
+    ("gauss", 100, 0, 8192, 0), ("gauss", 64, 0, 9728, 0),                      # 152 tiles of 64 at most
+    ("logistic", 25, 1000, 2432, 0), ("logistic", 64, 300, 4096, 0),            # of 16, of 64 (streamed)
+    ("gauss", 64, 0, 40000, 1), ("gauss", 32, 0, 30000, 0),                      # the gather costs what it saves; no tiles
+])
+def test_moves_that_ordering_makes_slower_are_not_ordered(lib, kind, dim, obs, n, precision):
+    m = _model(lib, model(kind, dim, obs))
+    assert not _ordered(lib, m, 16, n, precision)
     lib.smc_model_destroy(m)
 
 
