@@ -1375,6 +1375,8 @@ smc_status smc_model_create(smc_dev_model** out, const smc_model* model, void* s
 void smc_model_destroy(smc_dev_model* m) {
     if (!m) return;
     cudaStream_t s = m->mem.s;
+    // the room is written by moves on any stream: it is freed behind the last
+    if (m->order.any) (void)cudaStreamWaitEvent(s, m->order.used, 0);
     m->mem.release();
     cudaStreamSynchronize(s);
     if (m->order.used) cudaEventDestroy(m->order.used);

@@ -14,7 +14,7 @@
 
 namespace {
 std::map<const void*, std::string> names;      // host stub -> kernel name
-std::string launched;                          // names, one per line
+std::string launched;                          // names, one per line, and waits for events
 std::string fail_name;
 int fail_code = 0, fail_after = 0;
 cudaError_t last = cudaSuccess;
@@ -144,7 +144,10 @@ cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) {
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = (cudaStream_t)calloc(1, 1), cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { return free(s), cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) {
+    launched += "wait\n";
+    return cudaSuccess;
+}
 cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long* id) { return *id = (unsigned long long)s, cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* c) {
     return *c = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone, cudaSuccess;

@@ -60,6 +60,18 @@ def test_a_move_without_the_room_runs_in_the_particles_order(lib):
     lib.smc_model_destroy(m)
 
 
+def test_a_model_outlives_the_moves_that_use_its_room(lib):
+    """The room is given back behind the last move that writes it, on whatever
+    stream that ran."""
+    m = _model(lib)
+    lib.smc_model_destroy(m)
+    assert host_cuda.launches(lib) == []
+    m = _model(lib)
+    assert _ordered(lib, m, 32)
+    lib.smc_model_destroy(m)
+    assert host_cuda.launches(lib) == ["wait"]
+
+
 @pytest.mark.parametrize("kind,dim,obs,n,precision", ORDERED)
 def test_the_gpu_tests_cases_are_ordered(lib, kind, dim, obs, n, precision):
     m = _model(lib, model(kind, dim, obs))
