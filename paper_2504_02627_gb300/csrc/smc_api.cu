@@ -1474,22 +1474,23 @@ smc_status smc_k_leapfrog(const smc_dev_model* m, float* theta, float* p, float*
     OrderRoom& room = const_cast<smc_dev_model*>(m)->order;
     if (!room.perm || N < 2 || N > OrderRoom::CAP || !order_pays(m->m, precision, N))
         return kstatus(launch_traj(m->m, a, precision, s));
+    if (cudaPeekAtLastError() != cudaSuccess)   // an earlier call's error: the move's launch reports it
+        return kstatus(launch_traj(m->m, a, precision, s));
     std::lock_guard<std::mutex> lock(room.mu);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     unsigned long long id = 0;
     bool mine = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
                 cudaStreamGetId(s, &id) == cudaSuccess;
     if (mine && room.any && id != room.stream_id) mine = room.finished();
-    if (!mine) {
-        (void)cudaGetLastError();   // cudaErrorNotReady is no error of this call
+    // cudaErrorNotReady, or an order that could not be launched, is no error of
+    // this call: the move runs without
+    if (!mine || launch_order_steps(steps, N, room.perm, s) != cudaSuccess) {
+        (void)cudaGetLastError();
         return kstatus(launch_traj(m->m, a, precision, s));
     }
-    cudaError_t e = launch_order_steps(steps, N, room.perm, s);
-    if (e == cudaSuccess) {
-        a.perm = room.perm;
-        a.order_wait = 1;
-        e = launch_traj(m->m, a, precision, s);
-    }
+    a.perm = room.perm;
+    a.order_wait = 1;
+    cudaError_t e = launch_traj(m->m, a, precision, s);
     room.any = true;
     room.stream_id = id;
     if (cudaEventRecord(room.used, s) != cudaSuccess && e == cudaSuccess) e = cudaGetLastError();

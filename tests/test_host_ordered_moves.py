@@ -72,6 +72,20 @@ def test_a_model_outlives_the_moves_that_use_its_room(lib):
     assert host_cuda.launches(lib) == ["wait"]
 
 
+def test_a_move_whose_order_fails_still_runs(lib):
+    m = _model(lib)
+    lib.host_cuda_fail(b"k_order_steps", host_cuda.NOMEM, 0)
+    assert not _ordered(lib, m, 16)
+    assert lib.host_cuda_last_error() == 0
+    lib.host_cuda_fail(b"", 0, 0)
+    # an error that an earlier call left behind is reported, as by any move
+    room = C.c_void_p(4096)
+    lib.host_cuda_leave_error(host_cuda.NOMEM)
+    assert lib.smc_k_leapfrog(m, room, room, room, room, room, 0.1, 6007, 6007, 0, None) == host_cuda.E_CUDA
+    assert not any("k_order_steps" in n for n in host_cuda.launches(lib))
+    lib.smc_model_destroy(m)
+
+
 @pytest.mark.parametrize("kind,dim,obs,n,precision", ORDERED)
 def test_the_gpu_tests_cases_are_ordered(lib, kind, dim, obs, n, precision):
     m = _model(lib, model(kind, dim, obs))
