@@ -1474,7 +1474,7 @@ smc_status smc_k_leapfrog(const smc_dev_model* m, float* theta, float* p, float*
     OrderRoom& room = const_cast<smc_dev_model*>(m)->order;
     if (!room.perm || N < 2 || N > OrderRoom::CAP || !order_pays(m->m, precision, N))
         return kstatus(launch_traj(m->m, a, precision, s));
-    if (cudaPeekAtLastError() != cudaSuccess)   // an earlier call's error: the move's launch reports it
+    if (cudaPeekAtLastError() != cudaSuccess)   // an earlier call's error, not to be taken for the order's or cleared here
         return kstatus(launch_traj(m->m, a, precision, s));
     std::lock_guard<std::mutex> lock(room.mu);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

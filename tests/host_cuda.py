@@ -13,7 +13,7 @@ from paper_2504_02627_gb300 import build as build_mod
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 NOMEM = 2                        # cudaErrorMemoryAllocation
-E_NOMEM, E_CUDA, E_STATE = -2, -3, -6   # SMC_E_*
+E_NOMEM, E_STATE = -2, -6        # SMC_E_*
 
 
 def _objects():
