@@ -16,8 +16,8 @@
 // of P per thread in registers and loading the deviations as broadcasts feeds one
 // (the same 10.6 us); 8 x 8 feeds four but leaves one warp a scheduler with
 // nothing to hide its chains behind (12.5 us).  The 8 x 4 tile here: 20 steps of
-// 8192 particles at D = 100 in 158 instead of 221 us, with the caller's copies (170 with the
-// FP64 sums as trees over a warp per particle).
+// 8192 particles at D = 100 in 156 instead of 221 us, with the caller's copies (170 with the
+// FP64 sums as trees over a warp per particle and a launch order that gained nothing).
 #include <algorithm>
 #include <type_traits>
 #include <math_constants.h>

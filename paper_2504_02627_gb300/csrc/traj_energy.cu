@@ -13,11 +13,11 @@
 // FP32x2 FMAs.  Each eta is one chain over the dimensions, a thread's eight
 // terms of a particle are summed in FP32, everything else in FP64.  Bound by
 // the FMA pipe (its throttle is the first stall, 1.7 of 4.2 warps; a value
-// loaded feeds four FMAs); one chunk buffer, so that two CTAs share an SM and
-// one computes while the other's copy is in flight.  Logistic regression, n =
-// 1e5, D = 100, 16384 particles: 9.1 ms, of which the 1.6e11 FMAs are 5.4; the
-// move with it 18.2 -> 15.2 ms.  With log1pf(expf(.)) written for either sign
-// of eta apart this kernel took 12.4 ms.
+// loaded feeds four FMAs); one chunk buffer, so that two CTAs share an SM (up to
+// 104 padded dimensions) and one computes while the other's copy is in flight.
+// Logistic regression, n = 1e5, D = 100, 16384 particles: 9.1 ms, of which the
+// 1.6e11 FMAs are 5.4; the move with it 18.2 -> 15.2 ms.  With log1pf(expf(.))
+// written for either sign of eta apart this kernel took 12.4 ms.
 #include <algorithm>
 #include <math_constants.h>
 #include "tc_ptx.cuh"
