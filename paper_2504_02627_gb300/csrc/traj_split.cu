@@ -225,14 +225,10 @@ __global__ void __launch_bounds__(128) traj_gauss_rows_kernel(DevModel m, TrajAr
     }
     Slot x{};
     float mu = 0.0f, th = 0.0f, p = 0.0f, g = 0.0f;
-    if (on) {
-        x = slot_of(a, t);
-        if (r == 0) {
-            j_s[pi] = x.j;
-            lp0_s[pi] = a.eval_only ? 0.0 : a.logpi_in[x.src];
-        }
-    }
+    if (on) x = slot_of(a, t);
     const int64_t o = (int64_t)r * a.ld;
+    // (kept in a register until the end: a store here would wait for it)
+    const double lp0 = on && r == 0 && !a.eval_only ? a.logpi_in[x.src] : 0.0;
     if (in) {
         mu = m.mu[r];
         th = a.theta_in[o + x.src];
@@ -297,6 +293,10 @@ __global__ void __launch_bounds__(128) traj_gauss_rows_kernel(DevModel m, TrajAr
             p1_s[pi][r] = p;
         }
         q_s[pi][r] = (th - mu) * g;
+        if (r == 0) {
+            j_s[pi] = x.j;
+            lp0_s[pi] = lp0;
+        }
         if (in) {
             a.grad_out[o + x.j] = g;
             if (!a.eval_only) {
